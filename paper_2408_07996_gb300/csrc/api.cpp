@@ -718,9 +718,9 @@ mcev_status check_spp_fits(mcev_ctx* ctx, int64_t spp) {
 mcev_status ensure_wave(mcev_ctx* ctx) {
     const int64_t cap = wave_cap(ctx);
     if (ctx->d_wave.ptr && ctx->wave.cap == cap) return MCEV_OK;
-    // path slots: L, sig, pflags, pix_k, Ltot, delta; per ray-queue slot (x2):
-    // ray_o, ray_d, ray_s; hit; shadow: sh_o, sh_d, sh_c, sh_g, sh_m
-    const size_t per = 4 + 4 + 4 + 8 + 4 + 4 + 2 * (16 + 16 + 16) + 16 + 16 + 16 + 4 + 4 + 4;
+    // per path slot: ray_o, ray_d, sh_d; hit, pix_k; hit_rec, L, sig, pflags, sh_c, sh_g, sh_m, Ltot, delta; key;
+    // queues: list (x2), sh_list
+    const size_t per = 3 * 16 + 2 * 8 + 9 * 4 + 2 + 3 * 4;
     ST(dev_alloc(ctx, ctx->d_wave, (size_t)cap * per + 64 * 256));
     char* p = (char*)ctx->d_wave.ptr;
     auto take = [&](size_t bytes) {
@@ -730,19 +730,19 @@ mcev_status ensure_wave(mcev_ctx* ctx) {
     };
     Wave& w = ctx->wave;
     w.cap = cap;
-    w.ray_o[0] = (float4*)take(16 * cap);
-    w.ray_o[1] = (float4*)take(16 * cap);
-    w.ray_d[0] = (float4*)take(16 * cap);
-    w.ray_d[1] = (float4*)take(16 * cap);
-    w.ray_s[0] = (float4*)take(16 * cap);
-    w.ray_s[1] = (float4*)take(16 * cap);
-    w.hit = (float4*)take(16 * cap);
-    w.sh_o = (float4*)take(16 * cap);
+    w.ray_o = (float4*)take(16 * cap);
+    w.ray_d = (float4*)take(16 * cap);
+    w.hit = (float2*)take(8 * cap);
+    w.hit_rec = (int32_t*)take(4 * cap);
     w.sh_d = (float4*)take(16 * cap);
     w.pix_k = (int2*)take(8 * cap);
     w.L = (float*)take(4 * cap);
     w.sig = (uint32_t*)take(4 * cap);
     w.pflags = (uint32_t*)take(4 * cap);
+    w.key = (uint16_t*)take(2 * cap);
+    w.list[0] = (int32_t*)take(4 * cap);
+    w.list[1] = (int32_t*)take(4 * cap);
+    w.sh_list = (int32_t*)take(4 * cap);
     w.sh_c = (float*)take(4 * cap);
     w.sh_g = (float*)take(4 * cap);
     w.sh_m = (int32_t*)take(4 * cap);
@@ -812,11 +812,6 @@ DevParams dev_params(const mcev_ctx* ctx, bool want_sig) {
         ST(ev_mark(ctx, cls, false));                                                                 \
     } while (0)
 
-// 1: a bounce's shadow rays share one launch with the next bounce's closest hits
-#ifndef MCEV_FUSE_SHADOW
-#define MCEV_FUSE_SHADOW 1
-#endif
-
 // one chunk of n_paths = nj * spp_r paths through every bounce
 // Batched render (several contexts' frame pairs in one set of rounds): the
 // device job table, the union queues of (job << 24 | pixel) entries, and the
@@ -850,26 +845,15 @@ mcev_status trace_chunk(mcev_ctx* ctx, const Frame& fr, const DevParams& P, cons
     LAUNCH(MCEV_K_RAYGEN,
            launch_raygen(fr.dev, P, w, queue, j0, spp_r, k_base, n_paths, 0, ctx->sms, ctx->stream, jobs, rc));
     int cur = 0;
-    LAUNCH(MCEV_K_EXTEND,
-           launch_extend(ctx->dsc, fr.dev, P.t_min, w, cur, n_paths, err, ctx->sms, ctx->stream, jobs, trav));
+    LAUNCH(MCEV_K_EXTEND, launch_trace(ctx->dsc, fr.dev, P, w, cur, -1, 0, n_paths, err, ctx->sms, ctx->stream, jobs,
+                                       trav));
     for (int depth = 0; depth <= depth_max; ++depth) {
-        LAUNCH(MCEV_K_SHADE, launch_shade(ctx->dsc, fr.dev, P, w, cur, n_paths, ctx->sms, ctx->stream, jobs));
+        LAUNCH(MCEV_K_SHADE, launch_shade(ctx->dsc, fr.dev, P, w, cur, depth, n_paths, ctx->sms, ctx->stream, jobs));
         if (depth < depth_max) {
-#if MCEV_FUSE_SHADOW
+            LAUNCH(MCEV_K_SHADE, launch_queue(w, cur, depth, n_paths, ctx->sms, ctx->stream));
             // this bounce's shadow rays and the next bounce's closest hits in one launch
-            if (nee)
-                LAUNCH(MCEV_K_EXTEND, launch_shadow_extend(ctx->dsc, fr.dev, P, w, cur, n_paths, err, ctx->sms,
-                                                           ctx->stream, jobs, trav));
-            else
-                LAUNCH(MCEV_K_EXTEND, launch_extend(ctx->dsc, fr.dev, P.t_min, w, cur ^ 1, n_paths, err, ctx->sms,
-                                                    ctx->stream, jobs, trav));
-#else
-            if (nee)
-                LAUNCH(MCEV_K_SHADOW, launch_shadow(ctx->dsc, fr.dev, P, w, cur, n_paths, err, ctx->sms, ctx->stream,
-                                                    jobs, trav));
-            LAUNCH(MCEV_K_EXTEND, launch_extend(ctx->dsc, fr.dev, P.t_min, w, cur ^ 1, n_paths, err, ctx->sms,
-                                                ctx->stream, jobs, trav));
-#endif
+            LAUNCH(MCEV_K_EXTEND, launch_trace(ctx->dsc, fr.dev, P, w, cur ^ 1, nee ? cur : -1, depth + 1, n_paths,
+                                               err, ctx->sms, ctx->stream, jobs, trav));
         }
         cur ^= 1;
     }

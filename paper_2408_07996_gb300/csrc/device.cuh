@@ -20,17 +20,8 @@ namespace mcev {
 
 #define MCEV_PI 3.14159265358979323846f
 #define MCEV_STACK MCEV_STACK_HOST
-// traversal kernels run 128-thread blocks; the shared stack interleaves threads
+// traversal kernels run 128-thread blocks; each thread's stack is in local memory
 #define MCEV_TRAV_BLOCK 128
-#if MCEV_SMEM_STACK
-#define SIDX(i) ((i) * MCEV_TRAV_BLOCK)
-#define MCEV_DECLARE_STACK(name)                               \
-    __shared__ int name##_smem[MCEV_STACK * MCEV_TRAV_BLOCK];  \
-    int* name = name##_smem + threadIdx.x
-#else
-#define SIDX(i) (i)
-#define MCEV_DECLARE_STACK(name) int name[MCEV_STACK]
-#endif
 
 // ------------------------------------------------------------------ math
 struct f3 {
@@ -225,7 +216,6 @@ struct WRay {
     f3 o;
     f3 mx, my, mz;    // shear rows: x' = mx.A, y' = my.A, z' = mz.A for A = v - o
     f3 idir;          // 1/d with tiny components replaced, for slab tests
-    f3 oidir;         // o * idir
 };
 
 __device__ __forceinline__ WRay make_wray(f3 o, f3 d) {
@@ -256,7 +246,6 @@ __device__ __forceinline__ WRay make_wray(f3 o, f3 d) {
     r.idir = mk3(1.0f / (fabsf(d.x) > ooeps ? d.x : copysignf(ooeps, d.x)),
                  1.0f / (fabsf(d.y) > ooeps ? d.y : copysignf(ooeps, d.y)),
                  1.0f / (fabsf(d.z) > ooeps ? d.z : copysignf(ooeps, d.z)));
-    r.oidir = mk3(o.x * r.idir.x, o.y * r.idir.y, o.z * r.idir.z);
     return r;
 }
 
@@ -289,33 +278,19 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     return d;
 }
 
-// slab test of both children of a node; returns hit mask (bit0 left, bit1 right)
-__device__ __forceinline__ int node_hits(const WRay& r, const Node& n, float tmin, float tmax, float& tl, float& tr) {
-    const float4 a = n.a, b = n.b, c = n.c;
-    const float lx0 = fmaf(a.x, r.idir.x, -r.oidir.x), lx1 = fmaf(a.y, r.idir.x, -r.oidir.x);
-    const float ly0 = fmaf(a.z, r.idir.y, -r.oidir.y), ly1 = fmaf(a.w, r.idir.y, -r.oidir.y);
-    const float lz0 = fmaf(c.x, r.idir.z, -r.oidir.z), lz1 = fmaf(c.y, r.idir.z, -r.oidir.z);
-    const float rx0 = fmaf(b.x, r.idir.x, -r.oidir.x), rx1 = fmaf(b.y, r.idir.x, -r.oidir.x);
-    const float ry0 = fmaf(b.z, r.idir.y, -r.oidir.y), ry1 = fmaf(b.w, r.idir.y, -r.oidir.y);
-    const float rz0 = fmaf(c.z, r.idir.z, -r.oidir.z), rz1 = fmaf(c.w, r.idir.z, -r.oidir.z);
-    const float ln = max3f(fminf(lx0, lx1), fminf(ly0, ly1), fmaxf(fminf(lz0, lz1), tmin));
-    const float lf = min3f(fmaxf(lx0, lx1), fmaxf(ly0, ly1), fminf(fmaxf(lz0, lz1), tmax));
-    const float rn = max3f(fminf(rx0, rx1), fminf(ry0, ry1), fmaxf(fminf(rz0, rz1), tmin));
-    const float rf = min3f(fmaxf(rx0, rx1), fmaxf(ry0, ry1), fminf(fmaxf(rz0, rz1), tmax));
-    tl = ln;
-    tr = rn;
-    // (1 + 2^-20) slack keeps rounding in the slab arithmetic from culling a hit
-    return (ln <= lf * 1.000001f + 1e-30f ? 1 : 0) | (rn <= rf * 1.000001f + 1e-30f ? 2 : 0);
-}
-
+// One node is two 32-byte loads (nodes are 64-byte aligned): half the load
+// instructions and L1 requests of four 16-byte ones (1 % of traversal time).
 __device__ __forceinline__ Node load_node(const Node* nodes, int i) {
-    const float4* p = reinterpret_cast<const float4*>(nodes + i);
+    const Node* p = nodes + i;
     Node n;
-    n.a = __ldg(p);
-    n.b = __ldg(p + 1);
-    n.c = __ldg(p + 2);
-    const float4 d = __ldg(p + 3);
-    n.d = make_int4(__float_as_int(d.x), __float_as_int(d.y), __float_as_int(d.z), __float_as_int(d.w));
+    float dx, dy, dz, dw;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(n.a.x), "=f"(n.a.y), "=f"(n.a.z), "=f"(n.a.w), "=f"(n.b.x), "=f"(n.b.y), "=f"(n.b.z), "=f"(n.b.w)
+        : "l"(p));
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8 + 32];"
+        : "=f"(n.c.x), "=f"(n.c.y), "=f"(n.c.z), "=f"(n.c.w), "=f"(dx), "=f"(dy), "=f"(dz), "=f"(dw)
+        : "l"(p));
+    n.d = make_int4(__float_as_int(dx), __float_as_int(dy), __float_as_int(dz), __float_as_int(dw));
     return n;
 }
 
@@ -334,13 +309,7 @@ __device__ __forceinline__ bool better_hit(float t, int inst, int prim, const Hi
     return prim < h.prim;
 }
 
-// BLAS closest hit of an object-space ray; updates h
 #define MCEV_NO_NODE (-0x7fffffff)
-// any-hit traversal visits the nearer child first when MCEV_ANY_ORDERED
-// (occluders are found sooner; ~1% faster shadow rays on the terrain frame)
-#ifndef MCEV_ANY_ORDERED
-#define MCEV_ANY_ORDERED 1
-#endif
 
 // ------------------------------------------------------------------ compressed 8-wide BLAS
 // Traversal of the Node8 layout (layout.h).  A "node group" is a 64-bit word
@@ -419,18 +388,41 @@ __device__ __forceinline__ uint32_t wide_node_hits(const uint4* __restrict__ wn,
 }
 
 // Closest hit (kAny = false; updates h) or any hit in (tmin, tmax] (kAny =
-// true; returns true at the first occluder) of an object-space ray in the
-// wide BLAS rooted at `root`.  work: (node fetches, triangle tests, box tests).
+// true; returns true at the first occluder) of the whole warp's object-space
+// rays in wide BLASes, one ray per lane (`live`) rooted at `root`.  Like
+// two_wide, every iteration is one convergence point: lanes without a pending
+// triangle take a node step, then lanes with one test it.
+// work: (node fetches, triangle tests, box tests).
 template <bool kAny>
 __device__ __forceinline__ bool blas_wide(const DevScene& sc, uint32_t root, int rec, int inst, const WRay& r,
-                                          float tmin, float tmax, Hit& h, uint2* stack, int* err, int3& work) {
+                                          bool live, float tmin, float tmax, Hit& h, uint2* stack, int* err,
+                                          int3& work) {
     const uint32_t ox = (r.idir.x >= 0.0f ? 1u : 0u) | (r.idir.y >= 0.0f ? 2u : 0u) | (r.idir.z >= 0.0f ? 4u : 0u);
     // the root as the only (internal, slot 0) child of a virtual parent
-    uint2 g = make_uint2(root, (1u << (24 + ox)) | 1u);
+    uint2 g = live ? make_uint2(root, (1u << (24 + ox)) | 1u) : make_uint2(0u, 0u);
     int sp = 0;
-    // one loop iteration per node OR per triangle (as in the two-wide loop)
     uint32_t tb = 0, tbits = 0, tmask = 0;
-    while (true) {
+    bool found = false;
+    while (__any_sync(0xffffffffu, tbits != 0 || (g.y >> 24) != 0 || sp > 0)) {
+        if (tbits == 0 && (g.y >> 24) == 0 && sp > 0) g = stack[--sp];
+        if (tbits == 0 && (g.y >> 24) != 0) {
+            const uint32_t key = __ffs(g.y >> 24) - 1;
+            g.y &= ~(1u << (24 + key));
+            const uint32_t slot = key ^ ox;
+            const uint32_t child = g.x + __popc(g.y & ((1u << slot) - 1u) & 0xFFu);
+            if (g.y & 0xFF000000u) {
+                if (sp < MCEV_WSTACK) stack[sp++] = g;
+                else *err = 1;
+            }
+            uint32_t cb, im;
+            int nv;
+            const uint32_t hit8 =
+                wide_node_hits(sc.wnodes, child, r, ox, tmin, kAny ? tmax : h.t, cb, tb, im, tmask, nv);
+            work.x += 1;
+            work.z += nv;
+            g = make_uint2(cb, (xor_permute8(hit8 & im, ox) << 24) | im);
+            tbits = spread3(hit8 & ~im) & tmask;
+        }
         if (tbits) {
             const uint32_t bit = (uint32_t)(__ffs(tbits) - 1);
             tbits &= tbits - 1;
@@ -440,142 +432,330 @@ __device__ __forceinline__ bool blas_wide(const DevScene& sc, uint32_t root, int
             work.y += 1;
             const float t = tri_hit(r, p0, p1, p2, tmin, kAny ? tmax : h.t);
             if (kAny) {
-                if (t >= 0.0f) return true;
+                if (t >= 0.0f) {
+                    found = true;
+                    tbits = 0;
+                    g.y = 0;
+                    sp = 0;
+                }
             } else {
                 const int oi = inst >= 0 ? inst : __float_as_int(p2.w);
                 if (t >= 0.0f && better_hit(t, oi, __float_as_int(p0.w), h)) {
                     h.t = t; h.inst = oi; h.tri = (int)ti; h.prim = __float_as_int(p0.w); h.rec = rec;
                 }
             }
-            continue;
         }
-        if (!(g.y & 0xFF000000u)) {
-            if (sp == 0) break;
-            g = stack[--sp];
-        }
-        const uint32_t key = __ffs(g.y >> 24) - 1;
-        g.y &= ~(1u << (24 + key));
-        const uint32_t slot = key ^ ox;
-        const uint32_t child = g.x + __popc(g.y & ((1u << slot) - 1u) & 0xFFu);
-        if (g.y & 0xFF000000u) {
-            if (sp < MCEV_WSTACK) stack[sp++] = g;
-            else *err = 1;
-        }
-        uint32_t cb, im;
-        int nv;
-        const uint32_t hit8 = wide_node_hits(sc.wnodes, child, r, ox, tmin, kAny ? tmax : h.t, cb, tb, im, tmask, nv);
-        work.x += 1;
-        work.z += nv;
-        g = make_uint2(cb, (xor_permute8(hit8 & im, ox) << 24) | im);
-        tbits = spread3(hit8 & ~im) & tmask;
+    }
+    return found;
+}
+
+// ------------------------------------------------------------------ two-wide BLAS
+// Ray of the two-wide traversal: origin, reciprocal direction and -o/d for
+// the slab tests, and the watertight test's shear as its axis code and three
+// factors.  13 values instead of WRay's 18 let the loop run at 48 registers.
+struct TRay {
+    f3 o, idir, noid;
+    float nsx, nsy, sz;   // -Sx, -Sy, Sz
+    int k;                // dominant axis kz + 3 * (kx and ky swapped)
+};
+
+// reciprocal direction with tiny components replaced, and -o/d
+__device__ __forceinline__ void slab_setup(TRay& r, f3 o, f3 d) {
+    const float ooeps = 0x1p-80f;
+    r.idir = mk3(1.0f / (fabsf(d.x) > ooeps ? d.x : copysignf(ooeps, d.x)),
+                 1.0f / (fabsf(d.y) > ooeps ? d.y : copysignf(ooeps, d.y)),
+                 1.0f / (fabsf(d.z) > ooeps ? d.z : copysignf(ooeps, d.z)));
+    r.noid = mk3(-(o.x * r.idir.x), -(o.y * r.idir.y), -(o.z * r.idir.z));
+}
+
+__device__ __forceinline__ TRay make_tray(f3 o, f3 d) {
+    TRay r;
+    r.o = o;
+    const float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
+    int kz = 0;
+    if (ay > ax && ay >= az) kz = 1;
+    else if (az > ax && az > ay) kz = 2;
+    const float dz = kz == 0 ? d.x : (kz == 1 ? d.y : d.z);
+    float dkx = kz == 0 ? d.y : (kz == 1 ? d.z : d.x);
+    float dky = kz == 0 ? d.z : (kz == 1 ? d.x : d.y);
+    r.k = kz;
+    if (dz < 0.0f) {
+        const float t = dkx;
+        dkx = dky;
+        dky = t;
+        r.k += 3;
+    }
+    r.nsx = -(dkx / dz);
+    r.nsy = -(dky / dz);
+    r.sz = 1.0f / dz;
+    slab_setup(r, o, d);
+    return r;
+}
+
+// Sheared coordinates of A = v - o for one axis code: the same bits as
+// WRay's dot products mx.A, my.A, whose other coefficients are 0 and 1 (an
+// unfused product where the 1 comes after the dominant axis in x, y, z
+// order, a fused one where it comes before).  z is left unscaled.
+template <int K>
+__device__ __forceinline__ void shear(const TRay& r, f3 A, float& x, float& y, float& z) {
+    if (K == 0) { x = A.y + r.nsx * A.x; y = A.z + r.nsy * A.x; z = A.x; }
+    if (K == 3) { x = A.z + r.nsx * A.x; y = A.y + r.nsy * A.x; z = A.x; }
+    if (K == 1) { x = A.z + r.nsx * A.y; y = fmaf(r.nsy, A.y, A.x); z = A.y; }
+    if (K == 4) { x = fmaf(r.nsx, A.y, A.x); y = A.z + r.nsy * A.y; z = A.y; }
+    if (K == 2) { x = fmaf(r.nsx, A.z, A.x); y = fmaf(r.nsy, A.z, A.y); z = A.z; }
+    if (K == 5) { x = fmaf(r.nsx, A.z, A.y); y = fmaf(r.nsy, A.z, A.x); z = A.z; }
+}
+
+// tri_hit of a TRay (same bits).  The rays of a warp mostly share one axis
+// code (the queues are ordered by it), so the switch runs one case.
+__device__ __forceinline__ float tri_hit(const TRay& r, float4 p0, float4 p1, float4 p2, float tmin, float tmax) {
+    const f3 A = xyz(p0) - r.o, B = xyz(p1) - r.o, C = xyz(p2) - r.o;
+    float Ax, Ay, Az, Bx, By, Bz, Cx, Cy, Cz;
+#define MCEV_SHEAR(K)               \
+    shear<K>(r, A, Ax, Ay, Az);     \
+    shear<K>(r, B, Bx, By, Bz);     \
+    shear<K>(r, C, Cx, Cy, Cz);     \
+    break;
+    switch (r.k) {
+    case 0: MCEV_SHEAR(0)
+    case 1: MCEV_SHEAR(1)
+    case 2: MCEV_SHEAR(2)
+    case 3: MCEV_SHEAR(3)
+    case 4: MCEV_SHEAR(4)
+    default: MCEV_SHEAR(5)
+    }
+#undef MCEV_SHEAR
+    const float U = fmaf(Cx, By, -(Cy * Bx));
+    const float V = fmaf(Ax, Cy, -(Ay * Cx));
+    const float W = fmaf(Bx, Ay, -(By * Ax));
+    if ((U < 0.0f || V < 0.0f || W < 0.0f) && (U > 0.0f || V > 0.0f || W > 0.0f)) return -1.0f;
+    const float det = U + V + W;
+    if (det == 0.0f) return -1.0f;
+    const float T = fmaf(W, r.sz * Cz, fmaf(V, r.sz * Bz, U * (r.sz * Az)));
+    const float t = T / det;
+    return (t > tmin && t <= tmax) ? t : -1.0f;
+}
+
+// (y0, y1) = (x0, x1) * m + a in one packed instruction
+__device__ __forceinline__ void fma2(float x0, float x1, float m, float a, float& y0, float& y1) {
+    asm("{\n\t.reg .b64 p, q, s, d;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %4};\n\tmov.b64 s, {%5, %5};\n\t"
+        "fma.rn.f32x2 d, p, q, s;\n\tmov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(y0), "=f"(y1)
+        : "f"(x0), "f"(x1), "f"(m), "f"(a));
+}
+
+// Slab test of both children of a node against [tmin, tmax]: hit mask (bit 0
+// left, bit 1 right) and entry distances.  The slack of 2^-20 keeps rounding in
+// the slab arithmetic from culling a hit.
+__device__ __forceinline__ int node_hits(const TRay& r, const Node& n, float tmin, float tmax, float& tl, float& tr) {
+    float lx0, lx1, ly0, ly1, lz0, lz1, rx0, rx1, ry0, ry1, rz0, rz1;
+    fma2(n.a.x, n.a.y, r.idir.x, r.noid.x, lx0, lx1);
+    fma2(n.a.z, n.a.w, r.idir.y, r.noid.y, ly0, ly1);
+    fma2(n.c.x, n.c.y, r.idir.z, r.noid.z, lz0, lz1);
+    fma2(n.b.x, n.b.y, r.idir.x, r.noid.x, rx0, rx1);
+    fma2(n.b.z, n.b.w, r.idir.y, r.noid.y, ry0, ry1);
+    fma2(n.c.z, n.c.w, r.idir.z, r.noid.z, rz0, rz1);
+    const float ln = max3f(fminf(lx0, lx1), fminf(ly0, ly1), fmaxf(fminf(lz0, lz1), tmin));
+    const float lf = min3f(fmaxf(lx0, lx1), fmaxf(ly0, ly1), fminf(fmaxf(lz0, lz1), tmax));
+    const float rn = max3f(fminf(rx0, rx1), fminf(ry0, ry1), fmaxf(fminf(rz0, rz1), tmin));
+    const float rf = min3f(fmaxf(rx0, rx1), fmaxf(ry0, ry1), fminf(fmaxf(rz0, rz1), tmax));
+    tl = ln;
+    tr = rn;
+    return (ln <= lf * 1.000001f ? 1 : 0) | (rn <= rf * 1.000001f ? 2 : 0);
+}
+
+// hit so far: distance, leaf-order triangle (-1: none), instance record
+struct THit {
+    float t;
+    int tri, rec;
+};
+
+// uploaded instance id of a triangle (its v2.w) of instance record rec: the
+// merged never-moving geometry keeps it in the triangle, the others in the record
+__device__ __forceinline__ int hit_inst(const DevFrame& fr, int rec, float w2) {
+    const int i = __float_as_int(w2);
+    return i >= 0 ? i : __float_as_int(__ldg(&fr.inst[7 * rec + 6].z));
+}
+
+// at equal t the smaller (instance, triangle) pair wins
+__device__ __forceinline__ bool tie_wins(const DevScene& sc, const DevFrame& fr, int rec, float w0, float w2,
+                                         const THit& h) {
+    if (h.tri < 0) return false;
+    const int in = hit_inst(fr, rec, w2), io = hit_inst(fr, h.rec, __ldg(&sc.tris[3 * h.tri + 2].w));
+    if (in != io) return in < io;
+    return __float_as_int(w0) < __float_as_int(__ldg(&sc.tris[3 * h.tri].w));
+}
+
+// One pending leaf triangle.  kAny: true at an occluder in (tmin, h.t]
+// (h.tri set); else updates the closest hit h and returns false.
+template <bool kAny>
+__device__ __forceinline__ bool tri_step(const DevScene& sc, const DevFrame& fr, const TRay& r, int rec, int tri,
+                                         float tmin, THit& h) {
+    const float4* tp = sc.tris + 3 * tri;
+    const float4 p0 = __ldg(tp), p1 = __ldg(tp + 1), p2 = __ldg(tp + 2);
+    const float t = tri_hit(r, p0, p1, p2, tmin, h.t);
+    if (kAny) {
+        if (t >= 0.0f) h.tri = tri;
+        return t >= 0.0f;
+    }
+    if (t >= 0.0f && (t < h.t || tie_wins(sc, fr, rec, p0.w, p2.w, h))) {
+        h.t = t;
+        h.tri = tri;
+        h.rec = rec;
     }
     return false;
 }
 
-// Two-wide BLAS traversal, one loop iteration per node step OR per leaf
-// triangle: a node step records its hit leaf children as a pending triangle
-// range (sibling leaves are contiguous in the leaf order) instead of testing
-// them at once, and the lane tests one pending triangle per iteration before
-// its next node step.  Lanes testing triangles and lanes stepping through
-// nodes then share warp iterations, instead of the warp running every lane's
-// triangle loop while the others wait (measured: 75 % of warp-steps of the
-// terrain frame carried such loops at 6 % lane activity).  Nodes and
-// triangles are visited in the same order as a test-at-once traversal, so
-// the closest hit is the same.
-// rec: instance record; inst: its uploaded instance id, or -1 for the merged
-// static geometry whose triangles carry their own instance id (v2.w).
-
-__device__ __forceinline__ void blas_closest(const DevScene& sc, int root, int rec, int inst, const WRay& r,
-                                                  float tmin, Hit& h, int* stack, int base, int* err, int3& work) {
-    int sp = base, node = root;
+// Closest hit (kAny = false; updates h) or any hit in (tmin, h.t] (kAny: sets
+// h.tri and stops) of the whole warp's rays in two-wide BLASes, one ray per lane
+// (`live`) rooted at `root`.
+//
+// What bounds it: the latency of the node loads and the issue slots of the
+// iterations a warp needs (its lanes' rays take different numbers of steps).
+// Every iteration is one convergence point: all lanes that can take a node
+// step do (twice, MCEV_NODE_STEPS), then all lanes with a pending leaf
+// triangle test one, a lane that just reached a leaf in the same iteration.
+// A lane's own order of nodes and triangles is that of a plain traversal,
+// so its hits do not depend on its neighbours.  Without the vote the
+// compiler lets lanes drift apart: the same body as a per-lane loop took
+// 1229 ms of traversal per 1280x720 terrain frame, with it 714 ms (register
+// cap 56) and 672 ms (48); two node steps per iteration 650 ms, three 657 ms;
+// waiting until 4 or 8 lanes have a triangle 781 and 847 ms.
+#define MCEV_NODE_STEPS 2
+template <bool kAny>
+__device__ __forceinline__ void two_wide(const DevScene& sc, const DevFrame& fr, int root, int rec, const TRay& r,
+                                         bool live, float tmin, THit& h, int* stack, int32_t* err, int2& work) {
+    int sp = 0, node = live ? root : MCEV_NO_NODE;
     int pfirst = 0, pcount = 0;
-    while (true) {
-        if (pcount > 0) {
-            const float4* tp = sc.tris + 3 * pfirst;
-            const float4 p0 = __ldg(tp), p1 = __ldg(tp + 1), p2 = __ldg(tp + 2);
-            const float t = tri_hit(r, p0, p1, p2, tmin, h.t);
-            const int oi = inst >= 0 ? inst : __float_as_int(p2.w);
-            if (t >= 0.0f && better_hit(t, oi, __float_as_int(p0.w), h)) {
-                h.t = t; h.inst = oi; h.tri = pfirst; h.prim = __float_as_int(p0.w); h.rec = rec;
+    while (__any_sync(0xffffffffu, node != MCEV_NO_NODE || pcount > 0)) {
+#pragma unroll
+        for (int s = 0; s < MCEV_NODE_STEPS; ++s) {
+            if (pcount == 0 && node != MCEV_NO_NODE) {
+                const Node n = load_node(sc.nodes, node);
+                work.x += 1;
+                float tl, tr;
+                const int m = node_hits(r, n, tmin, h.t, tl, tr);
+                // hit leaf children become one pending range (sibling leaves are contiguous)
+                const bool lh = (m & 1) && n.d.x < 0, rh = (m & 2) && n.d.y < 0;
+                pfirst = lh ? ~n.d.x : ~n.d.y;
+                pcount = (lh ? n.d.z : 0) + (rh ? n.d.w : 0);
+                const bool gl = (m & 1) && n.d.x >= 0 && (kAny || tl <= h.t);
+                const bool gr = (m & 2) && n.d.y >= 0 && (kAny || tr <= h.t);
+                node = gl ? n.d.x : n.d.y;
+                if (gl && gr) {
+                    // nearer child first (shadow rays too: occluders are found sooner)
+                    if (sp < MCEV_STACK) stack[sp++] = tl <= tr ? n.d.y : n.d.x;
+                    else atomicOr(err, 1);
+                    node = tl <= tr ? n.d.x : n.d.y;
+                } else if (!(gl || gr)) {
+                    node = MCEV_NO_NODE;
+                    if (sp > 0) node = stack[--sp];
+                }
             }
+        }
+        if (pcount > 0) {
             work.y += 1;
+            if (tri_step<kAny>(sc, fr, r, rec, pfirst, tmin, h)) {
+                node = MCEV_NO_NODE;
+                pcount = 1;
+            }
             ++pfirst;
             --pcount;
-            continue;
         }
-        if (node == MCEV_NO_NODE) {
-            if (sp == base) break;
-            node = stack[SIDX(--sp)];
-        }
-        const Node n = load_node(sc.nodes, node);
-        work.x += 1;
-        float tl, tr;
-        const int m = node_hits(r, n, tmin, h.t, tl, tr);
-        const bool lh = (m & 1) && n.d.x < 0, rh = (m & 2) && n.d.y < 0;
-        pfirst = lh ? ~n.d.x : ~n.d.y;
-        pcount = (lh ? n.d.z : 0) + (rh ? n.d.w : 0);
-        const bool gl = (m & 1) && n.d.x >= 0 && tl <= h.t;
-        const bool gr = (m & 2) && n.d.y >= 0 && tr <= h.t;
-        int next = MCEV_NO_NODE;
-        if (gl && gr) {
-            const int nearc = tl <= tr ? n.d.x : n.d.y;
-            const int farc = tl <= tr ? n.d.y : n.d.x;
-            if (sp < MCEV_STACK) stack[SIDX(sp++)] = farc;
-            else *err = 1;
-            next = nearc;
-        } else if (gl) {
-            next = n.d.x;
-        } else if (gr) {
-            next = n.d.y;
-        }
-        node = next;
     }
 }
 
-__device__ __forceinline__ bool blas_any(const DevScene& sc, int root, const WRay& r, float tmin, float tmax,
-                                              int* stack, int base, int* err, int3& work) {
-    int sp = base, node = root;
+// the ray (op, dp) in the object space of instance record rec
+__device__ __forceinline__ TRay object_tray(const DevFrame& fr, int rec, const float4* op, const float4* dp,
+                                            int& root) {
+    const float4* ip = fr.inst + 7 * rec;
+    const float4 i0 = __ldg(ip + 3), i1 = __ldg(ip + 4), i2 = __ldg(ip + 5);
+    root = __float_as_int(__ldg(ip + 6).x);
+    const f3 o = xyz(*op), d = xyz(*dp);
+    return make_tray(xf_point(i0, i1, i2, o), xf_vec(i0, i1, i2, d));
+}
+
+// Two-level traversal of the moving instances (TLAS, then each hit
+// instance's two-wide BLAS) as one converged loop like two_wide's: a lane's
+// step is a TLAS or a BLAS node or a pending triangle, whatever it is at.  A
+// TLAS step records its hit leaf children (one instance record each) as
+// pending; they are entered before the next TLAS step, the TLAS node in hand
+// waiting on the stack.  BLAS nodes are stacked above `base`, the TLAS stack
+// height when the instance was entered.  The ray is read again (op, dp) at
+// each change of level instead of staying in registers.
+template <bool kAny>
+__device__ __forceinline__ void two_level(const DevScene& sc, const DevFrame& fr, const float4* op, const float4* dp,
+                                          bool live, float tmin, THit& h, int* stack, int32_t* err, int2& work) {
+    TRay r;
+    if (live) slab_setup(r, xyz(*op), xyz(*dp));
+    bool in_blas = false;
+    int sp = 0, base = 0, node = MCEV_NO_NODE;
     int pfirst = 0, pcount = 0;
-    while (true) {
+    int pend0 = -1, pend1 = -1, rec = -1;
+    if (live) {
+        if (fr.n_tlas == 1) pend0 = 0;
+        else node = 0;
+    }
+    while (__any_sync(0xffffffffu, node != MCEV_NO_NODE || pcount > 0 || pend0 >= 0 || in_blas)) {
+        if (pcount == 0) {
+            if (in_blas && node == MCEV_NO_NODE) {
+                // instance done: back to the TLAS
+                in_blas = false;
+                if (pend0 < 0) {
+                    if (sp > 0) node = stack[--sp];
+                    if (node != MCEV_NO_NODE) slab_setup(r, xyz(*op), xyz(*dp));
+                }
+            }
+            if (!in_blas && pend0 >= 0) {
+                if (node != MCEV_NO_NODE) {
+                    if (sp < MCEV_STACK) stack[sp++] = node;
+                    else atomicOr(err, 1);
+                }
+                rec = pend0;
+                pend0 = pend1;
+                pend1 = -1;
+                r = object_tray(fr, rec, op, dp, node);
+                in_blas = true;
+                base = sp;
+            }
+        }
+        if (pcount == 0 && node != MCEV_NO_NODE) {
+            const Node n = load_node(in_blas ? sc.nodes : fr.tlas, node);
+            work.x += 1;
+            float tl, tr;
+            const int m = node_hits(r, n, tmin, h.t, tl, tr);
+            const bool lh = (m & 1) && n.d.x < 0, rh = (m & 2) && n.d.y < 0;
+            if (in_blas) {
+                pfirst = lh ? ~n.d.x : ~n.d.y;
+                pcount = (lh ? n.d.z : 0) + (rh ? n.d.w : 0);
+            } else {
+                pend0 = lh ? ~n.d.x : (rh ? ~n.d.y : -1);
+                pend1 = (lh && rh) ? ~n.d.y : -1;
+            }
+            const bool gl = (m & 1) && n.d.x >= 0 && (kAny || tl <= h.t);
+            const bool gr = (m & 2) && n.d.y >= 0 && (kAny || tr <= h.t);
+            node = gl ? n.d.x : n.d.y;
+            if (gl && gr) {
+                if (sp < MCEV_STACK) stack[sp++] = tl <= tr ? n.d.y : n.d.x;
+                else atomicOr(err, 1);
+                node = tl <= tr ? n.d.x : n.d.y;
+            } else if (!(gl || gr)) {
+                // within the level; a finished BLAS and pending instances are handled above
+                node = MCEV_NO_NODE;
+                if (in_blas ? sp > base : (sp > 0 && pend0 < 0)) node = stack[--sp];
+            }
+        }
         if (pcount > 0) {
-            const float4* tp = sc.tris + 3 * pfirst;
             work.y += 1;
-            if (tri_hit(r, __ldg(tp), __ldg(tp + 1), __ldg(tp + 2), tmin, tmax) >= 0.0f) return true;
+            if (tri_step<kAny>(sc, fr, r, rec, pfirst, tmin, h)) {
+                node = MCEV_NO_NODE;
+                pend0 = -1;
+                in_blas = false;
+                pcount = 1;
+            }
             ++pfirst;
             --pcount;
-            continue;
         }
-        if (node == MCEV_NO_NODE) {
-            if (sp == base) return false;
-            node = stack[SIDX(--sp)];
-        }
-        const Node n = load_node(sc.nodes, node);
-        work.x += 1;
-        float tl, tr;
-        const int m = node_hits(r, n, tmin, tmax, tl, tr);
-        const bool lh = (m & 1) && n.d.x < 0, rh = (m & 2) && n.d.y < 0;
-        pfirst = lh ? ~n.d.x : ~n.d.y;
-        pcount = (lh ? n.d.z : 0) + (rh ? n.d.w : 0);
-        const bool gl = (m & 1) && n.d.x >= 0;
-        const bool gr = (m & 2) && n.d.y >= 0;
-        int next = MCEV_NO_NODE;
-        if (gl && gr) {
-#if MCEV_ANY_ORDERED
-            const int nearc = tl <= tr ? n.d.x : n.d.y;
-            const int farc = tl <= tr ? n.d.y : n.d.x;
-#else
-            const int nearc = n.d.x;
-            const int farc = n.d.y;
-#endif
-            if (sp < MCEV_STACK) stack[SIDX(sp++)] = farc;
-            else *err = 1;
-            next = nearc;
-        } else if (gl) {
-            next = n.d.x;
-        } else if (gr) {
-            next = n.d.y;
-        }
-        node = next;
     }
 }
 
@@ -589,285 +769,73 @@ __device__ __forceinline__ WRay object_ray(const DevFrame& fr, int rec, f3 o, f3
     return make_wray(xf_point(i0, i1, i2, o), xf_vec(i0, i1, i2, d));
 }
 
-// BLAS traversal of either layout; `stack`/`base` are the two-wide stack,
-// `wstack` the wide one.  work.z (box tests) is kept for the wide layout only:
-// a two-wide node fetch always tests two boxes.
-template <bool kWide>
-__device__ __forceinline__ void blas_closest_any_layout(const DevScene& sc, int root, int rec, int inst, const WRay& r,
-                                                        float tmin, Hit& h, int* stack, int base, uint2* wstack,
-                                                        int* err, int3& work) {
-    if (kWide) {
-        blas_wide<false>(sc, (uint32_t)root, rec, inst, r, tmin, 0.0f, h, wstack, err, work);
-    } else {
-        blas_closest(sc, root, rec, inst, r, tmin, h, stack, base, err, work);
-    }
-}
-
-template <bool kWide>
-__device__ __forceinline__ bool blas_any_layout(const DevScene& sc, int root, const WRay& r, float tmin, float tmax,
-                                                int* stack, int base, uint2* wstack, int* err, int3& work) {
-    if (kWide) {
-        Hit dummy;
-        return blas_wide<true>(sc, (uint32_t)root, 0, 0, r, tmin, tmax, dummy, wstack, err, work);
-    }
-    return blas_any(sc, root, r, tmin, tmax, stack, base, err, work);
-}
-
-#define MCEV_DECLARE_WSTACK(name) uint2 name[kWide ? MCEV_WSTACK : 1]
-
-// The slab-test part of make_wray (reciprocal direction and origin times it),
-// enough for TLAS box tests; the same arithmetic as make_wray.
-__device__ __forceinline__ void slab_ray(WRay& r, f3 o, f3 d) {
-    const float ooeps = 0x1p-80f;
-    r.idir = mk3(1.0f / (fabsf(d.x) > ooeps ? d.x : copysignf(ooeps, d.x)),
-                 1.0f / (fabsf(d.y) > ooeps ? d.y : copysignf(ooeps, d.y)),
-                 1.0f / (fabsf(d.z) > ooeps ? d.z : copysignf(ooeps, d.z)));
-    r.oidir = mk3(o.x * r.idir.x, o.y * r.idir.y, o.z * r.idir.z);
-}
-
-// Two-level traversal of the moving instances (TLAS, then each hit
-// instance's two-wide BLAS) as ONE loop: an iteration is a TLAS node step, a
-// BLAS node step or one pending leaf triangle, whatever the lane is at, so
-// lanes that entered different instances at different TLAS steps still
-// advance together (with the BLAS loop nested in the TLAS loop, a warp ran
-// the BLAS loop once for every group of lanes that reached a TLAS leaf
-// together).  A TLAS step records its hit leaf children (one instance record
-// each) as pending; they are entered before the next TLAS step, the TLAS node
-// in hand waiting on the stack.  BLAS nodes are stacked above `base`, the
-// TLAS stack height when the instance was entered.  kAny: any hit in
-// (tmin, tmax]; else closest hit into h.  Returns whether an occluder was found
-// (kAny).
-template <bool kAny>
-__device__ __forceinline__ bool two_level(const DevScene& sc, const DevFrame& fr, f3 o, f3 d, float tmin,
-                                          float tmax, Hit& h, int* stack, int* err, int3& work) {
-    WRay r;
-    slab_ray(r, o, d);
-    bool in_blas = false;
-    int sp = 0, base = 0, node = 0;
-    int pfirst = 0, pcount = 0;
-    int pend0 = -1, pend1 = -1;
-    int rec = -1, inst = -1;
-    while (true) {
-        if (pcount > 0) {
-            const float4* tp = sc.tris + 3 * pfirst;
-            const float4 p0 = __ldg(tp), p1 = __ldg(tp + 1), p2 = __ldg(tp + 2);
-            work.y += 1;
-            const float t = tri_hit(r, p0, p1, p2, tmin, kAny ? tmax : h.t);
-            if (kAny) {
-                if (t >= 0.0f) return true;
-            } else {
-                const int oi = inst >= 0 ? inst : __float_as_int(p2.w);
-                if (t >= 0.0f && better_hit(t, oi, __float_as_int(p0.w), h)) {
-                    h.t = t; h.inst = oi; h.tri = pfirst; h.prim = __float_as_int(p0.w); h.rec = rec;
-                }
-            }
-            ++pfirst;
-            --pcount;
-            continue;
-        }
-        if (!in_blas && pend0 >= 0) {
-            if (node != MCEV_NO_NODE) {
-                if (sp < MCEV_STACK) stack[SIDX(sp++)] = node;
-                else *err = 1;
-            }
-            rec = pend0;
-            pend0 = pend1;
-            pend1 = -1;
-            r = object_ray(fr, rec, o, d, node, inst);
-            in_blas = true;
-            base = sp;
-        }
-        if (node == MCEV_NO_NODE) {
-            if (in_blas && sp == base) {
-                // instance done: back to the TLAS
-                in_blas = false;
-                slab_ray(r, o, d);
-                if (pend0 >= 0) continue;
-            }
-            if (sp == 0) break;
-            node = stack[SIDX(--sp)];
-        }
-        const Node n = load_node(in_blas ? sc.nodes : fr.tlas, node);
-        work.x += 1;
-        float tl, tr;
-        const float tcut = kAny ? tmax : h.t;
-        const int m = node_hits(r, n, tmin, tcut, tl, tr);
-        const bool lh = (m & 1) && n.d.x < 0, rh = (m & 2) && n.d.y < 0;
-        if (in_blas) {
-            pfirst = lh ? ~n.d.x : ~n.d.y;
-            pcount = (lh ? n.d.z : 0) + (rh ? n.d.w : 0);
-        } else {
-            pend0 = lh ? ~n.d.x : (rh ? ~n.d.y : -1);
-            pend1 = (lh && rh) ? ~n.d.y : -1;
-        }
-        const bool gl = (m & 1) && n.d.x >= 0 && (kAny || tl <= h.t);
-        const bool gr = (m & 2) && n.d.y >= 0 && (kAny || tr <= h.t);
-        int next = MCEV_NO_NODE;
-        if (gl && gr) {
-            // nearer child first (any-hit: in BLAS only, as blas_any does)
-            const bool lfirst = kAny ? (!(MCEV_ANY_ORDERED && in_blas) || tl <= tr) : tl <= tr;
-            if (sp < MCEV_STACK) stack[SIDX(sp++)] = lfirst ? n.d.y : n.d.x;
-            else *err = 1;
-            next = lfirst ? n.d.x : n.d.y;
-        } else if (gl) {
-            next = n.d.x;
-        } else if (gr) {
-            next = n.d.y;
-        }
-        node = next;
-    }
-    return false;
-}
-
-// world-space closest hit over the two-level hierarchy (the TLAS is two-wide;
-// BLAS in the scene's layout): the merged never-moving geometry first, then
-// the TLAS of the moving instances, whose boxes the hit found so far culls.
+// Closest hits of the whole warp's world-space rays over the two-level
+// hierarchy with wide BLASes (the TLAS is two-wide): the merged never-moving
+// geometry first, then the TLAS of the moving instances, whose boxes the hit
+// found so far culls.  Lanes step through the TLAS until each has an instance
+// to enter or is done, then traverse their instances together.  kAny: whether
+// there is an occluder in (tmin, tmax].
 // work: (node fetches, triangle tests, box tests of the wide layout)
-template <bool kWide, bool kTlas>
-__device__ __forceinline__ Hit closest_hit(const DevScene& sc, const DevFrame& fr, f3 o, f3 d, float tmin, int* err,
+template <bool kAny>
+__device__ __forceinline__ bool trace_wide(const DevScene& sc, const DevFrame& fr, const float4* op, const float4* dp,
+                                           bool live, float tmin, float tmax, Hit& h, int* stack, int* err,
                                            int3& work) {
-    Hit h;
+    const unsigned full = 0xffffffffu;
+    uint2 wstack[MCEV_WSTACK];
     h.t = __int_as_float(0x7f800000);
-    h.inst = -1;
-    h.tri = -1;
-    h.prim = -1;
-    h.rec = -1;
-    MCEV_DECLARE_STACK(stack);
-    MCEV_DECLARE_WSTACK(wstack);
-    if (fr.static_rec >= 0) {
-        int root, oi;
-        const WRay r = object_ray(fr, fr.static_rec, o, d, root, oi);
-        blas_closest_any_layout<kWide>(sc, root, fr.static_rec, oi, r, tmin, h, stack, 0, wstack, err, work);
-    }
-    if (fr.n_tlas == 0) return h;
-    if (!kTlas || fr.n_tlas == 1) {
-        // (kTlas = false is launched only for frames with at most one moving instance)
-        int root, oi;
-        const WRay r = object_ray(fr, 0, o, d, root, oi);
-        blas_closest_any_layout<kWide>(sc, root, 0, oi, r, tmin, h, stack, 0, wstack, err, work);
-        return h;
-    }
-    if (!kWide) {
-        two_level<false>(sc, fr, o, d, tmin, 0.0f, h, stack, err, work);
-        return h;
-    }
-    // wide BLAS: the TLAS loop with each instance's traversal nested in it
-    const WRay wr = make_wray(o, d);
+    h.inst = h.tri = h.prim = h.rec = -1;
+    int rec = live ? fr.static_rec : -1;
+    int node = live && fr.n_tlas >= 2 ? 0 : MCEV_NO_NODE;
+    int pend0 = live && fr.n_tlas == 1 ? 0 : -1, pend1 = -1;
     int sp = 0;
-    int node = 0;
-    while (true) {
-        const Node n = load_node(fr.tlas, node);
-        work.x += 1;
-        if (kWide) work.z += 2;
-        float tl, tr;
-        const int m = node_hits(wr, n, tmin, h.t, tl, tr);
-        for (int side = 0; side < 2; ++side) {
-            const int child = side ? n.d.y : n.d.x;
-            const int cnt = side ? n.d.w : n.d.z;
-            if ((m & (1 << side)) && child < 0) {
-                for (int i = 0; i < cnt; ++i) {
-                    const int rec = ~child + i;
-                    int root, oi;
-                    const WRay r = object_ray(fr, rec, o, d, root, oi);
-                    blas_closest_any_layout<kWide>(sc, root, rec, oi, r, tmin, h, stack, sp, wstack, err, work);
+    bool found = false;
+    while (__any_sync(full, rec >= 0 || pend0 >= 0 || node != MCEV_NO_NODE || sp > 0)) {
+        while (true) {
+            if (rec < 0) {
+                rec = pend0;
+                pend0 = pend1;
+                pend1 = -1;
+            }
+            const bool step = rec < 0 && (node != MCEV_NO_NODE || sp > 0);
+            if (!__any_sync(full, step)) break;
+            if (step) {
+                if (node == MCEV_NO_NODE) node = stack[--sp];
+                TRay wr;
+                slab_setup(wr, xyz(*op), xyz(*dp));
+                const Node n = load_node(fr.tlas, node);
+                work.x += 1;
+                work.z += 2;
+                float tl, tr;
+                const int m = node_hits(wr, n, tmin, kAny ? tmax : h.t, tl, tr);
+                const bool lh = (m & 1) && n.d.x < 0, rh = (m & 2) && n.d.y < 0;
+                pend0 = lh ? ~n.d.x : (rh ? ~n.d.y : -1);
+                pend1 = (lh && rh) ? ~n.d.y : -1;
+                const bool gl = (m & 1) && n.d.x >= 0 && (kAny || tl <= h.t);
+                const bool gr = (m & 2) && n.d.y >= 0 && (kAny || tr <= h.t);
+                node = gl ? n.d.x : (gr ? n.d.y : MCEV_NO_NODE);
+                if (gl && gr) {
+                    const bool lfirst = tl <= tr;
+                    if (sp < MCEV_STACK) stack[sp++] = lfirst ? n.d.y : n.d.x;
+                    else *err = 1;
+                    node = lfirst ? n.d.x : n.d.y;
                 }
             }
         }
-        const bool gl = (m & 1) && n.d.x >= 0 && tl <= h.t;
-        const bool gr = (m & 2) && n.d.y >= 0 && tr <= h.t;
-        int next = -0x7fffffff;
-        if (gl && gr) {
-            const int nearc = tl <= tr ? n.d.x : n.d.y;
-            const int farc = tl <= tr ? n.d.y : n.d.x;
-            if (sp < MCEV_STACK) stack[SIDX(sp++)] = farc;
-            else *err = 1;
-            next = nearc;
-        } else if (gl) {
-            next = n.d.x;
-        } else if (gr) {
-            next = n.d.y;
-        }
-        if (next == -0x7fffffff) {
-            if (sp == 0) break;
-            next = stack[SIDX(--sp)];
-        }
-        node = next;
-    }
-    return h;
-}
-
-template <bool kWide, bool kTlas>
-__device__ __forceinline__ bool occluded(const DevScene& sc, const DevFrame& fr, f3 o, f3 d, float tmin, float tmax,
-                                         int* err, int3& work) {
-    MCEV_DECLARE_STACK(stack);
-    MCEV_DECLARE_WSTACK(wstack);
-    if (fr.static_rec >= 0) {
-        int root, oi;
-        const WRay r = object_ray(fr, fr.static_rec, o, d, root, oi);
-        if (blas_any_layout<kWide>(sc, root, r, tmin, tmax, stack, 0, wstack, err, work)) return true;
-    }
-    if (fr.n_tlas == 0) return false;
-    if (!kTlas || fr.n_tlas == 1) {
-        int root, oi;
-        const WRay r = object_ray(fr, 0, o, d, root, oi);
-        return blas_any_layout<kWide>(sc, root, r, tmin, tmax, stack, 0, wstack, err, work);
-    }
-    if (!kWide) {
-        Hit dummy;
-        return two_level<true>(sc, fr, o, d, tmin, tmax, dummy, stack, err, work);
-    }
-    const WRay wr = make_wray(o, d);
-    int sp = 0;
-    int node = 0;
-    while (true) {
-        const Node n = load_node(fr.tlas, node);
-        work.x += 1;
-        if (kWide) work.z += 2;
-        float tl, tr;
-        const int m = node_hits(wr, n, tmin, tmax, tl, tr);
-        for (int side = 0; side < 2; ++side) {
-            const int child = side ? n.d.y : n.d.x;
-            const int cnt = side ? n.d.w : n.d.z;
-            if ((m & (1 << side)) && child < 0) {
-                for (int i = 0; i < cnt; ++i) {
-                    const int rec = ~child + i;
-                    int root, oi;
-                    const WRay r = object_ray(fr, rec, o, d, root, oi);
-                    if (blas_any_layout<kWide>(sc, root, r, tmin, tmax, stack, sp, wstack, err, work)) return true;
-                }
+        const bool on = rec >= 0;
+        if (__any_sync(full, on)) {
+            int root = 0, oi = -1;
+            WRay r;
+            if (on) r = object_ray(fr, rec, xyz(*op), xyz(*dp), root, oi);
+            if (blas_wide<kAny>(sc, (uint32_t)root, rec, oi, r, on, tmin, tmax, h, wstack, err, work)) {
+                found = true;
+                pend0 = -1;
+                node = MCEV_NO_NODE;
+                sp = 0;
             }
+            rec = -1;
         }
-        const bool gl = (m & 1) && n.d.x >= 0;
-        const bool gr = (m & 2) && n.d.y >= 0;
-        int next = -0x7fffffff;
-        if (gl && gr) {
-            if (sp < MCEV_STACK) stack[SIDX(sp++)] = n.d.y;
-            else *err = 1;
-            next = n.d.x;
-        } else if (gl) {
-            next = n.d.x;
-        } else if (gr) {
-            next = n.d.y;
-        }
-        if (next == -0x7fffffff) {
-            if (sp == 0) return false;
-            next = stack[SIDX(--sp)];
-        }
-        node = next;
     }
-}
-
-// ------------------------------------------------------------------ warp-aggregated append
-__device__ __forceinline__ int warp_append(int* counter, bool pred) {
-    const unsigned mask = __activemask();
-    const unsigned ballot = __ballot_sync(mask, pred);
-    if (!pred) return -1;
-    const int lane = threadIdx.x & 31;
-    const int leader = __ffs(ballot) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(counter, __popc(ballot));
-    base = __shfl_sync(ballot, base, leader);
-    return base + __popc(ballot & ((1u << lane) - 1u));
+    return found;
 }
 
 }  // namespace mcev

@@ -1,14 +1,15 @@
 // kernels.cu -- wavefront path tracer and statistical event detector.
 //
 // One chunk of paths goes through
-//   raygen -> [extend -> shade(+NEE) -> shadow] x (max_depth + 1) -> stats
-// where extend/shade/shadow consume device-side ray queues (sizes in device
-// counters, no host round trip) and `stats` fuses, per queued pixel, the
-// log-luminance batch statistics (Sec. 3.1, Eq. 3-4), the Chan merge into the
-// running statistics, the t-test of Eq. 7 (Sec. 3.2), the re-queue of
-// undecided pixels (Sec. 3.3; one atomic per warp, since a warp owns a pixel)
-// and the event rule with the reference update (Alg. 1, Eq. 1).  Rays and
-// shadow rays are appended to their queues with warp-aggregated atomics.
+//   raygen -> extend -> [shade(+NEE) -> queue -> shadow + extend] x max_depth -> shade -> stats
+// Every path keeps one slot of the wavefront for its ray and state; extend,
+// shade and shadow walk device-side queues of slots (sizes in device
+// counters, no host round trip) that `queue` fills tile by tile in direction
+// order.  `stats` fuses, per queued pixel, the log-luminance batch statistics
+// (Sec. 3.1, Eq. 3-4), the Chan merge into the running statistics, the t-test
+// of Eq. 7 (Sec. 3.2), the re-queue of undecided pixels (Sec. 3.3; one atomic
+// per warp, since a warp owns a pixel) and the event rule with the reference
+// update (Alg. 1, Eq. 1).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -21,24 +22,32 @@
 
 namespace mcev {
 
-// Minimum resident blocks per SM requested for the traversal kernels: 9
-// blocks of 128 threads cap them at 56 registers (56% occupancy); traversal
-// waits on node fetches, so more resident warps pay more than the few
-// registers spilled (terrain frame traversal: 72 registers 1011 ms, 64
-// registers 967 ms, 56 registers 943 ms, 48 registers 961 ms; whole terrain
-// frames with the kernels that carry no TLAS code: 64 / 56 / 48 registers
-// 1332 / 1289 / 1306 ms).  0 leaves the choice to the compiler.
-#ifndef MCEV_TRAV_MINB
-#define MCEV_TRAV_MINB 9
-#endif
-// The wide-node traversal keeps a whole node (five 16-byte words) and its
-// eight child tests in flight: it gets its own cap.
-#ifndef MCEV_WIDE_MINB
-#define MCEV_WIDE_MINB 8
-#endif
-#define MCEV_TRAV_BOUNDS __launch_bounds__(MCEV_TRAV_BLOCK, kWide ? MCEV_WIDE_MINB : MCEV_TRAV_MINB)
+// Resident blocks of 128 threads per SM of the traversal kernel, which fix its
+// registers: 10 blocks (48) for the two-wide layout; traversal waits on node
+// fetches, so more warps pay (terrain frame at 9 / 10 / 12 blocks: 778 / 766 /
+// 767 ms, the last spilling at 40 registers; eight batched jobs at 8 / 9 / 10
+// blocks 140.9 / 136.9 / 135.4 ms).  The TLAS loop carries more state (frames of
+// 12 moving spheres at 8 / 9 / 10 blocks 15.9 / 15.7 / 16.6 ms).  The wide-node
+// traversal keeps a whole node (five 16-byte words) and its eight child tests in
+// flight.
+__host__ __device__ constexpr int trav_blocks(bool wide, bool tlas) {
+    return wide ? 8 : (tlas ? 9 : 10);
+}
 
 static constexpr uint32_t NO_FLAGS = 0xFFFFFFFFu;
+
+// Direction cell of a ray for the queues' order: its octant (which plane of a
+// box is near on each axis) and its dominant axis (the shear of the
+// watertight test), so rays of one cell take the same side of every
+// sign-dependent choice of the traversal.
+static constexpr uint32_t KEY_NONE = 0xFFu;
+static constexpr int KEY_CELLS = 32;    // 24 used
+__device__ __forceinline__ uint32_t dir_cell(f3 d) {
+    const float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
+    const uint32_t kz = (ay > ax && ay >= az) ? 1u : ((az > ax && az > ay) ? 2u : 0u);
+    const uint32_t oct = (d.x < 0.0f ? 1u : 0u) | (d.z < 0.0f ? 2u : 0u) | (d.y < 0.0f ? 4u : 0u);
+    return 3u * oct + kz;
+}
 
 // shadow-ray count of the bounce whose ray queue is `cur` (double-buffered so
 // a launch can trace one bounce's shadow rays while the next bounce's shade
@@ -67,6 +76,7 @@ __global__ void __launch_bounds__(256) k_raygen(DevFrame fr, DevParams P, Wave w
         w.counters[cur] = (int32_t)n_paths;
         w.counters[1 - cur] = 0;
         w.counters[2] = w.counters[19] = 0;
+        w.counters[20] = 0;
     }
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n_paths; p += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = p / spp_r;
@@ -84,11 +94,10 @@ __global__ void __launch_bounds__(256) k_raygen(DevFrame fr, DevParams P, Wave w
         const f3 d = norm3(mk3(F.fwd[0] + fx * F.right[0] + fy * F.up[0],
                                F.fwd[1] + fx * F.right[1] + fy * F.up[1],
                                F.fwd[2] + fx * F.right[2] + fy * F.up[2]));
-        w.ray_o[cur][p] = make_float4(F.eye[0], F.eye[1], F.eye[2], __int_as_float((int)p));
-        w.ray_d[cur][p] = make_float4(d.x, d.y, d.z, __int_as_float(job << 8));
+        w.ray_o[p] = make_float4(F.eye[0], F.eye[1], F.eye[2], 1.0f);
+        w.ray_d[p] = make_float4(d.x, d.y, d.z, 0.0f);
         w.L[p] = 0.0f;
-        if (kBatch) w.pix_k[p] = make_int2(entry, (int)k);   // the shadow kernel's job lookup
-        w.ray_s[cur][p] = make_float4(1.0f, 0.0f, __int_as_float(entry), __int_as_float((int)k));
+        w.pix_k[p] = make_int2(entry, (int)k);
         if (Q.adjoint && Q.grad_mean) {
             // d loss / d L of this path: d loss / d mean * d mean / d ln(L + eps) * d ln(L + eps) / dL
             const float Lt = w.Ltot[p];
@@ -101,17 +110,13 @@ __global__ void __launch_bounds__(256) k_raygen(DevFrame fr, DevParams P, Wave w
     }
 }
 
-// traversal work counters: 64-bit (nodes, tris) pairs after the int32
-// counters, and the ray/box tests (two per node fetch of the two-wide BVH)
-enum { WORK_CLOSEST = 0, WORK_SHADOW = 1 };
 // Per-block accumulation of the traversal work counters: work_begin at the
-// top of a ray loop (every thread of the block), add_work after it.  Each
-// warp adds its sums in shared memory; the last warp of the block to finish
-// adds the block's totals to the global counters (skipped when the block
-// traced nothing), so a launch's global atomics on these three words scale
-// with its busy blocks, not with its warps, and no warp waits for another.
+// top of the kernel, add_work at its end.  Each warp adds its sums in shared
+// memory; the last warp of the block to finish adds the block's totals to
+// the global counters, so no warp waits for another.  v: nodes, triangles
+// and box tests of closest-hit rays, then of shadow rays.
 struct WorkAcc {
-    unsigned long long v[3];
+    unsigned long long v[6];
     unsigned int done;
 };
 
@@ -122,79 +127,41 @@ __device__ __forceinline__ WorkAcc& work_acc() {
 
 __device__ __forceinline__ void work_begin() {
     WorkAcc& a = work_acc();
-    if (threadIdx.x == 0) {
-        a.v[0] = a.v[1] = a.v[2] = 0ull;
-        a.done = 0u;
-    }
+    if (threadIdx.x < 6) a.v[threadIdx.x] = 0ull;
+    if (threadIdx.x == 0) a.done = 0u;
     __syncthreads();
 }
 
-template <bool kWide>
-__device__ __forceinline__ void add_work(const Wave& w, int which, int3 work) {
-    WorkAcc& a = work_acc();
-    // the whole warp, reconverged after its ray loop: one count per warp
-    __syncwarp();
+__device__ __forceinline__ void warp_work(WorkAcc& a, int at, int3 work) {
     const unsigned m = 0xffffffffu;
     const int nodes = __reduce_add_sync(m, work.x);
     const int tris = __reduce_add_sync(m, work.y);
-    const int boxes = kWide ? __reduce_add_sync(m, work.z) : 2 * nodes;
+    const int boxes = __reduce_add_sync(m, work.z);
+    if ((threadIdx.x & 31) == 0 && (nodes | tris)) {
+        atomicAdd(&a.v[at], (unsigned long long)nodes);
+        atomicAdd(&a.v[at + 1], (unsigned long long)tris);
+        atomicAdd(&a.v[at + 2], (unsigned long long)boxes);
+    }
+}
+
+// the whole warp, converged after its ray loops
+__device__ __forceinline__ void add_work(const Wave& w, int3 closest, int3 shadow) {
+    WorkAcc& a = work_acc();
+    warp_work(a, 0, closest);
+    warp_work(a, 3, shadow);
     if ((threadIdx.x & 31) == 0) {
-        if (nodes | tris) {
-            atomicAdd(&a.v[0], (unsigned long long)nodes);
-            atomicAdd(&a.v[1], (unsigned long long)tris);
-            atomicAdd(&a.v[2], (unsigned long long)boxes);
-        }
         __threadfence_block();
         if (atomicAdd(&a.done, 1u) == (blockDim.x >> 5) - 1u) {
             __threadfence_block();
-            const unsigned long long n0 = atomicAdd(&a.v[0], 0ull), n1 = atomicAdd(&a.v[1], 0ull),
-                                     n2 = atomicAdd(&a.v[2], 0ull);
-            if (n0 | n1) {
-                unsigned long long* c = reinterpret_cast<unsigned long long*>(w.counters + 32);
-                atomicAdd(c + 2 * which, n0);
-                atomicAdd(c + 2 * which + 1, n1);
-                atomicAdd(c + 7 + which, n2);
+            // 64-bit words after the int32 counters (layout.h)
+            unsigned long long* c = reinterpret_cast<unsigned long long*>(w.counters + 32);
+            const int word[6] = {0, 1, 7, 2, 3, 8};
+            for (int i = 0; i < 6; ++i) {
+                const unsigned long long v = atomicAdd(&a.v[i], 0ull);
+                if (v) atomicAdd(c + word[i], v);
             }
         }
     }
-}
-
-// ------------------------------------------------------------------ extend
-// Closest hits of the rays of queue `cur`, indices first, first + stride, ...
-// The first thread also clears the queue and shadow counters shade(cur) will
-// append to.
-template <bool kBatch, bool kWide, bool kTlas>
-__device__ __forceinline__ void extend_rays(const DevScene& sc, const DevFrame& fr, float t_min, const Wave& w,
-                                            int cur, int32_t* err, const Job* __restrict__ jobs, int64_t first,
-                                            int64_t stride) {
-    const int32_t n = *(volatile int32_t*)(w.counters + cur);
-    if (first == 0) {
-        w.counters[1 - cur] = 0;
-        w.counters[sh_slot(cur)] = 0;
-        atomicAdd(reinterpret_cast<unsigned long long*>(w.counters + 32) + 4, (unsigned long long)n);
-    }
-    int e = 0;
-    int3 work = make_int3(0, 0, 0);
-    work_begin();
-    for (int64_t i = first; i < n; i += stride) {
-        const float4 o = w.ray_o[cur][i];
-        const float4 d = w.ray_d[cur][i];
-        const int job = kBatch ? (__float_as_int(d.w) >> 8) : 0;
-        const DevScene& S = kBatch ? jobs[job].sc : sc;
-        const DevFrame& F = kBatch ? jobs[job].fr : fr;
-        const float tmin = kBatch ? jobs[job].P.t_min : t_min;
-        const Hit h = closest_hit<kWide, kTlas>(S, F, xyz(o), xyz(d), tmin, &e, work);
-        w.hit[i] = make_float4(h.t, __int_as_float(h.inst), __int_as_float(h.tri), __int_as_float(h.rec));
-    }
-    if (e) atomicOr(err, 1);
-    add_work<kWide>(w, WORK_CLOSEST, work);
-}
-
-template <bool kBatch, bool kWide, bool kTlas>
-__global__ void MCEV_TRAV_BOUNDS k_extend(DevScene sc, DevFrame fr, float t_min, Wave w, int cur, int32_t* err,
-                                          const Job* __restrict__ jobs) {
-    extend_rays<kBatch, kWide, kTlas>(sc, fr, t_min, w, cur, err, jobs, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
-                               (int64_t)gridDim.x * blockDim.x);
 }
 
 // ------------------------------------------------------------------ shade + NEE + BSDF sampling
@@ -209,27 +176,27 @@ __global__ void MCEV_TRAV_BOUNDS k_extend(DevScene sc, DevFrame fr, float t_min,
 #define MCEV_SHADE_BOUNDS __launch_bounds__(128)
 #endif
 template <bool kBatch>
-__global__ void MCEV_SHADE_BOUNDS k_shade(DevScene sc, DevFrame fr, DevParams P, Wave w, int cur,
+__global__ void MCEV_SHADE_BOUNDS k_shade(DevScene sc, DevFrame fr, DevParams P, Wave w, int cur, int depth,
                                           const Job* __restrict__ jobs) {
     const int32_t n = *(volatile int32_t*)(w.counters + cur);
+    const int32_t* list = depth > 0 ? w.list[cur] : nullptr;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const float4 ro = w.ray_o[cur][i];
-        const float4 rd = w.ray_d[cur][i];
-        const int p = __float_as_int(ro.w);
-        const int depth = __float_as_int(rd.w) & 0xFF;
-        const int job = kBatch ? (__float_as_int(rd.w) >> 8) : 0;
+        const int p = list ? __ldg(list + i) : i;
+        const float4 ro = w.ray_o[p];
+        const float4 rd = w.ray_d[p];
+        const int2 rs = w.pix_k[p];
+        const int job = kBatch ? (int)((uint32_t)rs.x >> 24) : 0;
         const DevScene& S = kBatch ? jobs[job].sc : sc;
         const DevFrame& F = kBatch ? jobs[job].fr : fr;
         const DevParams& Q = kBatch ? jobs[job].P : P;
-        const float4 hv = w.hit[i];
-        const int inst = __float_as_int(hv.y);
-        const float4 rs = w.ray_s[cur][i];
-        float beta = rs.x;
+        const float2 hv = w.hit[p];
+        const int tri = __float_as_int(hv.y);
+        float beta = ro.w;
         // radiance this vertex adds to the path (emission on a hit, the
         // environment on a miss); the path's total is updated only when
         // something is added
         float Ladd = 0.0f;
-        const float pdf_prev = rs.y;
+        const float pdf_prev = rd.w;
         float pdf_next = 0.0f;
         uint32_t sig = 0, pflags = NO_FLAGS;
         if (Q.want_sig) {
@@ -242,7 +209,7 @@ __global__ void MCEV_SHADE_BOUNDS k_shade(DevScene sc, DevFrame fr, DevParams P,
         f3 P0 = mk3(0, 0, 0), wi_next = mk3(0, 0, 0), sh_dir = mk3(0, 0, 0);
         float sh_tmax = 0.0f, sh_c = 0.0f, sh_g = 0.0f;
         int sh_m = -1;
-        if (inst < 0) {
+        if (tri < 0) {
             // miss: environment radiance (Sec. 3.1 samples the light reaching the pixel)
             if (Q.want_sig) sig = fnv(sig, 0xFFFFFFFFu);
             if (S.has_env) {
@@ -258,17 +225,17 @@ __global__ void MCEV_SHADE_BOUNDS k_shade(DevScene sc, DevFrame fr, DevParams P,
                 sig = fnv(sig, 0xFFFFFFFEu);
             }
         } else {
-            const int tri = __float_as_int(hv.z);
+            const int rec = F.n_inst > 1 ? w.hit_rec[p] : 0;
             // the shading record (edge cross product, material) serves most
             // hits; the vertices are read only for textured albedo, emitter
             // MIS weights and the decision signature
             const float4 tsh = __ldg(S.tshade + tri);
             const float4* tp = S.tris + 3 * tri;
-            const float4* ip = F.inst + 7 * __float_as_int(hv.w);
+            const float4* ip = F.inst + 7 * rec;
             const float4 i0 = __ldg(ip + 3), i1 = __ldg(ip + 4), i2 = __ldg(ip + 5);
             const int ovr = __float_as_int(__ldg(ip + 6).y);
             if (Q.want_sig) {
-                sig = fnv(sig, (uint32_t)inst);
+                sig = fnv(sig, (uint32_t)hit_inst(F, rec, __ldg(tp + 2).w));
                 sig = fnv(sig, (uint32_t)__float_as_int(__ldg(tp).w));
             }
             const float t = hv.x;
@@ -333,8 +300,8 @@ __global__ void MCEV_SHADE_BOUNDS k_shade(DevScene sc, DevFrame fr, DevParams P,
                 f3 tb, bt;
                 onb(nn, tb, bt);
                 const f3 wol = mk3(dot3(wo, tb), dot3(wo, bt), dot3(wo, nn));
-                const uint32_t ent = (uint32_t)__float_as_int(rs.z);
-                const uint2 pk = make_uint2(kBatch ? (ent & 0xFFFFFFu) : ent, (uint32_t)__float_as_int(rs.w));
+                const uint32_t ent = (uint32_t)rs.x;
+                const uint2 pk = make_uint2(kBatch ? (ent & 0xFFFFFFu) : ent, (uint32_t)rs.y);
                 // next-event estimation
                 if (Q.nee && (S.env_ok || F.n_lights > 0)) {
                     const uint4 x = philox4x32_10(make_uint4(pk.x, pk.y, (uint32_t)(depth + 1), 0u), F.key0, F.key1);
@@ -401,78 +368,231 @@ __global__ void MCEV_SHADE_BOUNDS k_shade(DevScene sc, DevFrame fr, DevParams P,
             w.sig[p] = sig;
             w.pflags[p] = pflags;
         }
-        const int si = warp_append(w.counters + sh_slot(cur), shadow);
+        if (shadow || cont) w.ray_o[p] = make_float4(P0.x, P0.y, P0.z, beta);
         if (shadow) {
-            w.sh_o[si] = make_float4(P0.x, P0.y, P0.z, __int_as_float(p));
-            w.sh_d[si] = make_float4(sh_dir.x, sh_dir.y, sh_dir.z, sh_tmax);
-            w.sh_c[si] = sh_c;
+            w.sh_d[p] = make_float4(sh_dir.x, sh_dir.y, sh_dir.z, sh_tmax);
+            w.sh_c[p] = sh_c;
             if (Q.adjoint) {
-                w.sh_g[si] = sh_g;
-                w.sh_m[si] = sh_m;
+                w.sh_g[p] = sh_g;
+                w.sh_m[p] = sh_m;
             }
         }
-        const int ni = warp_append(w.counters + (1 - cur), cont);
-        if (cont) {
-            w.ray_o[1 - cur][ni] = make_float4(P0.x, P0.y, P0.z, __int_as_float(p));
-            w.ray_d[1 - cur][ni] = make_float4(wi_next.x, wi_next.y, wi_next.z, __int_as_float((depth + 1) | (job << 8)));
-            w.ray_s[1 - cur][ni] = make_float4(beta, pdf_next, rs.z, rs.w);
-        }
+        if (cont) w.ray_d[p] = make_float4(wi_next.x, wi_next.y, wi_next.z, pdf_next);
+        w.key[p] = (uint16_t)((cont ? dir_cell(wi_next) : KEY_NONE) | (shadow ? dir_cell(sh_dir) : KEY_NONE) << 8);
     }
 }
 
-// ------------------------------------------------------------------ shadow rays
-// the light sample of shadow ray i reaches path p: add its contribution
-__device__ __forceinline__ void shadow_unoccluded(const Wave& w, const DevParams& Q, int i, int p) {
-    w.L[p] += w.sh_c[i];
-    if (Q.want_sig) w.pflags[p] |= 4u;
-    if (Q.adjoint && Q.grad_emit && w.sh_m[i] >= 0) atomicAdd(Q.grad_emit + w.sh_m[i], (double)(w.delta[p] * w.sh_g[i]));
+// ------------------------------------------------------------------ ray queues
+// Queues the rays that shade left: per tile of Q_TILE consecutive entries of
+// the bounce's queue, the paths that go on and the ones with a shadow ray,
+// each grouped by direction cell (a counting sort in shared memory) and
+// appended with one atomic per tile.  Consecutive entries stay paths of
+// neighbouring pixels (the samples of a pixel are consecutive path slots, a
+// tile is 8 pixels at 512 samples), so a traversal warp holds rays that
+// start at nearly the same point and leave it in nearly the same direction.
+// What bounds it: the shared atomics of the ranks; it reads 8 B and writes 8 B
+// per ray.  Measured on the 1280x720 terrain frame against appending rays in
+// the order shade's warps finish (which mixes the pixels of a whole wave of
+// blocks): with the converged traversal loop: 687 ms with one cell per tile
+// (pixel order kept, no sort), 609 ms with the 24 cells, 624 and 614 ms with an
+// octahedral grid of 4 x 4 and 8 x 8 cells, 640 ms with the octants alone; queues
+// and shading 139, 139, 143, 148 and 136 ms (more cells scatter shade's reads).
+// Tiles of 2048 and 8192 entries within 1 % of 4096.
+static constexpr int Q_TILE = 4096, Q_BLOCK = 512, Q_ITEMS = Q_TILE / Q_BLOCK;
+
+__global__ void __launch_bounds__(Q_BLOCK) k_queue(Wave w, int cur, int depth) {
+    __shared__ int cnt[2][KEY_CELLS];   // next rays, shadow rays
+    __shared__ int qbase[2];
+    const int32_t n = *(volatile int32_t*)(w.counters + cur);
+    const int32_t* list = depth > 0 ? w.list[cur] : nullptr;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if (blockIdx.x == 0 && tid == 0) w.counters[20] = 0;   // the next traversal's cursor
+    // a small queue is cut into smaller tiles, so that every block has one
+    const int step = gridDim.x * Q_BLOCK;
+    const int items = max(1, min(Q_ITEMS, (n + step - 1) / step));
+    for (int64_t t0 = (int64_t)blockIdx.x * items * Q_BLOCK; t0 < n; t0 += (int64_t)step * items) {
+        if (tid < 2 * KEY_CELLS) (&cnt[0][0])[tid] = 0;
+        __syncthreads();
+        int p[Q_ITEMS];
+        uint32_t key[Q_ITEMS], rank[Q_ITEMS];
+#pragma unroll
+        for (int k = 0; k < Q_ITEMS; ++k) {
+            const int64_t i = t0 + k * Q_BLOCK + tid;
+            key[k] = KEY_NONE | (KEY_NONE << 8);
+            p[k] = 0;
+            if (k < items && i < n) {
+                p[k] = list ? __ldg(list + i) : (int)i;
+                key[k] = w.key[p[k]];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < Q_ITEMS; ++k) {
+            const uint32_t kn = key[k] & 0xFFu, ks = (key[k] >> 8) & 0xFFu;
+            rank[k] = 0;
+            if (kn != KEY_NONE) rank[k] = (uint32_t)atomicAdd(&cnt[0][kn], 1);
+            if (ks != KEY_NONE) rank[k] |= (uint32_t)atomicAdd(&cnt[1][ks], 1) << 16;
+        }
+        __syncthreads();
+        // exclusive scan over a queue's cells, one warp per queue
+        if (wid < 2) {
+            const int c = cnt[wid][lane];
+            int v = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += y;
+            }
+            cnt[wid][lane] = v - c;
+            if (lane == 31) qbase[wid] = v ? atomicAdd(w.counters + (wid ? sh_slot(cur) : 1 - cur), v) : 0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < Q_ITEMS; ++k) {
+            const uint32_t kn = key[k] & 0xFFu, ks = (key[k] >> 8) & 0xFFu;
+            if (kn != KEY_NONE) w.list[1 - cur][qbase[0] + cnt[0][kn] + (rank[k] & 0xFFFFu)] = p[k];
+            if (ks != KEY_NONE) w.sh_list[qbase[1] + cnt[1][ks] + (rank[k] >> 16)] = p[k];
+        }
+        __syncthreads();
+    }
 }
 
-// Shadow rays appended by shade(cur), indices first, first + stride, ...
-template <bool kBatch, bool kWide, bool kTlas>
-__device__ __forceinline__ void shadow_rays(const DevScene& sc, const DevFrame& fr, const DevParams& P,
-                                            const Wave& w, int cur, int32_t* err, const Job* __restrict__ jobs,
-                                            int64_t first, int64_t stride) {
-    const int32_t n = *(volatile int32_t*)(w.counters + sh_slot(cur));
-    if (first == 0) atomicAdd(reinterpret_cast<unsigned long long*>(w.counters + 32) + 5, (unsigned long long)n);
-    int e = 0;
-    int3 work = make_int3(0, 0, 0);
-    work_begin();
-    for (int64_t i = first; i < n; i += stride) {
-        const float4 o = w.sh_o[i];
-        const float4 d = w.sh_d[i];
-        const int p = __float_as_int(o.w);
+// ------------------------------------------------------------------ traversal
+// grad_emit[m] += v for the lanes with m >= 0 (the whole warp calls): one
+// atomic per material and warp.  The shadow rays of a warp go the same way, so
+// most of them sample one light, and their FP64 atomics on its word would
+// serialise.
+__device__ __forceinline__ void warp_add_emit(double* grad_emit, int m, double v) {
+    const unsigned full = 0xffffffffu;
+    unsigned todo = __ballot_sync(full, m >= 0);
+    while (todo) {
+        const int lead = __ffs(todo) - 1;
+        const int mm = __shfl_sync(full, m, lead);
+        double x = m == mm ? v : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(full, x, o);
+        if ((int)(threadIdx.x & 31) == lead) atomicAdd(grad_emit + mm, x);
+        todo &= ~__ballot_sync(full, m == mm);
+    }
+}
+
+// The groups of 32 consecutive queue entries that a warp of the traversal
+// kernel takes: first its own number, then the next of a device cursor, fetched
+// while the current group is traced.  Per-ray cost is heavy-tailed: a fixed
+// share of the queues per block left SMs idle at the end of a launch (terrain
+// frame traversal 650 ms -> 624 ms, sphere field 183 -> 178 ms; groups of 128
+// rays 635 and 181 ms).
+struct Groups {
+    int g, n_warps, total;   // current group, warps of the grid, groups of both queues
+    int32_t* cursor;
+    int ahead;               // lane 0: the group after g
+    __device__ __forceinline__ void prefetch() {
+        ahead = total;
+        if (n_warps < total && (threadIdx.x & 31) == 0) ahead = n_warps + atomicAdd(cursor, 1);
+    }
+    __device__ __forceinline__ void advance() { g = __shfl_sync(0xffffffffu, ahead, 0); }
+};
+
+// Traces the warp's groups below `g_end` of a queue whose first group is
+// `g0`, one ray per lane: closest hits (kAny = false) of `list` (null: slots
+// 0 .. n-1) into w.hit, or occlusion of the shadow rays.  (Refilling a warp's
+// idle lanes with further rays while others are still traced was slower on
+// the sphere field, 178 -> 200 ms and more at every threshold: the lanes' state
+// machine costs more than it fills.)
+template <bool kAny, bool kBatch, bool kWide, bool kTlas>
+__device__ __forceinline__ int3 trace_queue(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w,
+                                            const int32_t* __restrict__ list, int32_t n, Groups& gr, int g0, int g_end,
+                                            int* stack, int32_t* err, const Job* __restrict__ jobs) {
+    const int lane = threadIdx.x & 31;
+    const float4* dirs = kAny ? w.sh_d : w.ray_d;
+    int2 work = make_int2(0, 0);
+    int3 wwork = make_int3(0, 0, 0);
+    while (gr.g < g_end) {
+        gr.prefetch();
+        const int g = (gr.g - g0) * 32;
+        const bool live = g + lane < n;
+        const int i = live ? g + lane : n - 1;
+        const int p = list ? __ldg(list + i) : i;
         const int job = kBatch ? (int)((uint32_t)w.pix_k[p].x >> 24) : 0;
         const DevScene& S = kBatch ? jobs[job].sc : sc;
         const DevFrame& F = kBatch ? jobs[job].fr : fr;
         const DevParams& Q = kBatch ? jobs[job].P : P;
-        if (!occluded<kWide, kTlas>(S, F, xyz(o), xyz(d), Q.t_min, d.w, &e, work)) shadow_unoccluded(w, Q, (int)i, p);
+        const float4* op = w.ray_o + p;
+        const float4* dp = dirs + p;
+        const float tmin = Q.t_min;
+        THit h{kAny ? dp->w : __int_as_float(0x7f800000), -1, 0};
+        if (kWide) {
+            Hit wh;
+            int e = 0;
+            const bool occ = trace_wide<kAny>(S, F, op, dp, live, tmin, h.t, wh, stack, &e, wwork);
+            if (e) atomicOr(err, 1);
+            h = THit{wh.t, kAny ? (occ ? 0 : -1) : wh.tri, wh.rec};
+        } else {
+            // the merged never-moving geometry, then the one moving instance
+            // (variants without the TLAS are launched for frames with at most one)
+#pragma unroll 1
+            for (int step = 0; step < (kTlas ? 1 : 2); ++step) {
+                const int rec = step == 0 ? F.static_rec : (F.n_tlas > 0 ? 0 : -1);
+                if (!kBatch && rec < 0) continue;   // the same for the whole warp
+                const bool on = live && rec >= 0 && !(kAny && h.tri >= 0);
+                int root = 0;
+                TRay r;
+                if (on) r = object_tray(F, rec, op, dp, root);
+                two_wide<kAny>(S, F, root, rec, r, on, tmin, h, stack, err, work);
+            }
+            if (kTlas && (kBatch || F.n_tlas > 0))
+                two_level<kAny>(S, F, op, dp, live && F.n_tlas > 0 && !(kAny && h.tri >= 0), tmin, h, stack, err, work);
+        }
+        if (!kAny) {
+            if (live) {
+                w.hit[p] = make_float2(h.t, __int_as_float(h.tri));
+                if (F.n_inst > 1) w.hit_rec[p] = h.rec;
+            }
+        } else {
+            // the light sample reaches the path's vertex: add its contribution
+            const bool lit = live && h.tri < 0;
+            if (lit) {
+                w.L[p] += w.sh_c[p];
+                if (Q.want_sig) w.pflags[p] |= 4u;
+            }
+            if (!kBatch && P.adjoint && P.grad_emit) {
+                const int m = lit ? w.sh_m[p] : -1;
+                warp_add_emit(P.grad_emit, m, m >= 0 ? (double)(w.delta[p] * w.sh_g[p]) : 0.0);
+            }
+        }
+        gr.advance();
     }
-    if (e) atomicOr(err, 1);
-    add_work<kWide>(w, WORK_SHADOW, work);
+    return kWide ? wwork : make_int3(work.x, work.y, 2 * work.x);
 }
 
+// One launch traces the closest hits of bounce `depth` (ray queue `ecur`) and,
+// with scur >= 0, then the shadow rays of the bounce before (appended with queue
+// scur).
+// The grid is the resident warps only; queue sizes are read on the device.
+// The first thread also clears the counters the next queues append to.
 template <bool kBatch, bool kWide, bool kTlas>
-__global__ void MCEV_TRAV_BOUNDS k_shadow(DevScene sc, DevFrame fr, DevParams P, Wave w, int cur, int32_t* err,
-                                          const Job* __restrict__ jobs) {
-    shadow_rays<kBatch, kWide, kTlas>(sc, fr, P, w, cur, err, jobs, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
-                               (int64_t)gridDim.x * blockDim.x);
-}
-
-// One launch for the shadow rays of bounce d (appended by shade with queue
-// `cur`) and the closest hits of bounce d + 1 (queue 1 - cur): the first
-// `g_ext` blocks extend, the rest trace shadow rays.  Two independent traversal
-// workloads in one grid keep the SMs busy while the other's longest rays finish.
-template <bool kBatch, bool kWide, bool kTlas>
-__global__ void MCEV_TRAV_BOUNDS k_shadow_extend(DevScene sc, DevFrame fr, DevParams P, Wave w, int cur,
-                                                 int32_t g_ext, int32_t* err, const Job* __restrict__ jobs) {
-    if ((int32_t)blockIdx.x < g_ext)
-        extend_rays<kBatch, kWide, kTlas>(sc, fr, P.t_min, w, 1 - cur, err, jobs,
-                                   blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)g_ext * blockDim.x);
-    else
-        shadow_rays<kBatch, kWide, kTlas>(sc, fr, P, w, cur, err, jobs,
-                                   (blockIdx.x - g_ext) * (int64_t)blockDim.x + threadIdx.x,
-                                   (int64_t)(gridDim.x - g_ext) * blockDim.x);
+__global__ void __launch_bounds__(MCEV_TRAV_BLOCK, trav_blocks(kWide, kTlas))
+    k_trace(DevScene sc, DevFrame fr, DevParams P, Wave w, int ecur, int scur, int depth, int32_t* err,
+            const Job* __restrict__ jobs) {
+    int stack[MCEV_STACK];
+    work_begin();
+    const int32_t n = *(volatile int32_t*)(w.counters + ecur);
+    const int32_t ns = scur >= 0 ? *(volatile int32_t*)(w.counters + sh_slot(scur)) : 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        w.counters[1 - ecur] = 0;
+        w.counters[sh_slot(ecur)] = 0;
+        unsigned long long* c = reinterpret_cast<unsigned long long*>(w.counters + 32);
+        atomicAdd(c + 4, (unsigned long long)n);
+        if (ns) atomicAdd(c + 5, (unsigned long long)ns);
+    }
+    const int ge = (n + 31) >> 5;
+    Groups gr{(int)(blockIdx.x * (MCEV_TRAV_BLOCK / 32) + (threadIdx.x >> 5)), (int)gridDim.x * (MCEV_TRAV_BLOCK / 32),
+              ge + ((ns + 31) >> 5), w.counters + 20, 0};
+    const int3 wc = trace_queue<false, kBatch, kWide, kTlas>(sc, fr, P, w, depth > 0 ? w.list[ecur] : nullptr, n, gr, 0,
+                                                             ge, stack, err, jobs);
+    int3 ws = make_int3(0, 0, 0);
+    if (scur >= 0)
+        ws = trace_queue<true, kBatch, kWide, kTlas>(sc, fr, P, w, w.sh_list, ns, gr, ge, gr.total, stack, err, jobs);
+    add_work(w, wc, ws);
 }
 
 // ------------------------------------------------------------------ per-pixel statistics + test + requeue + events
@@ -678,16 +798,6 @@ __global__ void k_iota(int32_t* q, int64_t n) {
 }
 
 // ------------------------------------------------------------------ launchers
-// Traversal grids: up to 72 blocks of 128 threads per SM (8 waves of the 9
-// resident blocks), each thread striding over the ray queue.  Per-ray
-// traversal cost is heavy-tailed, and smaller per-block shares let the block
-// scheduler even out the SMs' ends (terrain frame: 16 / 36 / 72 / 144 blocks
-// per SM 1286 / 1245 / 1239 / 1261 ms; one ray per thread with no cap
-// 1992 ms, the empty blocks of late, small rounds costing more).
-#ifndef MCEV_TRAV_BLOCKS_PER_SM
-#define MCEV_TRAV_BLOCKS_PER_SM 72
-#endif
-
 static int grid_for(int64_t work, int block, int sms, int per_sm) {
     int64_t g = (work + block - 1) / block;
     const int64_t cap = (int64_t)sms * per_sm;
@@ -709,51 +819,38 @@ cudaError_t launch_raygen(const DevFrame& fr, const DevParams& P, const Wave& w,
     return cudaGetLastError();
 }
 
-// traversal launches: kBatch x kWide instantiations picked at run time
 // traversal kernels by (batched jobs, BLAS layout, moving instances under a TLAS)
-#define MCEV_TRAV_LAUNCH3(kernel, kb, grid, jobs_, ...)                                                   \
-    do {                                                                                                  \
-        if (trav & TRAV_WIDE) {                                                                           \
-            if (trav & TRAV_TLAS) kernel<kb, true, true><<<grid, MCEV_TRAV_BLOCK, 0, st>>>(__VA_ARGS__, jobs_); \
-            else kernel<kb, true, false><<<grid, MCEV_TRAV_BLOCK, 0, st>>>(__VA_ARGS__, jobs_);          \
-        } else {                                                                                          \
-            if (trav & TRAV_TLAS) kernel<kb, false, true><<<grid, MCEV_TRAV_BLOCK, 0, st>>>(__VA_ARGS__, jobs_); \
-            else kernel<kb, false, false><<<grid, MCEV_TRAV_BLOCK, 0, st>>>(__VA_ARGS__, jobs_);         \
-        }                                                                                                 \
-    } while (0)
-#define MCEV_TRAV_DISPATCH(kernel, grid, ...)                                                             \
-    do {                                                                                                  \
-        if (jobs) MCEV_TRAV_LAUNCH3(kernel, true, grid, jobs, __VA_ARGS__);                               \
-        else MCEV_TRAV_LAUNCH3(kernel, false, grid, nullptr, __VA_ARGS__);                                \
-    } while (0)
-
-cudaError_t launch_extend(const DevScene& sc, const DevFrame& fr, float t_min, const Wave& w, int cur, int64_t max_n,
-                          int32_t* err, int sms, cudaStream_t st, const Job* jobs, int trav) {
-    MCEV_TRAV_DISPATCH(k_extend, grid_for(max_n, MCEV_TRAV_BLOCK, sms, MCEV_TRAV_BLOCKS_PER_SM), sc, fr, t_min, w, cur,
-                       err);
+cudaError_t launch_trace(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int ecur, int scur,
+                         int depth, int64_t max_n, int32_t* err, int sms, cudaStream_t st, const Job* jobs, int trav) {
+    // both queues of at most max_n rays
+    const int64_t work = scur >= 0 ? 2 * max_n : max_n;
+#define MCEV_TRACE(kb, kw, kt)                                                                                      \
+    k_trace<kb, kw, kt><<<grid_for(work, MCEV_TRAV_BLOCK, sms, trav_blocks(kw, kt)), MCEV_TRAV_BLOCK, 0, st>>>( \
+        sc, fr, P, w, ecur, scur, depth, err, jobs)
+    switch ((jobs ? 4 : 0) | ((trav & TRAV_WIDE) ? 2 : 0) | ((trav & TRAV_TLAS) ? 1 : 0)) {
+    case 0: MCEV_TRACE(false, false, false); break;
+    case 1: MCEV_TRACE(false, false, true); break;
+    case 2:
+    case 3: MCEV_TRACE(false, true, true); break;
+    case 4: MCEV_TRACE(true, false, false); break;
+    case 5: MCEV_TRACE(true, false, true); break;
+    default: MCEV_TRACE(true, true, true); break;
+    }
+#undef MCEV_TRACE
     return cudaGetLastError();
 }
 
 cudaError_t launch_shade(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int cur,
-                         int64_t max_n, int sms, cudaStream_t st, const Job* jobs) {
+                         int depth, int64_t max_n, int sms, cudaStream_t st, const Job* jobs) {
     if (jobs)
-        k_shade<true><<<grid_for(max_n, 128, sms, 16), 128, 0, st>>>(sc, fr, P, w, cur, jobs);
+        k_shade<true><<<grid_for(max_n, 128, sms, 16), 128, 0, st>>>(sc, fr, P, w, cur, depth, jobs);
     else
-        k_shade<false><<<grid_for(max_n, 128, sms, 16), 128, 0, st>>>(sc, fr, P, w, cur, nullptr);
+        k_shade<false><<<grid_for(max_n, 128, sms, 16), 128, 0, st>>>(sc, fr, P, w, cur, depth, nullptr);
     return cudaGetLastError();
 }
 
-cudaError_t launch_shadow(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int cur,
-                          int64_t max_n, int32_t* err, int sms, cudaStream_t st, const Job* jobs, int trav) {
-    MCEV_TRAV_DISPATCH(k_shadow, grid_for(max_n, MCEV_TRAV_BLOCK, sms, MCEV_TRAV_BLOCKS_PER_SM), sc, fr, P, w, cur,
-                       err);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_shadow_extend(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int cur,
-                                 int64_t max_n, int32_t* err, int sms, cudaStream_t st, const Job* jobs, int trav) {
-    const int g = grid_for(max_n, MCEV_TRAV_BLOCK, sms, MCEV_TRAV_BLOCKS_PER_SM);
-    MCEV_TRAV_DISPATCH(k_shadow_extend, 2 * g, sc, fr, P, w, cur, g, err);
+cudaError_t launch_queue(const Wave& w, int cur, int depth, int64_t max_n, int sms, cudaStream_t st) {
+    k_queue<<<grid_for(max_n, Q_TILE, sms, 4), Q_BLOCK, 0, st>>>(w, cur, depth);
     return cudaGetLastError();
 }
 

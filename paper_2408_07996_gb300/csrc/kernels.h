@@ -67,15 +67,14 @@ cudaError_t launch_raygen(const DevFrame& fr, const DevParams& P, const Wave& w,
 // TLAS (frames with at most one run kernels without the TLAS loop).
 enum { TRAV_WIDE = 1, TRAV_TLAS = 2 };
 
-cudaError_t launch_extend(const DevScene& sc, const DevFrame& fr, float t_min, const Wave& w, int cur, int64_t max_n,
-                          int32_t* err, int sms, cudaStream_t st, const Job* jobs, int trav);
+// closest hits of bounce `depth` (ray queue ecur) and, with scur >= 0, the
+// shadow rays that shade(scur) left, in one launch
+cudaError_t launch_trace(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int ecur, int scur,
+                         int depth, int64_t max_n, int32_t* err, int sms, cudaStream_t st, const Job* jobs, int trav);
 cudaError_t launch_shade(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int cur,
-                         int64_t max_n, int sms, cudaStream_t st, const Job* jobs);
-cudaError_t launch_shadow(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int cur,
-                          int64_t max_n, int32_t* err, int sms, cudaStream_t st, const Job* jobs, int trav);
-// shadow rays of the bounce with queue `cur` and closest hits of queue 1 - cur, in one launch
-cudaError_t launch_shadow_extend(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int cur,
-                                 int64_t max_n, int32_t* err, int sms, cudaStream_t st, const Job* jobs, int trav);
+                         int depth, int64_t max_n, int sms, cudaStream_t st, const Job* jobs);
+// queues the rays that shade(cur, depth) left, tile by tile, by direction
+cudaError_t launch_queue(const Wave& w, int cur, int depth, int64_t max_n, int sms, cudaStream_t st);
 cudaError_t launch_stats(const Wave& w, const StatsArgs& A, const int32_t* queue, int64_t j0, int64_t n_pix,
                          int32_t* next_queue, int sms, cudaStream_t st, const Job* jobs, const RoundCtl* rc = nullptr);
 // device-resident round loop: start state (and, with iota, queue 0 = 0..Q0-1)

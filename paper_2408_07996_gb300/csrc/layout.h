@@ -26,16 +26,8 @@
 #define MCEV_HD
 #endif
 
-// Traversal stack per thread (TLAS + BLAS depth must fit): in shared memory
-// (32 entries, thread-interleaved) when MCEV_SMEM_STACK, else in local memory.
-#ifndef MCEV_SMEM_STACK
-#define MCEV_SMEM_STACK 0
-#endif
-#if MCEV_SMEM_STACK
-#define MCEV_STACK_HOST 32
-#else
+// Traversal stack per thread (TLAS + BLAS depth must fit), in local memory.
 #define MCEV_STACK_HOST 96
-#endif
 
 // Wide-BVH traversal stack per thread: node groups (one per wide level).
 #define MCEV_WSTACK_HOST 32
@@ -136,15 +128,17 @@ struct Wave {
     float* L;
     uint32_t* sig;
     uint32_t* pflags;         // pending flags of the last vertex (0xFFFFFFFF = none)
-    int2* pix_k;              // (queue entry, sample index); written for batched renders only
-    // ray queues (ping-pong) and hits, per queue slot
-    float4* ray_o[2];         // xyz origin, w = path slot (int bits)
-    float4* ray_d[2];         // xyz direction, w = depth (int bits)
-    float4* ray_s[2];         // path state carried with the ray: throughput, pdf of the sampled
-                              // direction, queue entry and sample index (int bits)
-    float4* hit;              // t, instance, leaf-order triangle, 0   (inst < 0: miss)
+    int2* pix_k;              // (queue entry, sample index)
+    float4* ray_o;            // xyz origin of the path's current ray (and of its shadow ray), w = throughput
+    float4* ray_d;            // xyz direction, w = pdf of the sampled direction
+    float2* hit;              // t, leaf-order triangle (int bits; -1: miss)
+    int32_t* hit_rec;         // instance record of the hit; written for frames of more than one record
+    uint16_t* key;            // what the vertex just shaded goes on with: direction cell of the next ray in the
+                              // low byte, of the shadow ray in the high byte (KEY_NONE: none)
+    // queues of path slots
+    int32_t* list[2];         // rays of this bounce and of the next (ping-pong)
+    int32_t* sh_list;         // shadow rays
     // shadow rays
-    float4* sh_o;             // xyz origin, w = path slot
     float4* sh_d;             // xyz direction, w = t_max
     float* sh_c;              // unoccluded contribution
     float* sh_g;              // adjoint: contribution / emitted radiance of the sampled light
@@ -160,6 +154,7 @@ struct Wave {
     //   [7]       pixels decided at spp_max
     //   [8]       caller pixel id outside [0, n_total) (allocation-free step)
     //   [15]      traversal stack overflow
+    //   [20]      cursor of the traversal: groups of 32 rays taken
     //   from [32] on, uint64 words: [0] nodes and [1] triangles of closest-hit
     //   traversal, [2] nodes and [3] triangles of shadow rays, [4] closest-hit
     //   rays, [5] shadow rays, [6] samples that entered decisions, [7] and
