@@ -113,9 +113,10 @@ typedef struct {
                            fail with MCEV_ERR_ARG */
     int32_t profile;    /* 1: time every kernel launch with CUDA events (mcev_stats.kernel_ms) */
     int32_t batch_window; /* after the first batch, a round may trace up to this many batches of
-                             spp_batch per undecided pixel at once (as many as fill the wavefront),
-                             merging and testing them in order; samples after a pixel's decision
-                             are unused.  1 = one batch per round; 0 = library default (16). */
+                             spp_batch per undecided pixel at once, merging and testing them in
+                             order; samples after a pixel's decision are unused (a round adds about
+                             a quarter of a pixel's samples, more when that would leave the GPU
+                             idle, never more than fill the wavefront).  1 = one batch per round; 0 = library default (16). */
     int32_t bvh_width;  /* node layout of the per-mesh BVHs: 2 (two children per node) or 8
                            (compressed 8-wide nodes with 8-bit child boxes); 0 = library default.
                            Changing it rebuilds the BVHs of an uploaded scene.  Results are the

@@ -1034,16 +1034,14 @@ mcev_status run_rounds(mcev_ctx* ctx, const Frame& fr, StatsArgs A, int64_t* pat
     const int64_t window_max = ctx->params.batch_window > 0 ? ctx->params.batch_window : 16;
     while (Q > 0) {
         // first round: spp_min samples; later rounds: a window of m batches
-        // of spp_batch, as many as fill the wavefront (speculative samples of
-        // pixels that decide inside the window are traced but not used)
+        // of spp_batch (round_window; speculative samples of pixels that
+        // decide inside the window are traced but not used)
         int32_t spp_r, sub;
         if (n_done == 0) {
             spp_r = sub = std::min(A.spp_min, A.spp_max);
         } else {
             sub = A.spp_batch;
-            const int64_t left = (A.spp_max - n_done + sub - 1) / sub;
-            int64_t m = std::max<int64_t>(1, ctx->wave.cap / std::max<int64_t>(1, Q * sub));
-            m = std::min(std::min(m, left), window_max);
+            const int64_t m = round_window(ctx->wave.cap, Q, sub, n_done, A.spp_max, window_max);
             spp_r = (int32_t)std::min<int64_t>(m * sub, A.spp_max - n_done);
         }
         NvtxRange round_range("mcev round");

@@ -879,8 +879,8 @@ static cudaError_t launch_stats_checked(const Wave& w, const StatsArgs& A, const
 // one wavefront chunk (raygen, bounces, statistics) followed by
 // k_round_next, which moves to the next chunk of the round or, at the end
 // of a round, reads the number of re-queued pixels and sizes the next round
-// (first round spp_min samples, then windows of spp_batch batches that fill
-// the wavefront), and clears the condition when no pixel is left.  The loop
+// (first round spp_min samples, then windows of spp_batch batches:
+// round_window), and clears the condition when no pixel is left.  The loop
 // is bounded: after plan.max_iters chunks, or plan.timeout_ns of wall clock
 // (%globaltimer), it stops with RC_TIMEOUT, which the host reports as
 // MCEV_ERR_TIMEOUT.
@@ -944,9 +944,7 @@ __global__ void k_round_next(RoundCtl* rc, Wave w, RoundPlan plan, cudaGraphCond
             go = 0;
         } else {
             const int64_t sub = plan.spp_batch;
-            const int64_t left = (plan.spp_max - rc->n_done + sub - 1) / sub;
-            int64_t m = max((int64_t)1, plan.cap / max((int64_t)1, (int64_t)q * sub));
-            m = min(min(m, left), (int64_t)plan.window_max);
+            const int64_t m = round_window(plan.cap, q, sub, rc->n_done, plan.spp_max, plan.window_max);
             rc->sub = (int32_t)sub;
             rc->spp_r = (int32_t)min(m * sub, (int64_t)plan.spp_max - rc->n_done);
             round_first_chunk(rc, plan);

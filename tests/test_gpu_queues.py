@@ -36,3 +36,23 @@ def test_samples_do_not_depend_on_the_call(moving, width):
             assert torch.equal(sig[:, k], whole[k][1][:n, 0]), (n, k)
     assert whole[0][0].max() > 0
     r.close()
+
+
+@pytest.mark.parametrize("spp_max", [31, 96, 257])
+def test_round_window_only_changes_what_is_traced(spp_max):
+    """Any window of batches per round gives the frame of one batch per round."""
+    w = sg.workload("cornell64")
+    out = {}
+    for window in (1, 0, 64):
+        r = Renderer(w.width, w.height)
+        r.upload(w.scene)
+        r.configure(w)
+        r.set_params(batch_window=window)
+        o = r.render_events(0.0, 1.0, w.C, w.alpha, 8, spp_max)
+        out[window] = (o["events"].clone(), o["spp"].clone(), o["mean"].clone(), o["stats"])
+        r.close()
+    for window in (0, 64):
+        for a, b in zip(out[1][:3], out[window][:3]):
+            assert torch.equal(a, b)
+        assert out[window][3]["samples_used"] == out[1][3]["samples_used"]
+        assert out[window][3]["paths"] >= out[1][3]["paths"]
