@@ -718,9 +718,9 @@ mcev_status check_spp_fits(mcev_ctx* ctx, int64_t spp) {
 mcev_status ensure_wave(mcev_ctx* ctx) {
     const int64_t cap = wave_cap(ctx);
     if (ctx->d_wave.ptr && ctx->wave.cap == cap) return MCEV_OK;
-    // per path slot: ray_o, ray_d, sh_d; hit, pix_k; hit_rec, L, sig, pflags, sh_c, sh_g, sh_m, Ltot, delta; key;
+    // per path slot: ray_o, ray_d, sh_d; hit, pix_k; hit_rec, L, sig, pflags, sh_c, sh_g, sh_m, Ltot, delta;
     // queues: list (x2), sh_list
-    const size_t per = 3 * 16 + 2 * 8 + 9 * 4 + 2 + 3 * 4;
+    const size_t per = 3 * 16 + 2 * 8 + 9 * 4 + 3 * 4;
     ST(dev_alloc(ctx, ctx->d_wave, (size_t)cap * per + 64 * 256));
     char* p = (char*)ctx->d_wave.ptr;
     auto take = [&](size_t bytes) {
@@ -739,7 +739,6 @@ mcev_status ensure_wave(mcev_ctx* ctx) {
     w.L = (float*)take(4 * cap);
     w.sig = (uint32_t*)take(4 * cap);
     w.pflags = (uint32_t*)take(4 * cap);
-    w.key = (uint16_t*)take(2 * cap);
     w.list[0] = (int32_t*)take(4 * cap);
     w.list[1] = (int32_t*)take(4 * cap);
     w.sh_list = (int32_t*)take(4 * cap);
@@ -848,9 +847,9 @@ mcev_status trace_chunk(mcev_ctx* ctx, const Frame& fr, const DevParams& P, cons
     LAUNCH(MCEV_K_EXTEND, launch_trace(ctx->dsc, fr.dev, P, w, cur, -1, 0, n_paths, err, ctx->sms, ctx->stream, jobs,
                                        trav));
     for (int depth = 0; depth <= depth_max; ++depth) {
-        LAUNCH(MCEV_K_SHADE, launch_shade(ctx->dsc, fr.dev, P, w, cur, depth, n_paths, ctx->sms, ctx->stream, jobs));
+        LAUNCH(MCEV_K_SHADE, launch_shade(ctx->dsc, fr.dev, P, w, cur, depth, depth == depth_max, n_paths, ctx->sms,
+                                          ctx->stream, jobs));
         if (depth < depth_max) {
-            LAUNCH(MCEV_K_SHADE, launch_queue(w, cur, depth, n_paths, ctx->sms, ctx->stream));
             // this bounce's shadow rays and the next bounce's closest hits in one launch
             LAUNCH(MCEV_K_EXTEND, launch_trace(ctx->dsc, fr.dev, P, w, cur ^ 1, nee ? cur : -1, depth + 1, n_paths,
                                                err, ctx->sms, ctx->stream, jobs, trav));

@@ -1,10 +1,10 @@
 // kernels.cu -- wavefront path tracer and statistical event detector.
 //
 // One chunk of paths goes through
-//   raygen -> extend -> [shade(+NEE) -> queue -> shadow + extend] x max_depth -> shade -> stats
+//   raygen -> extend -> [shade(+NEE) -> shadow + extend] x max_depth -> shade -> stats
 // Every path keeps one slot of the wavefront for its ray and state; extend,
 // shade and shadow walk device-side queues of slots (sizes in device
-// counters, no host round trip) that `queue` fills tile by tile in direction
+// counters, no host round trip) that shade fills tile by tile in direction
 // order.  `stats` fuses, per queued pixel, the log-luminance batch statistics
 // (Sec. 3.1, Eq. 3-4), the Chan merge into the running statistics, the t-test
 // of Eq. 7 (Sec. 3.2), the re-queue of undecided pixels (Sec. 3.3; one atomic
@@ -165,275 +165,259 @@ __device__ __forceinline__ void add_work(const Wave& w, int3 closest, int3 shado
 }
 
 // ------------------------------------------------------------------ shade + NEE + BSDF sampling
-// shade is latency bound on per-path gathers: 64 registers (8 blocks/SM)
-// measured 15% faster than the unconstrained 80-register build
-#ifndef MCEV_SHADE_MINB
-#define MCEV_SHADE_MINB 8
-#endif
-#if MCEV_SHADE_MINB > 0
-#define MCEV_SHADE_BOUNDS __launch_bounds__(128, MCEV_SHADE_MINB)
-#else
-#define MCEV_SHADE_BOUNDS __launch_bounds__(128)
-#endif
+// Shades a bounce's hits and queues the rays it leaves.  A block takes tiles of
+// up to Q_TILE consecutive entries of the bounce's queue: it shades them, one
+// path per thread and step, and then appends the paths that go on and the ones
+// with a shadow ray to their queues, grouped by direction cell (a counting
+// sort in shared memory) with one atomic per tile and queue.  Consecutive
+// entries stay paths of neighbouring pixels (the samples of a pixel are
+// consecutive path slots, a tile is 8 pixels at 512 samples), so a traversal
+// warp holds rays that start at nearly the same point and leave it in nearly
+// the same direction.
+//
+// What bounds it: the latency of the per-path gathers (64 registers, 1024
+// threads per SM; 15 % faster than an unconstrained 80-register build).
+// Against appending rays in the order shade's warps finish, which mixes the
+// pixels of a whole wave of blocks, the 1280x720 terrain frame with the converged
+// traversal loop takes: 687 ms of traversal with one cell per tile (pixel
+// order kept, no sort), 609 ms with the 24 cells, 624 and 614 ms with an octahedral
+// grid of 4 x 4 and 8 x 8 cells, 640 ms with the octants alone; shading and
+// queues 139, 139, 143, 148 and 136 ms (more cells scatter shade's reads).
+// Tiles of 2048 and 8192 entries within 1 % of 4096.  Queues filled by a kernel of
+// their own cost 9 ms more (139 -> 130 ms, 4 bytes per path and a launch per
+// bounce); blocks of 128 / 256 / 512 threads 138 / 130 / 370 ms.
+static constexpr int Q_BLOCK = 256, Q_TILE = 4096, Q_ITEMS = Q_TILE / Q_BLOCK;
+static constexpr int Q_RESIDENT = 1024 / Q_BLOCK;   // blocks per SM
+
 template <bool kBatch>
-__global__ void MCEV_SHADE_BOUNDS k_shade(DevScene sc, DevFrame fr, DevParams P, Wave w, int cur, int depth,
-                                          const Job* __restrict__ jobs) {
-    const int32_t n = *(volatile int32_t*)(w.counters + cur);
-    const int32_t* list = depth > 0 ? w.list[cur] : nullptr;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int p = list ? __ldg(list + i) : i;
-        const float4 ro = w.ray_o[p];
-        const float4 rd = w.ray_d[p];
-        const int2 rs = w.pix_k[p];
-        const int job = kBatch ? (int)((uint32_t)rs.x >> 24) : 0;
-        const DevScene& S = kBatch ? jobs[job].sc : sc;
-        const DevFrame& F = kBatch ? jobs[job].fr : fr;
-        const DevParams& Q = kBatch ? jobs[job].P : P;
-        const float2 hv = w.hit[p];
-        const int tri = __float_as_int(hv.y);
-        float beta = ro.w;
-        // radiance this vertex adds to the path (emission on a hit, the
-        // environment on a miss); the path's total is updated only when
-        // something is added
-        float Ladd = 0.0f;
-        const float pdf_prev = rd.w;
-        float pdf_next = 0.0f;
-        uint32_t sig = 0, pflags = NO_FLAGS;
-        if (Q.want_sig) {
-            sig = w.sig[p];
-            const uint32_t pf = w.pflags[p];
-            if (pf != NO_FLAGS) sig = fnv(sig, pf);
-        }
-        const f3 d = xyz(rd);
-        bool cont = false, shadow = false;
-        f3 P0 = mk3(0, 0, 0), wi_next = mk3(0, 0, 0), sh_dir = mk3(0, 0, 0);
-        float sh_tmax = 0.0f, sh_c = 0.0f, sh_g = 0.0f;
-        int sh_m = -1;
-        if (tri < 0) {
-            // miss: environment radiance (Sec. 3.1 samples the light reaching the pixel)
-            if (Q.want_sig) sig = fnv(sig, 0xFFFFFFFFu);
-            if (S.has_env) {
-                int row, col;
-                float st;
-                env_texel(S, d, row, col, st);
-                if (Q.want_sig) sig = fnv(sig, (uint32_t)(row * S.env_w + col));
-                const float Le = __ldg(S.env + (int64_t)row * S.env_w + col);
-                float wgt = 1.0f;
-                if (depth > 0 && Q.nee) wgt = Q.mis ? power_heuristic(pdf_prev, F.p_env * texel_pdf(S, row, col, st)) : 0.0f;
-                Ladd = beta * wgt * Le;
-            } else if (Q.want_sig) {
-                sig = fnv(sig, 0xFFFFFFFEu);
-            }
-        } else {
-            const int rec = F.n_inst > 1 ? w.hit_rec[p] : 0;
-            // the shading record (edge cross product, material) serves most
-            // hits; the vertices are read only for textured albedo, emitter
-            // MIS weights and the decision signature
-            const float4 tsh = __ldg(S.tshade + tri);
-            const float4* tp = S.tris + 3 * tri;
-            const float4* ip = F.inst + 7 * rec;
-            const float4 i0 = __ldg(ip + 3), i1 = __ldg(ip + 4), i2 = __ldg(ip + 5);
-            const int ovr = __float_as_int(__ldg(ip + 6).y);
-            if (Q.want_sig) {
-                sig = fnv(sig, (uint32_t)hit_inst(F, rec, __ldg(tp + 2).w));
-                sig = fnv(sig, (uint32_t)__float_as_int(__ldg(tp).w));
-            }
-            const float t = hv.x;
-            P0 = xyz(ro) + d * t;
-            const f3 ng = norm3(xf_normal(i0, i1, i2, xyz(tsh)));
-            const f3 wo = d * -1.0f;
-            const int mat = ovr >= 0 ? ovr : __float_as_int(tsh.w);
-            const float4 mv = __ldg(S.mats + mat);
-            const int tword = __float_as_int(mv.x);
-            const int type = tword & 0xFF;
-            float alb = mv.y;
-            const float rough = mv.z;
-            // the override applies to the scene's emitters only (NEE samples that fixed set)
-            const float emit = (S.emit && mv.w > 0.0f) ? __ldg(S.emit + mat) : mv.w;
-            int texel = -1;
-            if ((tword & MAT_TEXTURED) && S.tex && S.tri_uv) {
-                // albedo = luminance of the nearest texel at the hit's texture coordinates
-                const float4 q0 = __ldg(tp), q1 = __ldg(tp + 1), q2 = __ldg(tp + 2);
-                float b1, b2;
-                barycentric(xf_point(i0, i1, i2, P0), xyz(q0), xyz(q1), xyz(q2), b1, b2);
-                const float b0 = 1.0f - b1 - b2;
-                const float2 t0 = __ldg(S.tri_uv + 3 * tri), t1 = __ldg(S.tri_uv + 3 * tri + 1),
-                             t2 = __ldg(S.tri_uv + 3 * tri + 2);
-                texel = texel_of(S, b0 * t0.x + b1 * t1.x + b2 * t2.x, b0 * t0.y + b1 * t1.y + b2 * t2.y);
-                const float* rgb = S.tex + 3 * (int64_t)texel;
-                alb = MCEV_Y_R * __ldg(rgb) + MCEV_Y_G * __ldg(rgb + 1) + MCEV_Y_B * __ldg(rgb + 2);
-                if (Q.want_sig) sig = fnv(sig, (uint32_t)texel);
-            }
-            const float dlt = Q.adjoint ? w.delta[p] : 0.0f;
-            uint32_t flags = 0;
-            const float cos_o = dot3(ng, wo);
-            if (emit > 0.0f && cos_o > 0.0f) {
-                flags |= 1u;
-                float wgt = 1.0f;
-                if (depth > 0 && Q.nee) {
-                    if (!Q.mis) {
-                        wgt = 0.0f;
-                    } else {
-                        const float4 q0 = __ldg(tp), q1 = __ldg(tp + 1), q2 = __ldg(tp + 2);
-                        const float4 m0 = __ldg(ip), m1 = __ldg(ip + 1), m2 = __ldg(ip + 2);
-                        const f3 e1 = xyz(q1) - xyz(q0), e2 = xyz(q2) - xyz(q0);
-                        const f3 we1 = xf_vec(m0, m1, m2, e1), we2 = xf_vec(m0, m1, m2, e2);
-                        const f3 wc = cross3(we1, we2);
-                        const float area = 0.5f * sqrtf(dot3(wc, wc));
-                        const float pl = F.p_area / ((float)F.n_lights * area) * t * t / cos_o;
-                        wgt = power_heuristic(pdf_prev, pl);
-                    }
-                }
-                Ladd = beta * wgt * emit;
-                if (Q.adjoint && Q.grad_emit) atomicAdd(Q.grad_emit + mat, (double)(dlt * beta * wgt));
-            }
-            if (depth < Q.max_depth && alb > 0.0f) {
-                // adjoint: every contribution after this vertex carries one factor of its albedo
-                if (Q.adjoint && texel >= 0 && Q.grad_tex && dlt != 0.0f) {
-                    const float g = dlt * (w.Ltot[p] - (w.L[p] + Ladd)) / alb;
-                    float* gt = Q.grad_tex + 3 * (int64_t)texel;
-                    atomicAdd(gt, g * MCEV_Y_R);
-                    atomicAdd(gt + 1, g * MCEV_Y_G);
-                    atomicAdd(gt + 2, g * MCEV_Y_B);
-                }
-                const f3 nn = cos_o < 0.0f ? ng * -1.0f : ng;
-                f3 tb, bt;
-                onb(nn, tb, bt);
-                const f3 wol = mk3(dot3(wo, tb), dot3(wo, bt), dot3(wo, nn));
-                const uint32_t ent = (uint32_t)rs.x;
-                const uint2 pk = make_uint2(kBatch ? (ent & 0xFFFFFFu) : ent, (uint32_t)rs.y);
-                // next-event estimation
-                if (Q.nee && (S.env_ok || F.n_lights > 0)) {
-                    const uint4 x = philox4x32_10(make_uint4(pk.x, pk.y, (uint32_t)(depth + 1), 0u), F.key0, F.key1);
-                    const bool use_env = S.env_ok && (F.n_lights == 0 || u01(x.x) < 0.5f);
-                    f3 wi = mk3(0, 0, 0);
-                    float pl = 0.0f, Le = 0.0f, tmax = __int_as_float(0x7f800000);
-                    int lmat = -1;
-                    if (use_env) {
-                        float pdf;
-                        wi = env_sample(S, u01(x.z), u01(x.w), pdf, Le);
-                        pl = F.p_env * pdf;
-                    } else {
-                        const uint64_t mm = (uint64_t)(x.y >> 8);
-                        const int li = (int)((mm * (uint64_t)F.n_lights) >> 24);
-                        const float4* lp = F.lights + 4 * li;
-                        const float4 a0 = __ldg(lp), a1 = __ldg(lp + 1), a2 = __ldg(lp + 2), an = __ldg(lp + 3);
-                        const float su = sqrtf(u01(x.z));
-                        const float b0 = 1.0f - su, b1 = u01(x.w) * su, b2 = 1.0f - b0 - b1;
-                        const f3 Ql = xyz(a0) * b0 + xyz(a1) * b1 + xyz(a2) * b2;
-                        const f3 dv = Ql - P0;
-                        const float dist = sqrtf(dot3(dv, dv));
-                        wi = dv * (1.0f / dist);
-                        const float cl = -dot3(xyz(an), wi);
-                        if (cl > 0.0f) {
-                            pl = F.p_area / ((float)F.n_lights * a1.w) * dist * dist / cl;
-                            lmat = __float_as_int(a2.w);
-                            Le = S.emit ? __ldg(S.emit + lmat) : a0.w;
-                        }
-                        tmax = dist - Q.t_min;
-                    }
-                    if (pl > 0.0f && Le > 0.0f) {
-                        const f3 wil = mk3(dot3(wi, tb), dot3(wi, bt), dot3(wi, nn));
-                        float pb;
-                        const float f = bsdf_eval(type, alb, rough, wol, wil, &pb);
-                        if (f > 0.0f && wil.z > 0.0f) {
-                            flags |= 2u;
-                            const float wgt = Q.mis ? power_heuristic(pl, pb) : 1.0f;
-                            sh_c = beta * f * wil.z * Le * wgt / pl;
-                            sh_g = beta * f * wil.z * wgt / pl;
-                            sh_m = lmat;
-                            sh_dir = wi;
-                            sh_tmax = tmax;
-                            shadow = true;
-                        }
-                    }
-                }
-                // BSDF sampling of the continuation
-                const uint4 y = philox4x32_10(make_uint4(pk.x, pk.y, (uint32_t)(depth + 1), 1u), F.key0, F.key1);
-                const f3 wil = bsdf_sample(type, rough, wol, u01(y.x), u01(y.y));
-                float pb;
-                const float f = bsdf_eval(type, alb, rough, wol, wil, &pb);
-                if (f > 0.0f && pb > 0.0f && wil.z > 0.0f) {
-                    flags |= 8u;
-                    beta *= f * wil.z / pb;
-                    pdf_next = pb;
-                    wi_next = norm3(tb * wil.x + bt * wil.y + nn * wil.z);
-                    cont = true;
-                }
-            }
-            pflags = flags;
-        }
-        if (Ladd != 0.0f) w.L[p] += Ladd;
-        if (Q.want_sig) {
-            w.sig[p] = sig;
-            w.pflags[p] = pflags;
-        }
-        if (shadow || cont) w.ray_o[p] = make_float4(P0.x, P0.y, P0.z, beta);
-        if (shadow) {
-            w.sh_d[p] = make_float4(sh_dir.x, sh_dir.y, sh_dir.z, sh_tmax);
-            w.sh_c[p] = sh_c;
-            if (Q.adjoint) {
-                w.sh_g[p] = sh_g;
-                w.sh_m[p] = sh_m;
-            }
-        }
-        if (cont) w.ray_d[p] = make_float4(wi_next.x, wi_next.y, wi_next.z, pdf_next);
-        w.key[p] = (uint16_t)((cont ? dir_cell(wi_next) : KEY_NONE) | (shadow ? dir_cell(sh_dir) : KEY_NONE) << 8);
+__device__ __forceinline__ uint32_t shade_path(const DevScene& sc, const DevFrame& fr, const DevParams& P,
+                                               const Wave& w, int p, int depth, const Job* __restrict__ jobs) {
+    const float4 ro = w.ray_o[p];
+    const float4 rd = w.ray_d[p];
+    const int2 rs = w.pix_k[p];
+    const int job = kBatch ? (int)((uint32_t)rs.x >> 24) : 0;
+    const DevScene& S = kBatch ? jobs[job].sc : sc;
+    const DevFrame& F = kBatch ? jobs[job].fr : fr;
+    const DevParams& Q = kBatch ? jobs[job].P : P;
+    const float2 hv = w.hit[p];
+    const int tri = __float_as_int(hv.y);
+    float beta = ro.w;
+    // radiance this vertex adds to the path (emission on a hit, the
+    // environment on a miss); the path's total is updated only when
+    // something is added
+    float Ladd = 0.0f;
+    const float pdf_prev = rd.w;
+    float pdf_next = 0.0f;
+    uint32_t sig = 0, pflags = NO_FLAGS;
+    if (Q.want_sig) {
+        sig = w.sig[p];
+        const uint32_t pf = w.pflags[p];
+        if (pf != NO_FLAGS) sig = fnv(sig, pf);
     }
+    const f3 d = xyz(rd);
+    bool cont = false, shadow = false;
+    f3 P0 = mk3(0, 0, 0), wi_next = mk3(0, 0, 0), sh_dir = mk3(0, 0, 0);
+    float sh_tmax = 0.0f, sh_c = 0.0f, sh_g = 0.0f;
+    int sh_m = -1;
+    if (tri < 0) {
+        // miss: environment radiance (Sec. 3.1 samples the light reaching the pixel)
+        if (Q.want_sig) sig = fnv(sig, 0xFFFFFFFFu);
+        if (S.has_env) {
+            int row, col;
+            float st;
+            env_texel(S, d, row, col, st);
+            if (Q.want_sig) sig = fnv(sig, (uint32_t)(row * S.env_w + col));
+            const float Le = __ldg(S.env + (int64_t)row * S.env_w + col);
+            float wgt = 1.0f;
+            if (depth > 0 && Q.nee) wgt = Q.mis ? power_heuristic(pdf_prev, F.p_env * texel_pdf(S, row, col, st)) : 0.0f;
+            Ladd = beta * wgt * Le;
+        } else if (Q.want_sig) {
+            sig = fnv(sig, 0xFFFFFFFEu);
+        }
+    } else {
+        const int rec = F.n_inst > 1 ? w.hit_rec[p] : 0;
+        // the shading record (edge cross product, material) serves most
+        // hits; the vertices are read only for textured albedo, emitter
+        // MIS weights and the decision signature
+        const float4 tsh = __ldg(S.tshade + tri);
+        const float4* tp = S.tris + 3 * tri;
+        const float4* ip = F.inst + 7 * rec;
+        const float4 i0 = __ldg(ip + 3), i1 = __ldg(ip + 4), i2 = __ldg(ip + 5);
+        const int ovr = __float_as_int(__ldg(ip + 6).y);
+        if (Q.want_sig) {
+            sig = fnv(sig, (uint32_t)hit_inst(F, rec, __ldg(tp + 2).w));
+            sig = fnv(sig, (uint32_t)__float_as_int(__ldg(tp).w));
+        }
+        const float t = hv.x;
+        P0 = xyz(ro) + d * t;
+        const f3 ng = norm3(xf_normal(i0, i1, i2, xyz(tsh)));
+        const f3 wo = d * -1.0f;
+        const int mat = ovr >= 0 ? ovr : __float_as_int(tsh.w);
+        const float4 mv = __ldg(S.mats + mat);
+        const int tword = __float_as_int(mv.x);
+        const int type = tword & 0xFF;
+        float alb = mv.y;
+        const float rough = mv.z;
+        // the override applies to the scene's emitters only (NEE samples that fixed set)
+        const float emit = (S.emit && mv.w > 0.0f) ? __ldg(S.emit + mat) : mv.w;
+        int texel = -1;
+        if ((tword & MAT_TEXTURED) && S.tex && S.tri_uv) {
+            // albedo = luminance of the nearest texel at the hit's texture coordinates
+            const float4 q0 = __ldg(tp), q1 = __ldg(tp + 1), q2 = __ldg(tp + 2);
+            float b1, b2;
+            barycentric(xf_point(i0, i1, i2, P0), xyz(q0), xyz(q1), xyz(q2), b1, b2);
+            const float b0 = 1.0f - b1 - b2;
+            const float2 t0 = __ldg(S.tri_uv + 3 * tri), t1 = __ldg(S.tri_uv + 3 * tri + 1),
+                         t2 = __ldg(S.tri_uv + 3 * tri + 2);
+            texel = texel_of(S, b0 * t0.x + b1 * t1.x + b2 * t2.x, b0 * t0.y + b1 * t1.y + b2 * t2.y);
+            const float* rgb = S.tex + 3 * (int64_t)texel;
+            alb = MCEV_Y_R * __ldg(rgb) + MCEV_Y_G * __ldg(rgb + 1) + MCEV_Y_B * __ldg(rgb + 2);
+            if (Q.want_sig) sig = fnv(sig, (uint32_t)texel);
+        }
+        const float dlt = Q.adjoint ? w.delta[p] : 0.0f;
+        uint32_t flags = 0;
+        const float cos_o = dot3(ng, wo);
+        if (emit > 0.0f && cos_o > 0.0f) {
+            flags |= 1u;
+            float wgt = 1.0f;
+            if (depth > 0 && Q.nee) {
+                if (!Q.mis) {
+                    wgt = 0.0f;
+                } else {
+                    const float4 q0 = __ldg(tp), q1 = __ldg(tp + 1), q2 = __ldg(tp + 2);
+                    const float4 m0 = __ldg(ip), m1 = __ldg(ip + 1), m2 = __ldg(ip + 2);
+                    const f3 e1 = xyz(q1) - xyz(q0), e2 = xyz(q2) - xyz(q0);
+                    const f3 we1 = xf_vec(m0, m1, m2, e1), we2 = xf_vec(m0, m1, m2, e2);
+                    const f3 wc = cross3(we1, we2);
+                    const float area = 0.5f * sqrtf(dot3(wc, wc));
+                    const float pl = F.p_area / ((float)F.n_lights * area) * t * t / cos_o;
+                    wgt = power_heuristic(pdf_prev, pl);
+                }
+            }
+            Ladd = beta * wgt * emit;
+            if (Q.adjoint && Q.grad_emit) atomicAdd(Q.grad_emit + mat, (double)(dlt * beta * wgt));
+        }
+        if (depth < Q.max_depth && alb > 0.0f) {
+            // adjoint: every contribution after this vertex carries one factor of its albedo
+            if (Q.adjoint && texel >= 0 && Q.grad_tex && dlt != 0.0f) {
+                const float g = dlt * (w.Ltot[p] - (w.L[p] + Ladd)) / alb;
+                float* gt = Q.grad_tex + 3 * (int64_t)texel;
+                atomicAdd(gt, g * MCEV_Y_R);
+                atomicAdd(gt + 1, g * MCEV_Y_G);
+                atomicAdd(gt + 2, g * MCEV_Y_B);
+            }
+            const f3 nn = cos_o < 0.0f ? ng * -1.0f : ng;
+            f3 tb, bt;
+            onb(nn, tb, bt);
+            const f3 wol = mk3(dot3(wo, tb), dot3(wo, bt), dot3(wo, nn));
+            const uint32_t ent = (uint32_t)rs.x;
+            const uint2 pk = make_uint2(kBatch ? (ent & 0xFFFFFFu) : ent, (uint32_t)rs.y);
+            // next-event estimation
+            if (Q.nee && (S.env_ok || F.n_lights > 0)) {
+                const uint4 x = philox4x32_10(make_uint4(pk.x, pk.y, (uint32_t)(depth + 1), 0u), F.key0, F.key1);
+                const bool use_env = S.env_ok && (F.n_lights == 0 || u01(x.x) < 0.5f);
+                f3 wi = mk3(0, 0, 0);
+                float pl = 0.0f, Le = 0.0f, tmax = __int_as_float(0x7f800000);
+                int lmat = -1;
+                if (use_env) {
+                    float pdf;
+                    wi = env_sample(S, u01(x.z), u01(x.w), pdf, Le);
+                    pl = F.p_env * pdf;
+                } else {
+                    const uint64_t mm = (uint64_t)(x.y >> 8);
+                    const int li = (int)((mm * (uint64_t)F.n_lights) >> 24);
+                    const float4* lp = F.lights + 4 * li;
+                    const float4 a0 = __ldg(lp), a1 = __ldg(lp + 1), a2 = __ldg(lp + 2), an = __ldg(lp + 3);
+                    const float su = sqrtf(u01(x.z));
+                    const float b0 = 1.0f - su, b1 = u01(x.w) * su, b2 = 1.0f - b0 - b1;
+                    const f3 Ql = xyz(a0) * b0 + xyz(a1) * b1 + xyz(a2) * b2;
+                    const f3 dv = Ql - P0;
+                    const float dist = sqrtf(dot3(dv, dv));
+                    wi = dv * (1.0f / dist);
+                    const float cl = -dot3(xyz(an), wi);
+                    if (cl > 0.0f) {
+                        pl = F.p_area / ((float)F.n_lights * a1.w) * dist * dist / cl;
+                        lmat = __float_as_int(a2.w);
+                        Le = S.emit ? __ldg(S.emit + lmat) : a0.w;
+                    }
+                    tmax = dist - Q.t_min;
+                }
+                if (pl > 0.0f && Le > 0.0f) {
+                    const f3 wil = mk3(dot3(wi, tb), dot3(wi, bt), dot3(wi, nn));
+                    float pb;
+                    const float f = bsdf_eval(type, alb, rough, wol, wil, &pb);
+                    if (f > 0.0f && wil.z > 0.0f) {
+                        flags |= 2u;
+                        const float wgt = Q.mis ? power_heuristic(pl, pb) : 1.0f;
+                        sh_c = beta * f * wil.z * Le * wgt / pl;
+                        sh_g = beta * f * wil.z * wgt / pl;
+                        sh_m = lmat;
+                        sh_dir = wi;
+                        sh_tmax = tmax;
+                        shadow = true;
+                    }
+                }
+            }
+            // BSDF sampling of the continuation
+            const uint4 y = philox4x32_10(make_uint4(pk.x, pk.y, (uint32_t)(depth + 1), 1u), F.key0, F.key1);
+            const f3 wil = bsdf_sample(type, rough, wol, u01(y.x), u01(y.y));
+            float pb;
+            const float f = bsdf_eval(type, alb, rough, wol, wil, &pb);
+            if (f > 0.0f && pb > 0.0f && wil.z > 0.0f) {
+                flags |= 8u;
+                beta *= f * wil.z / pb;
+                pdf_next = pb;
+                wi_next = norm3(tb * wil.x + bt * wil.y + nn * wil.z);
+                cont = true;
+            }
+        }
+        pflags = flags;
+    }
+    if (Ladd != 0.0f) w.L[p] += Ladd;
+    if (Q.want_sig) {
+        w.sig[p] = sig;
+        w.pflags[p] = pflags;
+    }
+    if (shadow || cont) w.ray_o[p] = make_float4(P0.x, P0.y, P0.z, beta);
+    if (shadow) {
+        w.sh_d[p] = make_float4(sh_dir.x, sh_dir.y, sh_dir.z, sh_tmax);
+        w.sh_c[p] = sh_c;
+        if (Q.adjoint) {
+            w.sh_g[p] = sh_g;
+            w.sh_m[p] = sh_m;
+        }
+    }
+    if (cont) w.ray_d[p] = make_float4(wi_next.x, wi_next.y, wi_next.z, pdf_next);
+    return (cont ? dir_cell(wi_next) : KEY_NONE) | (shadow ? dir_cell(sh_dir) : KEY_NONE) << 8;
 }
 
-// ------------------------------------------------------------------ ray queues
-// Queues the rays that shade left: per tile of Q_TILE consecutive entries of
-// the bounce's queue, the paths that go on and the ones with a shadow ray,
-// each grouped by direction cell (a counting sort in shared memory) and
-// appended with one atomic per tile.  Consecutive entries stay paths of
-// neighbouring pixels (the samples of a pixel are consecutive path slots, a
-// tile is 8 pixels at 512 samples), so a traversal warp holds rays that
-// start at nearly the same point and leave it in nearly the same direction.
-// What bounds it: the shared atomics of the ranks; it reads 8 B and writes 8 B
-// per ray.  Measured on the 1280x720 terrain frame against appending rays in
-// the order shade's warps finish (which mixes the pixels of a whole wave of
-// blocks): with the converged traversal loop: 687 ms with one cell per tile
-// (pixel order kept, no sort), 609 ms with the 24 cells, 624 and 614 ms with an
-// octahedral grid of 4 x 4 and 8 x 8 cells, 640 ms with the octants alone; queues
-// and shading 139, 139, 143, 148 and 136 ms (more cells scatter shade's reads).
-// Tiles of 2048 and 8192 entries within 1 % of 4096.
-static constexpr int Q_TILE = 4096, Q_BLOCK = 512, Q_ITEMS = Q_TILE / Q_BLOCK;
-
-__global__ void __launch_bounds__(Q_BLOCK) k_queue(Wave w, int cur, int depth) {
+template <bool kBatch>
+__global__ void __launch_bounds__(Q_BLOCK, Q_RESIDENT)
+    k_shade(DevScene sc, DevFrame fr, DevParams P, Wave w, int cur, int depth, int last, int resident,
+            const Job* __restrict__ jobs) {
+    __shared__ uint16_t keys[Q_TILE];
     __shared__ int cnt[2][KEY_CELLS];   // next rays, shadow rays
-    __shared__ int qbase[2];
     const int32_t n = *(volatile int32_t*)(w.counters + cur);
     const int32_t* list = depth > 0 ? w.list[cur] : nullptr;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (blockIdx.x == 0 && tid == 0) w.counters[20] = 0;   // the next traversal's cursor
-    // a small queue is cut into smaller tiles, so that every block has one
-    const int step = gridDim.x * Q_BLOCK;
+    // a small queue is cut into smaller tiles, so that every resident block has one
+    const int step = resident * Q_BLOCK;
     const int items = max(1, min(Q_ITEMS, (n + step - 1) / step));
-    for (int64_t t0 = (int64_t)blockIdx.x * items * Q_BLOCK; t0 < n; t0 += (int64_t)step * items) {
+    for (int64_t t0 = (int64_t)blockIdx.x * items * Q_BLOCK; t0 < n; t0 += (int64_t)gridDim.x * items * Q_BLOCK) {
         if (tid < 2 * KEY_CELLS) (&cnt[0][0])[tid] = 0;
         __syncthreads();
-        int p[Q_ITEMS];
-        uint32_t key[Q_ITEMS], rank[Q_ITEMS];
-#pragma unroll
-        for (int k = 0; k < Q_ITEMS; ++k) {
+        for (int k = 0; k < items; ++k) {
             const int64_t i = t0 + k * Q_BLOCK + tid;
-            key[k] = KEY_NONE | (KEY_NONE << 8);
-            p[k] = 0;
-            if (k < items && i < n) {
-                p[k] = list ? __ldg(list + i) : (int)i;
-                key[k] = w.key[p[k]];
-            }
+            uint32_t key = KEY_NONE | (KEY_NONE << 8);
+            if (i < n) key = shade_path<kBatch>(sc, fr, P, w, list ? __ldg(list + i) : (int)i, depth, jobs);
+            keys[k * Q_BLOCK + tid] = (uint16_t)key;
+            if ((key & 0xFFu) != KEY_NONE) atomicAdd(&cnt[0][key & 0xFFu], 1);
+            if ((key >> 8) != KEY_NONE) atomicAdd(&cnt[1][key >> 8], 1);
         }
-#pragma unroll
-        for (int k = 0; k < Q_ITEMS; ++k) {
-            const uint32_t kn = key[k] & 0xFFu, ks = (key[k] >> 8) & 0xFFu;
-            rank[k] = 0;
-            if (kn != KEY_NONE) rank[k] = (uint32_t)atomicAdd(&cnt[0][kn], 1);
-            if (ks != KEY_NONE) rank[k] |= (uint32_t)atomicAdd(&cnt[1][ks], 1) << 16;
-        }
+        if (last) continue;   // no ray goes on from the last bounce
         __syncthreads();
-        // exclusive scan over a queue's cells, one warp per queue
+        // first queue position of each cell, one warp per queue
         if (wid < 2) {
             const int c = cnt[wid][lane];
             int v = c;
@@ -442,15 +426,18 @@ __global__ void __launch_bounds__(Q_BLOCK) k_queue(Wave w, int cur, int depth) {
                 const int y = __shfl_up_sync(0xffffffffu, v, o);
                 if (lane >= o) v += y;
             }
-            cnt[wid][lane] = v - c;
-            if (lane == 31) qbase[wid] = v ? atomicAdd(w.counters + (wid ? sh_slot(cur) : 1 - cur), v) : 0;
+            int base = 0;
+            if (lane == 31 && v) base = atomicAdd(w.counters + (wid ? sh_slot(cur) : 1 - cur), v);
+            cnt[wid][lane] = __shfl_sync(0xffffffffu, base, 31) + v - c;
         }
         __syncthreads();
-#pragma unroll
-        for (int k = 0; k < Q_ITEMS; ++k) {
-            const uint32_t kn = key[k] & 0xFFu, ks = (key[k] >> 8) & 0xFFu;
-            if (kn != KEY_NONE) w.list[1 - cur][qbase[0] + cnt[0][kn] + (rank[k] & 0xFFFFu)] = p[k];
-            if (ks != KEY_NONE) w.sh_list[qbase[1] + cnt[1][ks] + (rank[k] >> 16)] = p[k];
+        for (int k = 0; k < items; ++k) {
+            const uint32_t kn = keys[k * Q_BLOCK + tid] & 0xFFu, ks = keys[k * Q_BLOCK + tid] >> 8;
+            if (kn == KEY_NONE && ks == KEY_NONE) continue;
+            const int64_t i = t0 + k * Q_BLOCK + tid;
+            const int p = list ? __ldg(list + i) : (int)i;
+            if (kn != KEY_NONE) w.list[1 - cur][atomicAdd(&cnt[0][kn], 1)] = p;
+            if (ks != KEY_NONE) w.sh_list[atomicAdd(&cnt[1][ks], 1)] = p;
         }
         __syncthreads();
     }
@@ -841,16 +828,13 @@ cudaError_t launch_trace(const DevScene& sc, const DevFrame& fr, const DevParams
 }
 
 cudaError_t launch_shade(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int cur,
-                         int depth, int64_t max_n, int sms, cudaStream_t st, const Job* jobs) {
+                         int depth, bool last, int64_t max_n, int sms, cudaStream_t st, const Job* jobs) {
+    const int resident = sms * Q_RESIDENT;
+    const int grid = grid_for(max_n, Q_BLOCK, sms, 4 * Q_RESIDENT);
     if (jobs)
-        k_shade<true><<<grid_for(max_n, 128, sms, 16), 128, 0, st>>>(sc, fr, P, w, cur, depth, jobs);
+        k_shade<true><<<grid, Q_BLOCK, 0, st>>>(sc, fr, P, w, cur, depth, last ? 1 : 0, resident, jobs);
     else
-        k_shade<false><<<grid_for(max_n, 128, sms, 16), 128, 0, st>>>(sc, fr, P, w, cur, depth, nullptr);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_queue(const Wave& w, int cur, int depth, int64_t max_n, int sms, cudaStream_t st) {
-    k_queue<<<grid_for(max_n, Q_TILE, sms, 4), Q_BLOCK, 0, st>>>(w, cur, depth);
+        k_shade<false><<<grid, Q_BLOCK, 0, st>>>(sc, fr, P, w, cur, depth, last ? 1 : 0, resident, nullptr);
     return cudaGetLastError();
 }
 

@@ -99,10 +99,9 @@ enum { TRAV_WIDE = 1, TRAV_TLAS = 2 };
 // shadow rays that shade(scur) left, in one launch
 cudaError_t launch_trace(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int ecur, int scur,
                          int depth, int64_t max_n, int32_t* err, int sms, cudaStream_t st, const Job* jobs, int trav);
+// hits of bounce `depth` (ray queue cur), queueing the rays that go on unless it is the last
 cudaError_t launch_shade(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int cur,
-                         int depth, int64_t max_n, int sms, cudaStream_t st, const Job* jobs);
-// queues the rays that shade(cur, depth) left, tile by tile, by direction
-cudaError_t launch_queue(const Wave& w, int cur, int depth, int64_t max_n, int sms, cudaStream_t st);
+                         int depth, bool last, int64_t max_n, int sms, cudaStream_t st, const Job* jobs);
 cudaError_t launch_stats(const Wave& w, const StatsArgs& A, const int32_t* queue, int64_t j0, int64_t n_pix,
                          int32_t* next_queue, int sms, cudaStream_t st, const Job* jobs, const RoundCtl* rc = nullptr);
 // device-resident round loop: start state (and, with iota, queue 0 = 0..Q0-1)

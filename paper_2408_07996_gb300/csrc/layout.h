@@ -133,8 +133,6 @@ struct Wave {
     float4* ray_d;            // xyz direction, w = pdf of the sampled direction
     float2* hit;              // t, leaf-order triangle (int bits; -1: miss)
     int32_t* hit_rec;         // instance record of the hit; written for frames of more than one record
-    uint16_t* key;            // what the vertex just shaded goes on with: direction cell of the next ray in the
-                              // low byte, of the shadow ray in the high byte (KEY_NONE: none)
     // queues of path slots
     int32_t* list[2];         // rays of this bounce and of the next (ping-pong)
     int32_t* sh_list;         // shadow rays
