@@ -438,7 +438,7 @@ mcev_status mcev_detect_batch_static(const mcev_detect_args* args, int64_t* n_un
  *   - PSCD = (mean_a d(a, B) + mean_b d(b, A)) / (2 D);
  *   - MSE over all W*H*T mapped values, RMSE = sqrt(MSE),
  *     PSNR = -10 log10(MSE) (HUGE_VAL for identical videos).
- * The distances are exact (integer distance transform on the GPU).
+ * The distances are exact integers.
  * ------------------------------------------------------------------------ */
 typedef struct mcev_quality {
     int64_t voxels;       /* W * H * T */
@@ -463,8 +463,9 @@ typedef struct mcev_quality {
  * event voxel of a (of b), the squared distance d^2 to the other video's
  * nearest same-polarity event, -2 where it has none, and -1 at voxels
  * without an event; NULL to skip.  Results go to *out (host).  The context
- * needs no scene; scratch (8 bytes per voxel, plus up to 2 GiB of envelope
- * stacks) is allocated through it.
+ * needs no scene; scratch (half a byte per voxel; where very many events have
+ * their nearest counterpart far away also 8 bytes per voxel and up to 2 GiB of
+ * envelope stacks) is allocated through it.
  * Errors: ARG (NULL inputs, an extent outside 1..16384, tau2 < 0, a value
  * outside {-1, 0, 1}), OOM, CUDA.
  * Paper: the quality metrics of Sec. 4.2 (RMSE, PSNR, F1, PSCD). */

@@ -109,7 +109,8 @@ struct mcev_ctx {
     float static_lo[3], static_hi[3];
 
     // device scene
-    DevBuf d_quality;                       // event-quality scratch: two int32 volumes + accumulators
+    DevBuf d_quality;                       // event-quality scratch: accumulators, event bits, far events
+    DevBuf d_qedt;                          // its distance transform: two int32 volumes, envelope stacks
     DevBuf d_gemit;                         // FP64 emission-gradient accumulator of mcev_backward
     DevBuf d_nodes, d_wnodes, d_tris, d_tshade, d_uv, d_mats, d_env, d_marg, d_cond, d_tpdf;
     DevScene dsc{};
@@ -1198,7 +1199,7 @@ void mcev_destroy(mcev_ctx* ctx) {
     cudaStreamSynchronize(ctx->stream);
     DevBuf* bufs[] = {&ctx->d_nodes, &ctx->d_wnodes, &ctx->d_tris, &ctx->d_tshade, &ctx->d_uv, &ctx->d_mats, &ctx->d_env, &ctx->d_marg, &ctx->d_cond,
                       &ctx->d_tpdf, &ctx->frames[0].buf, &ctx->frames[1].buf, &ctx->d_wave, &ctx->d_counters,
-                      &ctx->d_pix, &ctx->d_tcrit, &ctx->d_jobs, &ctx->d_bqueue, &ctx->d_quality, &ctx->d_gemit,
+                      &ctx->d_pix, &ctx->d_tcrit, &ctx->d_jobs, &ctx->d_bqueue, &ctx->d_quality, &ctx->d_qedt, &ctx->d_gemit,
                       &ctx->d_round};
     for (DevBuf* b : bufs) dev_free(ctx, *b);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
@@ -1728,9 +1729,12 @@ mcev_status mcev_event_quality(mcev_ctx* ctx, const int8_t* a, const int8_t* b, 
     if (tau2 < 0) return fail(ctx, MCEV_ERR_ARG, "tau2 must be >= 0");
     CU(cudaSetDevice(ctx->device));
     const int64_t n = (int64_t)width * height * frames;
-    const size_t vol = ((size_t)n * sizeof(int32_t) + 255) & ~size_t(255);
-    const size_t stk = ((size_t)quality_stack_bytes(width, height, frames, ctx->sms) + 255) & ~size_t(255);
-    ST(dev_alloc(ctx, ctx->d_quality, 2 * vol + stk + QACC_WORDS * sizeof(unsigned long long)));
+    auto al = [](int64_t x) { return ((size_t)x + 255) & ~size_t(255); };
+    const size_t nb_acc = QACC_WORDS * sizeof(unsigned long long);
+    const size_t nb_mask = al(quality_mask_bytes(width, height, frames));
+    const size_t nb_cell = al(quality_cell_bytes(width, height, frames));
+    const size_t nb_far = 8 * (size_t)quality_far_cap(width, height, frames);
+    ST(dev_alloc(ctx, ctx->d_quality, al(nb_acc) + nb_mask + nb_cell + nb_far));
     char* base = (char*)ctx->d_quality.ptr;
     QualityArgs A{};
     A.a = a;
@@ -1741,44 +1745,65 @@ mcev_status mcev_event_quality(mcev_ctx* ctx, const int8_t* a, const int8_t* b, 
     A.tau2 = tau2;
     A.d2_a = d2_a;
     A.d2_b = d2_b;
-    A.vol0 = (int32_t*)base;
-    A.vol1 = (int32_t*)(base + vol);
-    A.stack = base + 2 * vol;
-    A.acc = (unsigned long long*)(base + 2 * vol + stk);
+    A.acc = (unsigned long long*)base;
+    A.masks = (uint32_t*)(base + al(nb_acc));
+    A.cells = (uint32_t*)(base + al(nb_acc) + nb_mask);
+    A.far_list = (uint64_t*)(base + al(nb_acc) + nb_mask + nb_cell);
     int nl = 0;
+    std::vector<unsigned long long> acc(QACC_WORDS);
+    auto read_acc = [&]() -> mcev_status {
+        CU(cudaMemcpyAsync(acc.data(), A.acc, nb_acc, cudaMemcpyDeviceToHost, ctx->stream));
+        CU(cudaStreamSynchronize(ctx->stream));
+        ctx->d2h += (int64_t)nb_acc;
+        return MCEV_OK;
+    };
     CU(cudaEventRecord(ctx->ev0, ctx->stream));
     CU(launch_quality(A, ctx->sms, ctx->stream, &nl));
     CU(cudaEventRecord(ctx->ev1, ctx->stream));
-    std::vector<unsigned long long> acc(QACC_WORDS);
-    CU(cudaMemcpyAsync(acc.data(), A.acc, QACC_WORDS * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                       ctx->stream));
-    CU(cudaStreamSynchronize(ctx->stream));
-    ctx->d2h += (int64_t)(QACC_WORDS * sizeof(unsigned long long));
+    ST(read_acc());
     if (acc[QACC_BAD]) return fail(ctx, MCEV_ERR_ARG, "event values must be -1, 0 or +1");
+    // sets with more far events than their list holds: exact distance transform
+    bool again = false;
+    for (int set = 0; set < QSETS; ++set) {
+        if (!acc[QACC_SET + set * QSET_WORDS + QSET_OPEN]) continue;
+        const size_t vol = al(4 * n);
+        ST(dev_alloc(ctx, ctx->d_qedt, 2 * vol + al(quality_stack_bytes(width, height, frames, ctx->sms))));
+        A.vol0 = (int32_t*)ctx->d_qedt.ptr;
+        A.vol1 = (int32_t*)((char*)ctx->d_qedt.ptr + vol);
+        A.stack = (char*)ctx->d_qedt.ptr + 2 * vol;
+        CU(launch_quality_edt(A, set, ctx->sms, ctx->stream, &nl));
+        again = true;
+    }
+    if (again) {
+        CU(cudaEventRecord(ctx->ev1, ctx->stream));
+        ST(read_acc());
+    }
     float ms = 0.0f;
     CU(cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
     mcev_quality q{};
     q.voxels = n;
-    q.n_a = (int64_t)acc[QACC_NA];
-    q.n_b = (int64_t)acc[QACC_NB];
-    q.matched_a = (int64_t)acc[QACC_MATCH_A];
-    q.matched_b = (int64_t)acc[QACC_MATCH_B];
-    q.none_a = (int64_t)acc[QACC_NONE_A];
-    q.none_b = (int64_t)acc[QACC_NONE_B];
+    q.n_a = (int64_t)(acc[QACC_COUNT] + acc[QACC_COUNT + 1]);
+    q.n_b = (int64_t)(acc[QACC_COUNT + 2] + acc[QACC_COUNT + 3]);
     q.sq_diff = (int64_t)acc[QACC_SQ];
-    double sa, sb;
-    std::memcpy(&sa, &acc[QACC_SUM_A], sizeof sa);
-    std::memcpy(&sb, &acc[QACC_SUM_B], sizeof sb);
     const double D = std::sqrt((double)(width - 1) * (width - 1) + (double)(height - 1) * (height - 1) +
                                (double)(frames - 1) * (frames - 1));
     q.diag = D;
-    // distances of d^2 < QHIST come as counts per value
-    for (int v = 1; v < QHIST; ++v) {
-        sa += (double)acc[QACC_HIST_A + v] * std::sqrt((double)v);
-        sb += (double)acc[QACC_HIST_B + v] * std::sqrt((double)v);
+    for (int dir = 0; dir < 2; ++dir) {
+        const unsigned long long* p = &acc[QACC_SET + 2 * dir * QSET_WORDS];
+        const unsigned long long* m = p + QSET_WORDS;
+        const int64_t matched = (int64_t)(p[QSET_MATCH] + m[QSET_MATCH]);
+        const int64_t none = (int64_t)(p[QSET_NONE] + m[QSET_NONE]);
+        double sp, sm;
+        std::memcpy(&sp, p + QSET_SUM, sizeof sp);
+        std::memcpy(&sm, m + QSET_SUM, sizeof sm);
+        double sum = sp + sm;
+        // distances of d^2 < QHIST come as counts per value
+        for (int v = 1; v < QHIST; ++v) sum += (double)(p[QSET_HIST + v] + m[QSET_HIST + v]) * std::sqrt((double)v);
+        sum += (double)none * D;
+        (dir ? q.matched_b : q.matched_a) = matched;
+        (dir ? q.none_b : q.none_a) = none;
+        (dir ? q.sum_dist_b : q.sum_dist_a) = sum;
     }
-    q.sum_dist_a = sa + (double)q.none_a * D;
-    q.sum_dist_b = sb + (double)q.none_b * D;
     // frames mapped {-1, 0, 1} -> {0, 0.5, 1}: each unit of (a - b)^2 is 1/4
     const double mse = (double)q.sq_diff / (4.0 * (double)n);
     q.rmse = std::sqrt(mse);
