@@ -9,7 +9,7 @@
 // per voxel, which stays in L2), events whose own bit is set in the target are
 // counted by AND and population count, and only the rest search the target's
 // rows around them ring by ring until no nearer event can exist.  Events
-// without a neighbour within 15 columns and rings are searched for by a warp each
+// without a neighbour in the rows and columns around them are searched for by a warp each
 // through a coarse grid of cells.  Sets (polarity and direction) with more of
 // them than their list holds are matched by an exact squared Euclidean
 // distance transform on the integer lattice (x, y, t), separable by axis:
