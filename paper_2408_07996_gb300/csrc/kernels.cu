@@ -8,7 +8,7 @@
 // order.  `stats` fuses, per queued pixel, the log-luminance batch statistics
 // (Sec. 3.1, Eq. 3-4), the Chan merge into the running statistics, the t-test
 // of Eq. 7 (Sec. 3.2), the re-queue of undecided pixels (Sec. 3.3; one atomic
-// per warp, since a warp owns a pixel) and the event rule with the reference
+// per warp) and the event rule with the reference
 // update (Alg. 1, Eq. 1).
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -610,6 +610,20 @@ __device__ __forceinline__ Moments chan(Moments a, Moments b) {
 #define MCEV_LOG(x) logf(x)
 #endif
 
+// Four lanes per pixel, eight pixels per warp.  A round traced spp_r samples of
+// a pixel: one batch, or a window of several spp_batch-sized batches.  Each
+// batch is merged and tested in order exactly as Alg. 1 would; once the pixel is
+// decided, the rest of the window is left unused.
+//
+// What bounds it: the instructions of the merge and the test (six divisions
+// and a square root), which every lane of a pixel repeats; with a warp per pixel
+// and 16-sample batches they were done 32 times over (90k pixels x 15 batches:
+// 431 us with a warp per pixel, 137 us with four lanes; eight jobs 131 -> 124 ms,
+// terrain 720p 751 -> 742 ms).  The order of the additions is fixed: sample s of a batch
+// belongs to leaf s % 32, leaves add up pairwise 16, 8, 4, 2 and 1 apart (a warp's
+// butterfly).  A lane holds every fourth leaf, so the last two steps are shuffles
+// (a + b on one lane, b + a on its partner: the same bits), and every lane of a
+// pixel ends with identical statistics and takes the same decisions.
 template <bool kChecked, bool kBatch>
 __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32_t* __restrict__ queue, int64_t j0,
                                                int64_t n_pix, int32_t* __restrict__ next_queue,
@@ -624,15 +638,19 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
         A0.sub = rc->sub;
         A0.k_base = rc->n_done;
     }
-    const int lane = threadIdx.x & 31;
+    constexpr unsigned full = 0xffffffffu;
+    constexpr int LANES = 4, PIX = 32 / LANES, LEAVES = 32 / LANES;
+    const int lane = threadIdx.x & 31, q = lane & (LANES - 1);
     const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t j = warp0; j < n_pix; j += nwarps) {
-        const int32_t entry = __ldg(queue + j0 + j);
+    for (int64_t jw = warp0 * PIX; jw < n_pix; jw += nwarps * PIX) {
+        const int64_t j = jw + lane / LANES;
+        bool on = j < n_pix;
+        const int32_t entry = on ? __ldg(queue + j0 + j) : 0;
         const int32_t pix = kBatch ? (entry & 0xFFFFFF) : entry;
         // per-pixel state and outputs of the pixel's job
         StatsArgs A = A0;
-        if (kBatch) {
+        if (kBatch && on) {
             const Job& J = jobs[(uint32_t)entry >> 24];
             A.cur = J.cur;
             A.ref = J.ref;
@@ -641,69 +659,73 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
             A.mean_out = J.mean_out;
             A.eps = J.P.eps;
         }
-        if (kChecked && (pix < 0 || (int64_t)pix >= A.n_total)) {
-            if (lane == 0) atomicOr(w.counters + 8, 1);
-            continue;
+        if (kChecked && on && (pix < 0 || (int64_t)pix >= A.n_total)) {
+            if (q == 0) atomicOr(w.counters + 8, 1);
+            on = false;
         }
-        // The round traced spp_r samples of this pixel: one batch, or a window
-        // of several spp_batch-sized batches.  Each batch is merged and tested
-        // in order exactly as Alg. 1 would; once the pixel is decided, the
-        // rest of the window is left unused.  Every lane computes the same
-        // statistics (butterfly merges in a fixed order), so the decisions
-        // are warp-uniform.
         Moments c{0.0f, 0.0f, 0.0f};
-        if (A.k_base > 0) c = Moments{(float)A.cur.n[pix], A.cur.mean[pix], A.cur.m2[pix]};
+        if (on && A.k_base > 0) c = Moments{(float)A.cur.n[pix], A.cur.mean[pix], A.cur.m2[pix]};
         const bool detect = A.mode == MODE_DETECT;
-        const float ma = detect ? A.ref.mean[pix] : 0.0f;
-        const int32_t na = detect ? A.ref.n[pix] : 0;
+        const float ma = detect && on ? A.ref.mean[pix] : 0.0f;
+        const int32_t na = detect && on ? A.ref.n[pix] : 0;
         const float va = (detect && na > 1) ? A.ref.m2[pix] / (float)(na - 1) : 0.0f;
         int bad = 0;
-        bool decided = false;
+        bool open = on;        // neither decided nor off
         int32_t n = (int32_t)c.n;
-        const float* Lp = w.L + j * A.spp_r;
-        for (int s0 = 0; s0 < A.spp_r && !decided; s0 += A.sub) {
+        const float* Lp = w.L + (on ? j : 0) * A.spp_r;
+        for (int s0 = 0; s0 < A.spp_r && __any_sync(full, open); s0 += A.sub) {
             const int s1 = min(s0 + A.sub, A.spp_r);
-            // moments of this batch from sums shifted by one warp-uniform value
-            // (the running mean, or the batch's first sample for a pixel's
-            // first batch), so lanes merge by plain addition: the butterfly
-            // below adds a + b on one lane and b + a on its partner, which
-            // are the same bits, so every lane ends with identical sums
-            float sh;
-            if (c.n > 0.0f) {
-                sh = c.mean;
-            } else {
+            // moments of this batch from sums shifted by one value (the running
+            // mean, or the batch's first sample for a pixel's first batch), so
+            // lanes merge by plain addition
+            float sh = c.mean;
+            if (open && !(c.n > 0.0f)) {
                 const float L0 = Lp[s0];
                 sh = MCEV_LOG((isfinite(L0) ? L0 : 0.0f) + A.eps);
             }
-            float s1d = 0.0f, s2d = 0.0f;
-            int cnt = 0;
-            for (int s = s0 + lane; s < s1; s += 32) {
-                float Lv = Lp[s];
-                if (!isfinite(Lv)) {
-                    Lv = 0.0f;
-                    ++bad;
+            float a1[LEAVES], a2[LEAVES];
+#pragma unroll
+            for (int m = 0; m < LEAVES; ++m) a1[m] = a2[m] = 0.0f;
+            if (open) {
+                for (int b = s0 + q; b < s1; b += 32) {
+#pragma unroll
+                    for (int m = 0; m < LEAVES; ++m) {
+                        const int s = b + LANES * m;
+                        if (s < s1) {
+                            float Lv = Lp[s];
+                            if (!isfinite(Lv)) {
+                                Lv = 0.0f;
+                                ++bad;
+                            }
+                            const float d = MCEV_LOG(Lv + A.eps) - sh;
+                            a1[m] += d;
+                            a2[m] = fmaf(d, d, a2[m]);
+                        }
+                    }
                 }
-                const float d = MCEV_LOG(Lv + A.eps) - sh;
-                s1d += d;
-                s2d = fmaf(d, d, s2d);
-                ++cnt;
             }
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                s1d += __shfl_xor_sync(0xffffffffu, s1d, off);
-                s2d += __shfl_xor_sync(0xffffffffu, s2d, off);
-                cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
+            for (int h = LEAVES / 2; h > 0; h >>= 1) {
+#pragma unroll
+                for (int m = 0; m < h; ++m) {
+                    a1[m] += a1[m + h];
+                    a2[m] += a2[m + h];
+                }
             }
-            Moments m{0.0f, 0.0f, 0.0f};
-            if (cnt > 0) {
-                const float fn = (float)cnt;
-                const float md = s1d / fn;
-                m = Moments{fn, sh + md, fmaxf(s2d - s1d * md, 0.0f)};
+            float s1d = a1[0], s2d = a2[0];
+#pragma unroll
+            for (int off = LANES / 2; off > 0; off >>= 1) {
+                s1d += __shfl_xor_sync(full, s1d, off);
+                s2d += __shfl_xor_sync(full, s2d, off);
             }
+            if (!open) continue;
+            const float fn = (float)(s1 - s0);
+            const float md = s1d / fn;
+            const Moments m{fn, sh + md, fmaxf(s2d - s1d * md, 0.0f)};
             c = (A.k_base == 0 && s0 == 0) ? m : chan(c, m);
             n = (int32_t)c.n;
             if (!detect) continue;
-            decided = n >= A.spp_max;
+            bool decided = n >= A.spp_max;
             if (!decided && A.variant != VAR_UNIFORM) {
                 const float gap = fabsf(c.mean - ma);
                 if (A.variant == VAR_MEAN_ONLY) {
@@ -724,28 +746,35 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
                     }
                 }
             }
+            open = !decided;
         }
-        bad = __reduce_add_sync(0xffffffffu, bad);
-        if (lane != 0) continue;
+#pragma unroll
+        for (int off = LANES / 2; off > 0; off >>= 1) bad += __shfl_xor_sync(full, bad, off);
+        // the pixel's first lane writes it back; undecided pixels go on in queue order
+        const bool own = on && q == 0;
+        const bool again = own && (detect ? open : n < A.spp_max);
+        const unsigned more = __ballot_sync(full, again);
+        int at = 0;
+        if (lane == 0 && more) at = atomicAdd(w.counters + 3, __popc(more));
+        at = __shfl_sync(full, at, 0);
+        if (!own) continue;
         if (bad) atomicAdd(w.counters + 4, bad);
         A.cur.n[pix] = n;
         A.cur.mean[pix] = c.mean;
         A.cur.m2[pix] = c.m2;
+        if (again) {
+            next_queue[at + __popc(more & ((1u << lane) - 1u))] = entry;
+            continue;
+        }
         if (!detect) {
-            if (n >= A.spp_max && A.mode == MODE_MEAN) {
+            if (A.mode == MODE_MEAN) {
                 A.mean_out[pix] = c.mean;
                 if (A.spp_out) A.spp_out[pix] = n;
-            } else if (n >= A.spp_max) {
+            } else {
                 A.ref.n[pix] = n;
                 A.ref.mean[pix] = c.mean;
                 A.ref.m2[pix] = c.m2;
-            } else {
-                next_queue[atomicAdd(w.counters + 3, 1)] = entry;
             }
-            continue;
-        }
-        if (!decided) {
-            next_queue[atomicAdd(w.counters + 3, 1)] = entry;
             continue;
         }
         const float delta = c.mean - ma;
@@ -842,17 +871,17 @@ cudaError_t launch_stats(const Wave& w, const StatsArgs& A, const int32_t* queue
                          int32_t* next_queue, int sms, cudaStream_t st, const Job* jobs, const RoundCtl* rc) {
     // with rc, n_pix is an upper bound of the chunk's pixels (the size is on the device)
     if (jobs)
-        k_stats<false, true><<<grid_for(n_pix * 32, 256, sms, 8), 256, 0, st>>>(w, A, queue, j0, n_pix, next_queue,
+        k_stats<false, true><<<grid_for(n_pix * 4, 256, sms, 8), 256, 0, st>>>(w, A, queue, j0, n_pix, next_queue,
                                                                                  jobs, rc);
     else
-        k_stats<false, false><<<grid_for(n_pix * 32, 256, sms, 8), 256, 0, st>>>(w, A, queue, j0, n_pix, next_queue,
+        k_stats<false, false><<<grid_for(n_pix * 4, 256, sms, 8), 256, 0, st>>>(w, A, queue, j0, n_pix, next_queue,
                                                                                   nullptr, rc);
     return cudaGetLastError();
 }
 
 static cudaError_t launch_stats_checked(const Wave& w, const StatsArgs& A, const int32_t* queue, int64_t n_pix,
                                         int32_t* next_queue, int sms, cudaStream_t st) {
-    k_stats<true, false><<<grid_for(n_pix * 32, 256, sms, 8), 256, 0, st>>>(w, A, queue, 0, n_pix, next_queue,
+    k_stats<true, false><<<grid_for(n_pix * 4, 256, sms, 8), 256, 0, st>>>(w, A, queue, 0, n_pix, next_queue,
                                                                              nullptr, nullptr);
     return cudaGetLastError();
 }
