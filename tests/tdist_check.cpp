@@ -2,6 +2,7 @@
 // table (rounded to FP32) equals the root of the same CDF by plain bisection.
 #include <cmath>
 #include <cstdio>
+#include <initializer_list>
 
 #include "tdist.h"
 
