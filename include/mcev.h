@@ -135,7 +135,8 @@ typedef struct {
 /* kernel classes reported in mcev_stats.  MCEV_K_EXTEND counts the traversal
  * launches: closest hits, and the shadow rays a bounce traces in the same
  * launch as the next bounce's closest hits (MCEV_K_SHADOW then stays 0).
- * MCEV_K_SHADE counts shading and the queueing of the rays it leaves. */
+ * MCEV_K_SHADE counts shading and the queueing of the rays it leaves.  Camera rays
+ * are started in the traversal launch of the first bounce (MCEV_K_RAYGEN stays 0). */
 enum { MCEV_K_RAYGEN = 0, MCEV_K_EXTEND = 1, MCEV_K_SHADE = 2, MCEV_K_SHADOW = 3, MCEV_K_STATS = 4,
        MCEV_K_CLASSES = 5 };
 

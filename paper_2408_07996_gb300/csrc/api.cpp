@@ -842,18 +842,17 @@ mcev_status trace_chunk(mcev_ctx* ctx, const Frame& fr, const DevParams& P, cons
     const bool tlas = B ? B->any_tlas : fr.dev.n_tlas >= 2;
     const int trav = (wide ? TRAV_WIDE : 0) | (tlas ? TRAV_TLAS : 0);
     NvtxRange range("mcev chunk");
-    LAUNCH(MCEV_K_RAYGEN,
-           launch_raygen(fr.dev, P, w, queue, j0, spp_r, k_base, n_paths, 0, ctx->sms, ctx->stream, jobs, rc));
     int cur = 0;
-    LAUNCH(MCEV_K_EXTEND, launch_trace(ctx->dsc, fr.dev, P, w, cur, -1, 0, n_paths, err, ctx->sms, ctx->stream, jobs,
-                                       trav));
+    const Chunk ch{queue, j0, k_base, (int32_t)n_paths, spp_r};
+    LAUNCH(MCEV_K_EXTEND, launch_trace(ctx->dsc, fr.dev, P, w, cur, -1, 0, ch, n_paths, err, ctx->sms, ctx->stream,
+                                       jobs, trav, rc));
     for (int depth = 0; depth <= depth_max; ++depth) {
         LAUNCH(MCEV_K_SHADE, launch_shade(ctx->dsc, fr.dev, P, w, cur, depth, depth == depth_max, n_paths, ctx->sms,
                                           ctx->stream, jobs));
         if (depth < depth_max) {
             // this bounce's shadow rays and the next bounce's closest hits in one launch
-            LAUNCH(MCEV_K_EXTEND, launch_trace(ctx->dsc, fr.dev, P, w, cur ^ 1, nee ? cur : -1, depth + 1, n_paths,
-                                               err, ctx->sms, ctx->stream, jobs, trav));
+            LAUNCH(MCEV_K_EXTEND, launch_trace(ctx->dsc, fr.dev, P, w, cur ^ 1, nee ? cur : -1, depth + 1, ch,
+                                               n_paths, err, ctx->sms, ctx->stream, jobs, trav, nullptr));
         }
         cur ^= 1;
     }

@@ -1,7 +1,7 @@
 // kernels.cu -- wavefront path tracer and statistical event detector.
 //
 // One chunk of paths goes through
-//   raygen -> extend -> [shade(+NEE) -> shadow + extend] x max_depth -> shade -> stats
+//   camera rays + extend -> [shade(+NEE) -> shadow + extend] x max_depth -> shade -> stats
 // Every path keeps one slot of the wavefront for its ray and state; extend,
 // shade and shadow walk device-side queues of slots (sizes in device
 // counters, no host round trip) that shade fills tile by tile in direction
@@ -55,58 +55,41 @@ __device__ __forceinline__ uint32_t dir_cell(f3 d) {
 __device__ __forceinline__ int sh_slot(int cur) { return cur ? 19 : 2; }
 static constexpr uint32_t FNV_BASIS = 2166136261u;
 
-// ------------------------------------------------------------------ raygen
+// ------------------------------------------------------------------ camera rays
+// Starts path p of a chunk: sample k_base + p % spp_r of queue entry j0 + p / spp_r.
 // kBatch: queue entries are (job << 24 | pixel) and every path reads its
 // job's frame and settings from the job table; otherwise entries are pixels
-// of the single context whose frame and settings are kernel arguments.  A
-// ray's `w` lane carries its bounce depth | job << 8.
+// of the single context whose frame and settings are kernel arguments.
 template <bool kBatch>
-__global__ void __launch_bounds__(256) k_raygen(DevFrame fr, DevParams P, Wave w, const int32_t* __restrict__ queue,
-                                                int64_t j0, int32_t spp_r, int64_t k_base, int64_t n_paths, int cur,
-                                                const Job* __restrict__ jobs, const RoundCtl* __restrict__ rc) {
-    if (rc) {
-        // sizes of the current chunk of the device-resident round loop
-        queue = rc->queue[rc->qi];
-        j0 = rc->j0;
-        spp_r = rc->spp_r;
-        k_base = rc->n_done;
-        n_paths = rc->nj * (int64_t)rc->spp_r;
+__device__ __forceinline__ void start_path(const DevFrame& fr, const DevParams& P, const Wave& w, const Chunk& ch,
+                                           int p, const Job* __restrict__ jobs) {
+    const int j = p / ch.spp_r;
+    const int32_t s = p - j * ch.spp_r;
+    const int32_t entry = __ldg(ch.queue + ch.j0 + j);
+    const int job = kBatch ? (int)((uint32_t)entry >> 24) : 0;
+    const int32_t pix = kBatch ? (entry & 0xFFFFFF) : entry;
+    const DevFrame& F = kBatch ? jobs[job].fr : fr;
+    const DevParams& Q = kBatch ? jobs[job].P : P;
+    const uint32_t k = (uint32_t)(ch.k_base + s);
+    const uint4 x = philox4x32_10(make_uint4((uint32_t)pix, k, 0u, 0u), F.key0, F.key1);
+    const int px = pix % Q.width, py = pix / Q.width;
+    const float fx = 2.0f * ((float)px + u01(x.x)) / (float)Q.width - 1.0f;
+    const float fy = 1.0f - 2.0f * ((float)py + u01(x.y)) / (float)Q.height;
+    const f3 d = norm3(mk3(F.fwd[0] + fx * F.right[0] + fy * F.up[0],
+                           F.fwd[1] + fx * F.right[1] + fy * F.up[1],
+                           F.fwd[2] + fx * F.right[2] + fy * F.up[2]));
+    w.ray_o[p] = make_float4(F.eye[0], F.eye[1], F.eye[2], 1.0f);
+    w.ray_d[p] = make_float4(d.x, d.y, d.z, 0.0f);
+    w.L[p] = 0.0f;
+    w.pix_k[p] = make_int2(entry, (int)k);
+    if (Q.adjoint && Q.grad_mean) {
+        // d loss / d L of this path: d loss / d mean * d mean / d ln(L + eps) * d ln(L + eps) / dL
+        const float Lt = w.Ltot[p];
+        w.delta[p] = isfinite(Lt) ? __ldg(Q.grad_mean + pix) / ((float)Q.spp * (Lt + Q.eps)) : 0.0f;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        w.counters[cur] = (int32_t)n_paths;
-        w.counters[1 - cur] = 0;
-        w.counters[2] = w.counters[19] = 0;
-        w.counters[20] = 0;
-    }
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n_paths; p += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = p / spp_r;
-        const int32_t s = (int32_t)(p - j * spp_r);
-        const int32_t entry = __ldg(queue + j0 + j);
-        const int job = kBatch ? (int)((uint32_t)entry >> 24) : 0;
-        const int32_t pix = kBatch ? (entry & 0xFFFFFF) : entry;
-        const DevFrame& F = kBatch ? jobs[job].fr : fr;
-        const DevParams& Q = kBatch ? jobs[job].P : P;
-        const uint32_t k = (uint32_t)(k_base + s);
-        const uint4 x = philox4x32_10(make_uint4((uint32_t)pix, k, 0u, 0u), F.key0, F.key1);
-        const int px = pix % Q.width, py = pix / Q.width;
-        const float fx = 2.0f * ((float)px + u01(x.x)) / (float)Q.width - 1.0f;
-        const float fy = 1.0f - 2.0f * ((float)py + u01(x.y)) / (float)Q.height;
-        const f3 d = norm3(mk3(F.fwd[0] + fx * F.right[0] + fy * F.up[0],
-                               F.fwd[1] + fx * F.right[1] + fy * F.up[1],
-                               F.fwd[2] + fx * F.right[2] + fy * F.up[2]));
-        w.ray_o[p] = make_float4(F.eye[0], F.eye[1], F.eye[2], 1.0f);
-        w.ray_d[p] = make_float4(d.x, d.y, d.z, 0.0f);
-        w.L[p] = 0.0f;
-        w.pix_k[p] = make_int2(entry, (int)k);
-        if (Q.adjoint && Q.grad_mean) {
-            // d loss / d L of this path: d loss / d mean * d mean / d ln(L + eps) * d ln(L + eps) / dL
-            const float Lt = w.Ltot[p];
-            w.delta[p] = isfinite(Lt) ? __ldg(Q.grad_mean + pix) / ((float)Q.spp * (Lt + Q.eps)) : 0.0f;
-        }
-        if (Q.want_sig) {
-            w.sig[p] = FNV_BASIS;
-            w.pflags[p] = NO_FLAGS;
-        }
+    if (Q.want_sig) {
+        w.sig[p] = FNV_BASIS;
+        w.pflags[p] = NO_FLAGS;
     }
 }
 
@@ -396,6 +379,8 @@ __global__ void __launch_bounds__(Q_BLOCK, Q_RESIDENT)
     k_shade(DevScene sc, DevFrame fr, DevParams P, Wave w, int cur, int depth, int last, int resident,
             const Job* __restrict__ jobs) {
     __shared__ uint16_t keys[Q_TILE];
+    __shared__ uint16_t order[Q_TILE];  // the tile's entries, misses first
+    __shared__ int n_miss, n_hit;
     __shared__ int cnt[2][KEY_CELLS];   // next rays, shadow rays
     const int32_t n = *(volatile int32_t*)(w.counters + cur);
     const int32_t* list = depth > 0 ? w.list[cur] : nullptr;
@@ -406,12 +391,37 @@ __global__ void __launch_bounds__(Q_BLOCK, Q_RESIDENT)
     const int items = max(1, min(Q_ITEMS, (n + step - 1) / step));
     for (int64_t t0 = (int64_t)blockIdx.x * items * Q_BLOCK; t0 < n; t0 += (int64_t)gridDim.x * items * Q_BLOCK) {
         if (tid < 2 * KEY_CELLS) (&cnt[0][0])[tid] = 0;
+        if (tid == 0) n_miss = n_hit = 0;
         __syncthreads();
+        const int size = (int)min((int64_t)items * Q_BLOCK, n - t0);
+        // After the camera rays (whose pixels mostly see one thing), rays that hit and
+        // rays that leave the scene are shaded apart: mixed, 15 of 32 lanes were active.
+        const bool split = list != nullptr;
+        if (split) {
+            for (int k = 0; k < items; ++k) {
+                const int e = k * Q_BLOCK + tid;
+                const bool in = e < size;
+                const bool miss = in && __float_as_int(w.hit[__ldg(list + t0 + e)].y) < 0;
+                const unsigned bm = __ballot_sync(0xffffffffu, miss), bh = __ballot_sync(0xffffffffu, in && !miss);
+                int am = 0, ah = 0;
+                if (lane == 0) {
+                    if (bm) am = atomicAdd(&n_miss, __popc(bm));
+                    if (bh) ah = atomicAdd(&n_hit, __popc(bh));
+                }
+                am = __shfl_sync(0xffffffffu, am, 0) + __popc(bm & ((1u << lane) - 1u));
+                ah = size - 1 - __shfl_sync(0xffffffffu, ah, 0) - __popc(bh & ((1u << lane) - 1u));
+                if (in) order[miss ? am : ah] = (uint16_t)e;
+            }
+            __syncthreads();
+        }
         for (int k = 0; k < items; ++k) {
-            const int64_t i = t0 + k * Q_BLOCK + tid;
+            int e = k * Q_BLOCK + tid;
             uint32_t key = KEY_NONE | (KEY_NONE << 8);
-            if (i < n) key = shade_path<kBatch>(sc, fr, P, w, list ? __ldg(list + i) : (int)i, depth, jobs);
-            keys[k * Q_BLOCK + tid] = (uint16_t)key;
+            if (e < size) {
+                if (split) e = order[e];
+                key = shade_path<kBatch>(sc, fr, P, w, list ? __ldg(list + t0 + e) : (int)(t0 + e), depth, jobs);
+            }
+            keys[e] = (uint16_t)key;
             if ((key & 0xFFu) != KEY_NONE) atomicAdd(&cnt[0][key & 0xFFu], 1);
             if ((key >> 8) != KEY_NONE) atomicAdd(&cnt[1][key >> 8], 1);
         }
@@ -487,8 +497,9 @@ struct Groups {
 // machine costs more than it fills.)
 template <bool kAny, bool kBatch, bool kWide, bool kTlas>
 __device__ __forceinline__ int3 trace_queue(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w,
-                                            const int32_t* __restrict__ list, int32_t n, Groups& gr, int g0, int g_end,
-                                            int* stack, int32_t* err, const Job* __restrict__ jobs) {
+                                            const int32_t* __restrict__ list, const Chunk* ch, int32_t n, Groups& gr,
+                                            int g0, int g_end, int* stack, int32_t* err,
+                                            const Job* __restrict__ jobs) {
     const int lane = threadIdx.x & 31;
     const float4* dirs = kAny ? w.sh_d : w.ray_d;
     int2 work = make_int2(0, 0);
@@ -499,6 +510,10 @@ __device__ __forceinline__ int3 trace_queue(const DevScene& sc, const DevFrame& 
         const bool live = g + lane < n;
         const int i = live ? g + lane : n - 1;
         const int p = list ? __ldg(list + i) : i;
+        if (!kAny && ch) {
+            if (live) start_path<kBatch>(fr, P, w, *ch, p, jobs);
+            __syncwarp();
+        }
         const int job = kBatch ? (int)((uint32_t)w.pix_k[p].x >> 24) : 0;
         const DevScene& S = kBatch ? jobs[job].sc : sc;
         const DevFrame& F = kBatch ? jobs[job].fr : fr;
@@ -554,17 +569,22 @@ __device__ __forceinline__ int3 trace_queue(const DevScene& sc, const DevFrame& 
 // One launch traces the closest hits of bounce `depth` (ray queue `ecur`) and,
 // with scur >= 0, then the shadow rays of the bounce before (appended with queue
 // scur).
+// At depth 0 the rays are the chunk's camera rays (rc: the device-resident round
+// loop's current chunk), started here: a kernel of their own wrote and this one
+// read 32 bytes more per path (7.8 ms of a terrain 720p frame).
 // The grid is the resident warps only; queue sizes are read on the device.
 // The first thread also clears the counters the next queues append to.
 template <bool kBatch, bool kWide, bool kTlas>
 __global__ void __launch_bounds__(MCEV_TRAV_BLOCK, trav_blocks(kWide, kTlas))
-    k_trace(DevScene sc, DevFrame fr, DevParams P, Wave w, int ecur, int scur, int depth, int32_t* err,
-            const Job* __restrict__ jobs) {
+    k_trace(DevScene sc, DevFrame fr, DevParams P, Wave w, int ecur, int scur, int depth, Chunk ch, int32_t* err,
+            const Job* __restrict__ jobs, const RoundCtl* __restrict__ rc) {
     int stack[MCEV_STACK];
     work_begin();
-    const int32_t n = *(volatile int32_t*)(w.counters + ecur);
+    if (rc) ch = Chunk{rc->queue[rc->qi], rc->j0, rc->n_done, (int32_t)(rc->nj * rc->spp_r), rc->spp_r};
+    const int32_t n = depth == 0 ? ch.n_paths : *(volatile int32_t*)(w.counters + ecur);
     const int32_t ns = scur >= 0 ? *(volatile int32_t*)(w.counters + sh_slot(scur)) : 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (depth == 0) w.counters[ecur] = n;
         w.counters[1 - ecur] = 0;
         w.counters[sh_slot(ecur)] = 0;
         unsigned long long* c = reinterpret_cast<unsigned long long*>(w.counters + 32);
@@ -574,11 +594,12 @@ __global__ void __launch_bounds__(MCEV_TRAV_BLOCK, trav_blocks(kWide, kTlas))
     const int ge = (n + 31) >> 5;
     Groups gr{(int)(blockIdx.x * (MCEV_TRAV_BLOCK / 32) + (threadIdx.x >> 5)), (int)gridDim.x * (MCEV_TRAV_BLOCK / 32),
               ge + ((ns + 31) >> 5), w.counters + 20, 0};
-    const int3 wc = trace_queue<false, kBatch, kWide, kTlas>(sc, fr, P, w, depth > 0 ? w.list[ecur] : nullptr, n, gr, 0,
-                                                             ge, stack, err, jobs);
+    const int3 wc = trace_queue<false, kBatch, kWide, kTlas>(sc, fr, P, w, depth > 0 ? w.list[ecur] : nullptr,
+                                                             depth > 0 ? nullptr : &ch, n, gr, 0, ge, stack, err, jobs);
     int3 ws = make_int3(0, 0, 0);
     if (scur >= 0)
-        ws = trace_queue<true, kBatch, kWide, kTlas>(sc, fr, P, w, w.sh_list, ns, gr, ge, gr.total, stack, err, jobs);
+        ws = trace_queue<true, kBatch, kWide, kTlas>(sc, fr, P, w, w.sh_list, nullptr, ns, gr, ge, gr.total, stack, err,
+                                                       jobs);
     add_work(w, wc, ws);
 }
 
@@ -822,27 +843,15 @@ static int grid_for(int64_t work, int block, int sms, int per_sm) {
     return (int)g;
 }
 
-cudaError_t launch_raygen(const DevFrame& fr, const DevParams& P, const Wave& w, const int32_t* queue, int64_t j0,
-                          int32_t spp_r, int64_t k_base, int64_t n_paths, int cur, int sms, cudaStream_t st,
-                          const Job* jobs, const RoundCtl* rc) {
-    // with rc, n_paths is the wavefront capacity (the chunk's size is on the device)
-    if (jobs)
-        k_raygen<true><<<grid_for(n_paths, 256, sms, 16), 256, 0, st>>>(fr, P, w, queue, j0, spp_r, k_base, n_paths,
-                                                                          cur, jobs, rc);
-    else
-        k_raygen<false><<<grid_for(n_paths, 256, sms, 16), 256, 0, st>>>(fr, P, w, queue, j0, spp_r, k_base, n_paths,
-                                                                           cur, nullptr, rc);
-    return cudaGetLastError();
-}
-
 // traversal kernels by (batched jobs, BLAS layout, moving instances under a TLAS)
 cudaError_t launch_trace(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int ecur, int scur,
-                         int depth, int64_t max_n, int32_t* err, int sms, cudaStream_t st, const Job* jobs, int trav) {
+                         int depth, const Chunk& ch, int64_t max_n, int32_t* err, int sms, cudaStream_t st,
+                         const Job* jobs, int trav, const RoundCtl* rc) {
     // both queues of at most max_n rays
     const int64_t work = scur >= 0 ? 2 * max_n : max_n;
 #define MCEV_TRACE(kb, kw, kt)                                                                                      \
     k_trace<kb, kw, kt><<<grid_for(work, MCEV_TRAV_BLOCK, sms, trav_blocks(kw, kt)), MCEV_TRAV_BLOCK, 0, st>>>( \
-        sc, fr, P, w, ecur, scur, depth, err, jobs)
+        sc, fr, P, w, ecur, scur, depth, ch, err, jobs, depth == 0 ? rc : nullptr)
     switch ((jobs ? 4 : 0) | ((trav & TRAV_WIDE) ? 2 : 0) | ((trav & TRAV_TLAS) ? 1 : 0)) {
     case 0: MCEV_TRACE(false, false, false); break;
     case 1: MCEV_TRACE(false, false, true); break;

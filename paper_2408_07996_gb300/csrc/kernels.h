@@ -26,10 +26,18 @@ struct StatsArgs {
     int64_t n_total;      // per-pixel array length, checked only by the allocation-free entry point
 };
 
+// The paths of one chunk: spp_r samples, from number k_base on, of consecutive
+// entries of a pixel queue from j0 on.
+struct Chunk {
+    const int32_t* queue;
+    int64_t j0, k_base;
+    int32_t n_paths, spp_r;
+};
+
 // State of the device-resident round loop of one call (device memory): the
 // round's pixel queue and sizes, the current chunk, and what was done.  The
-// control kernel advances it after every chunk; raygen and the statistics
-// kernel read their sizes from it instead of from launch arguments.
+// control kernel advances it after every chunk; the first traversal launch and
+// the statistics kernel read their sizes from it instead of from launch arguments.
 struct RoundCtl {
     int32_t* queue[2];        // ping-pong pixel queues; queue[qi] is this round's
     int64_t Q;                // pixels queued this round
@@ -86,19 +94,18 @@ MCEV_HD inline int64_t round_window(int64_t cap, int64_t q, int64_t sub, int64_t
 // `jobs`: device job table of a batched render, or nullptr for a single
 // context (then the frame / settings / state arguments are used).  `rc`:
 // sizes from the device-resident round loop instead of the arguments.
-cudaError_t launch_raygen(const DevFrame& fr, const DevParams& P, const Wave& w, const int32_t* queue, int64_t j0,
-                          int32_t spp_r, int64_t k_base, int64_t n_paths, int cur, int sms, cudaStream_t st,
-                          const Job* jobs, const RoundCtl* rc = nullptr);
 // `wide`: the scenes' BLAS use the compressed 8-wide layout (Node8)
 // Traversal kernel variant (the `trav` argument of the launchers): the BLAS
 // layout, and whether the frame has two or more moving instances under a
 // TLAS (frames with at most one run kernels without the TLAS loop).
 enum { TRAV_WIDE = 1, TRAV_TLAS = 2 };
 
-// closest hits of bounce `depth` (ray queue ecur) and, with scur >= 0, the
+// closest hits of bounce `depth` (ray queue ecur; at depth 0 the camera rays of
+// chunk `ch`, or of the round loop's) and, with scur >= 0, the
 // shadow rays that shade(scur) left, in one launch
 cudaError_t launch_trace(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int ecur, int scur,
-                         int depth, int64_t max_n, int32_t* err, int sms, cudaStream_t st, const Job* jobs, int trav);
+                         int depth, const Chunk& ch, int64_t max_n, int32_t* err, int sms, cudaStream_t st,
+                         const Job* jobs, int trav, const RoundCtl* rc);
 // hits of bounce `depth` (ray queue cur), queueing the rays that go on unless it is the last
 cudaError_t launch_shade(const DevScene& sc, const DevFrame& fr, const DevParams& P, const Wave& w, int cur,
                          int depth, bool last, int64_t max_n, int sms, cudaStream_t st, const Job* jobs);
