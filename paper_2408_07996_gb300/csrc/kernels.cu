@@ -93,6 +93,69 @@ __device__ __forceinline__ void start_path(const DevFrame& fr, const DevParams& 
     }
 }
 
+// ------------------------------------------------------------------ gradient sums
+// Millions of contributions land on a few lights and, within a warp, on a few
+// texels; atomics on one word serialise (FP64 ones on four lights' words took
+// 140 us of a 200-us traversal launch and 140 us of a 250-us shading launch of
+// the 256x256 gradient step).  They are added up first: per warp, and for the
+// first EMIT_SLOTS materials per block.
+constexpr int EMIT_SLOTS = 32;
+
+// acc[m] (or grad_emit[m]) += v for the lanes with m >= 0; the whole warp calls
+__device__ __forceinline__ void warp_add_emit(double* acc, double* grad_emit, int m, double v) {
+    const unsigned full = 0xffffffffu;
+    unsigned todo = __ballot_sync(full, m >= 0);
+    while (todo) {
+        const int lead = __ffs(todo) - 1;
+        const int mm = __shfl_sync(full, m, lead);
+        double x = m == mm ? v : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(full, x, o);
+        if ((int)(threadIdx.x & 31) == lead) atomicAdd((mm < EMIT_SLOTS ? acc : grad_emit) + mm, x);
+        todo &= ~__ballot_sync(full, m == mm);
+    }
+}
+
+// d loss / d texel += g * (luminance weights) for the lanes with texel >= 0; the
+// whole warp calls.  Texels that several lanes share are added up first.
+__device__ __forceinline__ void warp_add_tex(float* grad_tex, int texel, float g) {
+    const unsigned full = 0xffffffffu;
+    unsigned todo = __ballot_sync(full, texel >= 0);
+    while (todo) {
+        const int lead = __ffs(todo) - 1;
+        const int tt = __shfl_sync(full, texel, lead);
+        const unsigned same = __ballot_sync(full, texel == tt);
+        if (__popc(same) < 4) break;       // scattered: the loop would cost more than it saves
+        float x = texel == tt ? g : 0.0f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(full, x, o);
+        if (texel == tt) {
+            g = x;
+            if ((int)(threadIdx.x & 31) != lead) texel = -1;
+        }
+        if ((int)(threadIdx.x & 31) == lead) {
+            float* gt = grad_tex + 3 * (int64_t)tt;
+            atomicAdd(gt, x * MCEV_Y_R);
+            atomicAdd(gt + 1, x * MCEV_Y_G);
+            atomicAdd(gt + 2, x * MCEV_Y_B);
+            texel = -1;
+        }
+        todo &= ~same;
+    }
+    if (texel >= 0) {
+        float* gt = grad_tex + 3 * (int64_t)texel;
+        atomicAdd(gt, g * MCEV_Y_R);
+        atomicAdd(gt + 1, g * MCEV_Y_G);
+        atomicAdd(gt + 2, g * MCEV_Y_B);
+    }
+}
+
+// what a shaded vertex adds to the gradients (material / texel -1: nothing)
+struct VertexGrad {
+    int mat, texel;
+    float emit, tex;
+};
+
 // Per-block accumulation of the traversal work counters: work_begin at the
 // top of the kernel, add_work at its end.  Each warp adds its sums in shared
 // memory; the last warp of the block to finish adds the block's totals to
@@ -100,6 +163,7 @@ __device__ __forceinline__ void start_path(const DevFrame& fr, const DevParams& 
 // and box tests of closest-hit rays, then of shadow rays.
 struct WorkAcc {
     unsigned long long v[6];
+    double emit[EMIT_SLOTS];      // adjoint: the block's emission gradients
     unsigned int done;
 };
 
@@ -111,6 +175,7 @@ __device__ __forceinline__ WorkAcc& work_acc() {
 __device__ __forceinline__ void work_begin() {
     WorkAcc& a = work_acc();
     if (threadIdx.x < 6) a.v[threadIdx.x] = 0ull;
+    if (threadIdx.x < EMIT_SLOTS) a.emit[threadIdx.x] = 0.0;
     if (threadIdx.x == 0) a.done = 0u;
     __syncthreads();
 }
@@ -128,7 +193,7 @@ __device__ __forceinline__ void warp_work(WorkAcc& a, int at, int3 work) {
 }
 
 // the whole warp, converged after its ray loops
-__device__ __forceinline__ void add_work(const Wave& w, int3 closest, int3 shadow) {
+__device__ __forceinline__ void add_work(const Wave& w, int3 closest, int3 shadow, double* grad_emit) {
     WorkAcc& a = work_acc();
     warp_work(a, 0, closest);
     warp_work(a, 3, shadow);
@@ -143,6 +208,11 @@ __device__ __forceinline__ void add_work(const Wave& w, int3 closest, int3 shado
                 const unsigned long long v = atomicAdd(&a.v[i], 0ull);
                 if (v) atomicAdd(c + word[i], v);
             }
+            if (grad_emit)
+                for (int m = 0; m < EMIT_SLOTS; ++m) {
+                    const double v = atomicAdd(&a.emit[m], 0.0);
+                    if (v != 0.0) atomicAdd(grad_emit + m, v);
+                }
         }
     }
 }
@@ -172,9 +242,11 @@ __device__ __forceinline__ void add_work(const Wave& w, int3 closest, int3 shado
 static constexpr int Q_BLOCK = 256, Q_TILE = 4096, Q_ITEMS = Q_TILE / Q_BLOCK;
 static constexpr int Q_RESIDENT = 1024 / Q_BLOCK;   // blocks per SM
 
-template <bool kBatch>
+// kAdjoint: the replay pass of mcev_backward (never batched)
+template <bool kBatch, bool kAdjoint>
 __device__ __forceinline__ uint32_t shade_path(const DevScene& sc, const DevFrame& fr, const DevParams& P,
-                                               const Wave& w, int p, int depth, const Job* __restrict__ jobs) {
+                                               const Wave& w, int p, int depth, const Job* __restrict__ jobs,
+                                               VertexGrad& vg) {
     const float4 ro = w.ray_o[p];
     const float4 rd = w.ray_d[p];
     const int2 rs = w.pix_k[p];
@@ -257,7 +329,7 @@ __device__ __forceinline__ uint32_t shade_path(const DevScene& sc, const DevFram
             alb = MCEV_Y_R * __ldg(rgb) + MCEV_Y_G * __ldg(rgb + 1) + MCEV_Y_B * __ldg(rgb + 2);
             if (Q.want_sig) sig = fnv(sig, (uint32_t)texel);
         }
-        const float dlt = Q.adjoint ? w.delta[p] : 0.0f;
+        const float dlt = kAdjoint ? w.delta[p] : 0.0f;
         uint32_t flags = 0;
         const float cos_o = dot3(ng, wo);
         if (emit > 0.0f && cos_o > 0.0f) {
@@ -278,16 +350,16 @@ __device__ __forceinline__ uint32_t shade_path(const DevScene& sc, const DevFram
                 }
             }
             Ladd = beta * wgt * emit;
-            if (Q.adjoint && Q.grad_emit) atomicAdd(Q.grad_emit + mat, (double)(dlt * beta * wgt));
+            if (kAdjoint && Q.grad_emit) {
+                vg.mat = mat;
+                vg.emit = dlt * beta * wgt;
+            }
         }
         if (depth < Q.max_depth && alb > 0.0f) {
             // adjoint: every contribution after this vertex carries one factor of its albedo
-            if (Q.adjoint && texel >= 0 && Q.grad_tex && dlt != 0.0f) {
-                const float g = dlt * (w.Ltot[p] - (w.L[p] + Ladd)) / alb;
-                float* gt = Q.grad_tex + 3 * (int64_t)texel;
-                atomicAdd(gt, g * MCEV_Y_R);
-                atomicAdd(gt + 1, g * MCEV_Y_G);
-                atomicAdd(gt + 2, g * MCEV_Y_B);
+            if (kAdjoint && texel >= 0 && Q.grad_tex && dlt != 0.0f) {
+                vg.texel = texel;
+                vg.tex = dlt * (w.Ltot[p] - (w.L[p] + Ladd)) / alb;
             }
             const f3 nn = cos_o < 0.0f ? ng * -1.0f : ng;
             f3 tb, bt;
@@ -365,7 +437,7 @@ __device__ __forceinline__ uint32_t shade_path(const DevScene& sc, const DevFram
     if (shadow) {
         w.sh_d[p] = make_float4(sh_dir.x, sh_dir.y, sh_dir.z, sh_tmax);
         w.sh_c[p] = sh_c;
-        if (Q.adjoint) {
+        if (kAdjoint) {
             w.sh_g[p] = sh_g;
             w.sh_m[p] = sh_m;
         }
@@ -374,19 +446,21 @@ __device__ __forceinline__ uint32_t shade_path(const DevScene& sc, const DevFram
     return (cont ? dir_cell(wi_next) : KEY_NONE) | (shadow ? dir_cell(sh_dir) : KEY_NONE) << 8;
 }
 
-template <bool kBatch>
+template <bool kBatch, bool kAdjoint>
 __global__ void __launch_bounds__(Q_BLOCK, Q_RESIDENT)
     k_shade(DevScene sc, DevFrame fr, DevParams P, Wave w, int cur, int depth, int last, int resident,
             const Job* __restrict__ jobs) {
     __shared__ uint16_t keys[Q_TILE];
     __shared__ uint16_t order[Q_TILE];  // the tile's entries, misses first
     __shared__ int n_miss, n_hit;
+    __shared__ double emit[EMIT_SLOTS];
     __shared__ int cnt[2][KEY_CELLS];   // next rays, shadow rays
     const int32_t n = *(volatile int32_t*)(w.counters + cur);
     const int32_t* list = depth > 0 ? w.list[cur] : nullptr;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (blockIdx.x == 0 && tid == 0) w.counters[20] = 0;   // the next traversal's cursor
     // a small queue is cut into smaller tiles, so that every resident block has one
+    if (kAdjoint && tid < EMIT_SLOTS) emit[tid] = 0.0;     // (synchronised by the first tile)
     const int step = resident * Q_BLOCK;
     const int items = max(1, min(Q_ITEMS, (n + step - 1) / step));
     for (int64_t t0 = (int64_t)blockIdx.x * items * Q_BLOCK; t0 < n; t0 += (int64_t)gridDim.x * items * Q_BLOCK) {
@@ -417,9 +491,15 @@ __global__ void __launch_bounds__(Q_BLOCK, Q_RESIDENT)
         for (int k = 0; k < items; ++k) {
             int e = k * Q_BLOCK + tid;
             uint32_t key = KEY_NONE | (KEY_NONE << 8);
+            VertexGrad vg{-1, -1, 0.0f, 0.0f};
             if (e < size) {
                 if (split) e = order[e];
-                key = shade_path<kBatch>(sc, fr, P, w, list ? __ldg(list + t0 + e) : (int)(t0 + e), depth, jobs);
+                key = shade_path<kBatch, kAdjoint>(sc, fr, P, w, list ? __ldg(list + t0 + e) : (int)(t0 + e), depth, jobs, vg);
+            }
+            if (kAdjoint) {
+                __syncwarp();
+                if (P.grad_emit) warp_add_emit(emit, P.grad_emit, vg.mat, (double)vg.emit);
+                if (P.grad_tex) warp_add_tex(P.grad_tex, vg.texel, vg.tex);
             }
             keys[e] = (uint16_t)key;
             if ((key & 0xFFu) != KEY_NONE) atomicAdd(&cnt[0][key & 0xFFu], 1);
@@ -451,27 +531,13 @@ __global__ void __launch_bounds__(Q_BLOCK, Q_RESIDENT)
         }
         __syncthreads();
     }
-}
-
-// ------------------------------------------------------------------ traversal
-// grad_emit[m] += v for the lanes with m >= 0 (the whole warp calls): one
-// atomic per material and warp.  The shadow rays of a warp go the same way, so
-// most of them sample one light, and their FP64 atomics on its word would
-// serialise.
-__device__ __forceinline__ void warp_add_emit(double* grad_emit, int m, double v) {
-    const unsigned full = 0xffffffffu;
-    unsigned todo = __ballot_sync(full, m >= 0);
-    while (todo) {
-        const int lead = __ffs(todo) - 1;
-        const int mm = __shfl_sync(full, m, lead);
-        double x = m == mm ? v : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(full, x, o);
-        if ((int)(threadIdx.x & 31) == lead) atomicAdd(grad_emit + mm, x);
-        todo &= ~__ballot_sync(full, m == mm);
+    if (kAdjoint && P.grad_emit && (int64_t)blockIdx.x * items * Q_BLOCK < n) {
+        __syncthreads();
+        if (tid < EMIT_SLOTS && emit[tid] != 0.0) atomicAdd(P.grad_emit + tid, emit[tid]);
     }
 }
 
+// ------------------------------------------------------------------ traversal
 // The groups of 32 consecutive queue entries that a warp of the traversal
 // kernel takes: first its own number, then the next of a device cursor, fetched
 // while the current group is traced.  Per-ray cost is heavy-tailed: a fixed
@@ -558,7 +624,7 @@ __device__ __forceinline__ int3 trace_queue(const DevScene& sc, const DevFrame& 
             }
             if (!kBatch && P.adjoint && P.grad_emit) {
                 const int m = lit ? w.sh_m[p] : -1;
-                warp_add_emit(P.grad_emit, m, m >= 0 ? (double)(w.delta[p] * w.sh_g[p]) : 0.0);
+                warp_add_emit(work_acc().emit, P.grad_emit, m, m >= 0 ? (double)(w.delta[p] * w.sh_g[p]) : 0.0);
             }
         }
         gr.advance();
@@ -600,7 +666,7 @@ __global__ void __launch_bounds__(MCEV_TRAV_BLOCK, trav_blocks(kWide, kTlas))
     if (scur >= 0)
         ws = trace_queue<true, kBatch, kWide, kTlas>(sc, fr, P, w, w.sh_list, nullptr, ns, gr, ge, gr.total, stack, err,
                                                        jobs);
-    add_work(w, wc, ws);
+    add_work(w, wc, ws, !kBatch && P.adjoint ? P.grad_emit : nullptr);
 }
 
 // ------------------------------------------------------------------ per-pixel statistics + test + requeue + events
@@ -870,9 +936,11 @@ cudaError_t launch_shade(const DevScene& sc, const DevFrame& fr, const DevParams
     const int resident = sms * Q_RESIDENT;
     const int grid = grid_for(max_n, Q_BLOCK, sms, 4 * Q_RESIDENT);
     if (jobs)
-        k_shade<true><<<grid, Q_BLOCK, 0, st>>>(sc, fr, P, w, cur, depth, last ? 1 : 0, resident, jobs);
+        k_shade<true, false><<<grid, Q_BLOCK, 0, st>>>(sc, fr, P, w, cur, depth, last ? 1 : 0, resident, jobs);
+    else if (P.adjoint)
+        k_shade<false, true><<<grid, Q_BLOCK, 0, st>>>(sc, fr, P, w, cur, depth, last ? 1 : 0, resident, nullptr);
     else
-        k_shade<false><<<grid, Q_BLOCK, 0, st>>>(sc, fr, P, w, cur, depth, last ? 1 : 0, resident, nullptr);
+        k_shade<false, false><<<grid, Q_BLOCK, 0, st>>>(sc, fr, P, w, cur, depth, last ? 1 : 0, resident, nullptr);
     return cudaGetLastError();
 }
 
