@@ -167,10 +167,10 @@ struct QGrid {
     int64_t n_words;      // per mask
 };
 constexpr int QNEAR = 15;     // columns of the first search's window
-constexpr int QRINGS = 2;      // its rings (whole call on 1280x720x100 at 1 / 2 / 3 / 5: 0.80 / 0.81 / 0.89 / 1.14 ms)
-// cells of the far search: 32 columns (a mask word) x 8 rows x 4 frames, so that
-// a warp reads a cell's 32 rows at once
-constexpr int QCELL_Y = 8, QCELL_T = 4;
+constexpr int QRINGS = 2;      // its rings (a 1280x720x100 call at 1 / 2 / 3 / 5 rings: 0.80 / 0.81 / 0.89 / 1.14 ms)
+// cells of the far search: 32 columns (a mask word) x 8 rows x 8 frames; a warp
+// reads a cell row's 64 rows two per lane
+constexpr int QCELL = 8;
 __device__ __forceinline__ int set_target(int set) { return set ^ 2; }   // the other video, same polarity
 
 // squared column distance from x to the nearest set bit of the row within
@@ -269,6 +269,7 @@ __global__ void __launch_bounds__(32 * QWARPS) k_search(QGrid G, const uint32_t*
             if (d2)
                 for (; same; same &= same - 1) d2[vox + __ffs(same) - 1] = 0;
             if (lacks[s]) q = 0;
+            if (!__any_sync(0xffffffffu, q != 0)) continue;
             const int k = __popc(q);
             int v = k;
 #pragma unroll
@@ -338,7 +339,7 @@ __global__ void __launch_bounds__(QBLOCK) k_cells(QGrid G, const uint32_t* __res
                                                   uint32_t* __restrict__ cells, const unsigned long long* acc) {
     if (acc[QACC_FAR] == 0) return;
     const int lane = threadIdx.x & 31;
-    const int sw = (G.ww + 31) / 32, cy_n = (G.H + QCELL_Y - 1) / QCELL_Y, ct_n = (G.T + QCELL_T - 1) / QCELL_T;
+    const int sw = (G.ww + 31) / 32, cy_n = (G.H + QCELL - 1) / QCELL, ct_n = (G.T + QCELL - 1) / QCELL;
     const int64_t per_set = (int64_t)cy_n * ct_n * sw, n = QSETS * per_set;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += nw) {
@@ -348,8 +349,8 @@ __global__ void __launch_bounds__(QBLOCK) k_cells(QGrid G, const uint32_t* __res
         uint32_t any = 0;
         if (word < G.ww) {
 #pragma unroll
-            for (int j = 0; j < QCELL_Y * QCELL_T; ++j) {
-                const int t = ct * QCELL_T + j / QCELL_Y, y = cy * QCELL_Y + j % QCELL_Y;
+            for (int j = 0; j < QCELL * QCELL; ++j) {
+                const int t = ct * QCELL + j / QCELL, y = cy * QCELL + j % QCELL;
                 if (t < G.T && y < G.H) any |= __ldg(masks + set * G.n_words + ((int64_t)t * G.H + y) * G.ww + word);
             }
         }
@@ -382,11 +383,13 @@ __device__ __forceinline__ int32_t cells_near(const uint32_t* __restrict__ row, 
 }
 
 // The listed events, one warp each.  The warp's lanes look at the cell rows of a
-// ring around the event (ring r is at least 4 (r - 1) + 1 frames or rows away);
-// of those that could hold a nearer event the nearest is searched first, its
-// 32 rows one per lane.  Bound by the dependent loads of one event after the
-// other (482 us on 1280x720x100, with the two videos' spurious events); the exact
-// transform of the four sets took 8.3 ms there.
+// ring around the event (ring r is at least 8 (r - 1) + 1 frames or rows away);
+// an occupied cell bounds the distance from above and below, and of those that
+// could hold a nearer event the nearest is searched first, its 64 rows two per
+// lane.  Bound by the dependent loads of one event after the
+// other and some 4000 instructions each (477 us on 1280x720x100 with 60,000 of them;
+// cells of 4 frames and no bound from above 482 us); the exact transform of the four
+// sets took 8.3 ms there.
 __global__ void __launch_bounds__(QBLOCK) k_search_far(QGrid G, const uint32_t* __restrict__ masks,
                                                        const uint32_t* __restrict__ cells, int tau2,
                                                        int32_t* __restrict__ d2_a, int32_t* __restrict__ d2_b,
@@ -397,7 +400,7 @@ __global__ void __launch_bounds__(QBLOCK) k_search_far(QGrid G, const uint32_t* 
     const int64_t n = (int64_t)acc[QACC_FAR];
     // too many for the list: the sets with open events are matched by the transform
     if (n > far_cap) return;
-    const int sw = (G.ww + 31) / 32, cy_n = (G.H + QCELL_Y - 1) / QCELL_Y, ct_n = (G.T + QCELL_T - 1) / QCELL_T;
+    const int sw = (G.ww + 31) / 32, cy_n = (G.H + QCELL - 1) / QCELL, ct_n = (G.T + QCELL - 1) / QCELL;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += nw) {
         const uint64_t id = far_list[k];
@@ -408,16 +411,17 @@ __global__ void __launch_bounds__(QBLOCK) k_search_far(QGrid G, const uint32_t* 
         const int t = (int)(row / G.H), y = (int)(row - (int64_t)t * G.H);
         const uint32_t* M = masks + set_target(s) * G.n_words;
         const uint32_t* C = cells + (int64_t)set_target(s) * cy_n * ct_n * sw;
-        const int cy0 = y / QCELL_Y, ct0 = t / QCELL_T;
+        const int cy0 = y / QCELL, ct0 = t / QCELL;
         const int r_end = max(max(cy0, cy_n - 1 - cy0), max(ct0, ct_n - 1 - ct0));
         int32_t best = QINF;
         for (int r = 0; r <= r_end; ++r) {
-            const int ring = QCELL_T * (r - 1) + 1;
+            const int ring = QCELL * (r - 1) + 1;
             if (r > 0 && ring * ring >= best) break;
             const int rows = r == 0 ? 1 : 8 * r;
             for (int j0 = 0; j0 < rows; j0 += 32) {
                 const int j = j0 + lane;
-                int32_t bound = QINF;      // no event of this lane's cell row is nearer
+                int32_t bound = QINF;      // no event of this lane's cell row is nearer,
+                int32_t within = QINF;     // and one of them is nearer than this
                 int cy = 0, ct = 0;
                 if (j < rows) {
                     // two full sides of 2r + 1 cell rows, then pairs
@@ -431,26 +435,36 @@ __global__ void __launch_bounds__(QBLOCK) k_search_far(QGrid G, const uint32_t* 
                         cy = cy0 + ((p & 1) ? r : -r);
                     }
                     if (cy >= 0 && cy < cy_n && ct >= 0 && ct < ct_n) {
-                        const int dy = max(0, max(cy * QCELL_Y - y, y - (cy * QCELL_Y + QCELL_Y - 1)));
-                        const int dt = max(0, max(ct * QCELL_T - t, t - (ct * QCELL_T + QCELL_T - 1)));
+                        const int dy = max(0, max(cy * QCELL - y, y - (cy * QCELL + QCELL - 1)));
+                        const int dt = max(0, max(ct * QCELL - t, t - (ct * QCELL + QCELL - 1)));
                         const int32_t d = dy * dy + dt * dt;
                         if (d < best) {
                             const int32_t dx = cells_near(C + ((int64_t)ct * cy_n + cy) * sw, sw, x);
-                            if (dx < QINF) bound = d + dx * dx;
+                            if (dx < QINF) {
+                                const int uy = max(abs(cy * QCELL - y), abs(cy * QCELL + QCELL - 1 - y));
+                                const int ut = max(abs(ct * QCELL - t), abs(ct * QCELL + QCELL - 1 - t));
+                                bound = d + dx * dx;
+                                within = uy * uy + ut * ut + (dx + 31) * (dx + 31) + 1;
+                            }
                         }
                     }
                 }
+                best = min(best, __reduce_min_sync(full, within));
                 while (true) {
                     const int32_t first = __reduce_min_sync(full, bound);
                     if (first >= best) break;
                     const int src = __ffs(__ballot_sync(full, bound == first)) - 1;
-                    const int yy = __shfl_sync(full, cy, src) * QCELL_Y + (lane & (QCELL_Y - 1));
-                    const int tt = __shfl_sync(full, ct, src) * QCELL_T + lane / QCELL_Y;
+                    const int yy = __shfl_sync(full, cy, src) * QCELL + (lane & (QCELL - 1));
+                    const int tt0 = __shfl_sync(full, ct, src) * QCELL + lane / QCELL;
                     if (lane == src) bound = QINF;
-                    const int32_t d = (yy - y) * (yy - y) + (tt - t) * (tt - t);
                     int32_t got = best;
-                    if (yy < G.H && tt < G.T && d < best)
-                        got = row_wide(M + ((int64_t)tt * G.H + yy) * G.ww, G.ww, x, best - d) + d;
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        const int tt = tt0 + half * (QCELL / 2);
+                        const int32_t d = (yy - y) * (yy - y) + (tt - t) * (tt - t);
+                        if (yy < G.H && tt < G.T && d < got)
+                            got = row_wide(M + ((int64_t)tt * G.H + yy) * G.ww, G.ww, x, got - d) + d;
+                    }
                     best = min(best, __reduce_min_sync(full, got));
                 }
             }
@@ -684,7 +698,7 @@ int64_t quality_mask_bytes(int32_t W, int32_t H, int32_t T) {
 
 int64_t quality_cell_bytes(int32_t W, int32_t H, int32_t T) {
     const int64_t sw = ((W + 31) / 32 + 31) / 32;
-    return 4 * QSETS * sw * ((H + QCELL_Y - 1) / QCELL_Y) * ((T + QCELL_T - 1) / QCELL_T);
+    return 4 * QSETS * sw * ((H + QCELL - 1) / QCELL) * ((T + QCELL - 1) / QCELL);
 }
 
 // Far events the list holds; more of them are cheaper to settle by the exact
