@@ -671,7 +671,8 @@ __device__ __forceinline__ TRay object_tray(const DevFrame& fr, int rec, const f
     const float4* ip = fr.inst + 7 * rec;
     const float4 i0 = __ldg(ip + 3), i1 = __ldg(ip + 4), i2 = __ldg(ip + 5);
     root = __float_as_int(__ldg(ip + 6).x);
-    const f3 o = xyz(*op), d = xyz(*dp);
+    // (streaming loads: the ray queues are larger than L2, the nodes are worth keeping)
+    const f3 o = xyz(__ldcs(op)), d = xyz(__ldcs(dp));
     return make_tray(xf_point(i0, i1, i2, o), xf_vec(i0, i1, i2, d));
 }
 

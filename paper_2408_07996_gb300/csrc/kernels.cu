@@ -612,7 +612,7 @@ __device__ __forceinline__ int3 trace_queue(const DevScene& sc, const DevFrame& 
         }
         if (!kAny) {
             if (live) {
-                w.hit[p] = make_float2(h.t, __int_as_float(h.tri));
+                __stcs(w.hit + p, make_float2(h.t, __int_as_float(h.tri)));
                 if (F.n_inst > 1) w.hit_rec[p] = h.rec;
             }
         } else {
