@@ -720,7 +720,12 @@ __device__ __forceinline__ void two_level(const DevScene& sc, const DevFrame& fr
                 base = sp;
             }
         }
-        if (pcount == 0 && node != MCEV_NO_NODE) {
+#ifndef MCEV_TL_STEPS
+#define MCEV_TL_STEPS 2
+#endif
+#pragma unroll
+        for (int step = 0; step < MCEV_TL_STEPS; ++step) {
+        if (pcount == 0 && node != MCEV_NO_NODE && (in_blas || pend0 < 0)) {
             const Node n = load_node(in_blas ? sc.nodes : fr.tlas, node);
             work.x += 1;
             float tl, tr;
@@ -745,6 +750,7 @@ __device__ __forceinline__ void two_level(const DevScene& sc, const DevFrame& fr
                 node = MCEV_NO_NODE;
                 if (in_blas ? sp > base : (sp > 0 && pend0 < 0)) node = stack[--sp];
             }
+        }
         }
         if (pcount > 0) {
             work.y += 1;

@@ -728,6 +728,7 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
     constexpr unsigned full = 0xffffffffu;
     constexpr int LANES = 4, PIX = 32 / LANES, LEAVES = 32 / LANES;
     const int lane = threadIdx.x & 31, q = lane & (LANES - 1);
+    const int test0 = A0.mode == MODE_DETECT ? (int)((A0.k_base - A0.spp_min) / A0.spp_batch) : 0;
     const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t jw = warp0 * PIX; jw < n_pix; jw += nwarps * PIX) {
@@ -759,6 +760,8 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
         int bad = 0;
         bool open = on;        // neither decided nor off
         int32_t n = (int32_t)c.n;
+        // number of the last test: spp_min + test * spp_batch samples
+        int test = A.k_base == 0 ? -1 : test0;
         const float* Lp = w.L + (on ? j : 0) * A.spp_r;
         for (int s0 = 0; s0 < A.spp_r && __any_sync(full, open); s0 += A.sub) {
             const int s1 = min(s0 + A.sub, A.spp_r);
@@ -774,10 +777,11 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
 #pragma unroll
             for (int m = 0; m < LEAVES; ++m) a1[m] = a2[m] = 0.0f;
             if (open) {
-                for (int b = s0 + q; b < s1; b += 32) {
+                for (int b = s0; b < s1; b += 32) {
 #pragma unroll
                     for (int m = 0; m < LEAVES; ++m) {
-                        const int s = b + LANES * m;
+                        if (b + LANES * m >= s1) break;     // the same for the whole warp
+                        const int s = b + LANES * m + q;
                         if (s < s1) {
                             float Lv = Lp[s];
                             if (!isfinite(Lv)) {
@@ -812,6 +816,7 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
             c = (A.k_base == 0 && s0 == 0) ? m : chan(c, m);
             n = (int32_t)c.n;
             if (!detect) continue;
+            ++test;
             bool decided = n >= A.spp_max;
             if (!decided && A.variant != VAR_UNIFORM) {
                 const float gap = fabsf(c.mean - ma);
@@ -826,8 +831,10 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
                         decided = false;
                     } else {
                         const float t = (gap - A.C) / sqrtf(se2);
-                        int r = (n - A.spp_min) / A.spp_batch;
-                        if (kChecked) r = min(r, (A.spp_max - A.spp_min + A.spp_batch - 1) / A.spp_batch - 1);
+                        int r = test;
+                        if (kChecked)      // by the caller's own counts
+                            r = min((n - A.spp_min) / A.spp_batch,
+                                    (A.spp_max - A.spp_min + A.spp_batch - 1) / A.spp_batch - 1);
                         const float tc = __ldg(A.tcrit + r);
                         decided = A.variant == VAR_TWO_TAILED ? (t < tc || t > -tc) : (t < tc);
                     }

@@ -387,7 +387,7 @@ __device__ __forceinline__ int32_t cells_near(const uint32_t* __restrict__ row, 
 // an occupied cell bounds the distance from above and below, and of those that
 // could hold a nearer event the nearest is searched first, its 64 rows two per
 // lane.  Bound by the dependent loads of one event after the
-// other and some 4000 instructions each (477 us on 1280x720x100 with 60,000 of them;
+// other and some 4000 instructions each (477 us on 1280x720x100;
 // cells of 4 frames and no bound from above 482 us); the exact transform of the four
 // sets took 8.3 ms there.
 __global__ void __launch_bounds__(QBLOCK) k_search_far(QGrid G, const uint32_t* __restrict__ masks,
