@@ -722,7 +722,7 @@ mcev_status ensure_wave(mcev_ctx* ctx) {
     // per path slot: ray_o, ray_d, sh_d; hit, pix_k; hit_rec, L, sig, pflags, sh_c, sh_g, sh_m, Ltot, delta;
     // queues: list (x2), sh_list
     const size_t per = 3 * 16 + 2 * 8 + 9 * 4 + 3 * 4;
-    ST(dev_alloc(ctx, ctx->d_wave, (size_t)cap * per + 64 * 256));
+    ST(dev_alloc(ctx, ctx->d_wave, (size_t)cap * per + (size_t)cap / 8 + 64 * 256));
     char* p = (char*)ctx->d_wave.ptr;
     auto take = [&](size_t bytes) {
         char* r = p;
@@ -743,6 +743,7 @@ mcev_status ensure_wave(mcev_ctx* ctx) {
     w.list[0] = (int32_t*)take(4 * cap);
     w.list[1] = (int32_t*)take(4 * cap);
     w.sh_list = (int32_t*)take(4 * cap);
+    w.again = (uint32_t*)take(4 * ((cap + 31) / 32));
     w.sh_c = (float*)take(4 * cap);
     w.sh_g = (float*)take(4 * cap);
     w.sh_m = (int32_t*)take(4 * cap);
@@ -914,7 +915,8 @@ mcev_status run_rounds_device(mcev_ctx* ctx, const Frame& fr, StatsArgs A, int64
         CU(cudaStreamBeginCaptureToGraph(cs, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
         ctx->stream = cs;
         mcev_status st = MCEV_OK;
-        cudaError_t e = launch_round_init(rc, ctx->wave, plan, queue[0], queue[1], B == nullptr, ctx->sms, cs);
+        cudaError_t e = launch_round_init(rc, ctx->wave, plan, queue[0], queue[1], B ? 0 : ctx->W, B ? 0 : ctx->H,
+                                              ctx->sms, cs);
         cudaGraphNode_t cond = nullptr;
         if (e == cudaSuccess) {
             cudaStreamCaptureStatus cst;
@@ -1024,7 +1026,7 @@ mcev_status run_rounds(mcev_ctx* ctx, const Frame& fr, StatsArgs A, int64_t* pat
         Q = B->q0;
     } else {
         Q = (int64_t)ctx->W * ctx->H;
-        LAUNCH(MCEV_K_STATS, launch_iota(queue[0], Q, ctx->sms, ctx->stream));
+        LAUNCH(MCEV_K_STATS, launch_pixel_queue(queue[0], ctx->W, ctx->H, ctx->sms, ctx->stream));
     }
     const Job* jobs = B ? B->d_jobs : nullptr;
     int64_t n_done = 0, paths = 0;
@@ -1054,6 +1056,7 @@ mcev_status run_rounds(mcev_ctx* ctx, const Frame& fr, StatsArgs A, int64_t* pat
             ST(trace_chunk(ctx, fr, P, queue[qi], j0, spp_r, n_done, nj * spp_r, B));
             LAUNCH(MCEV_K_STATS,
                    launch_stats(ctx->wave, A, queue[qi], j0, nj, queue[qi ^ 1], ctx->sms, ctx->stream, jobs, nullptr));
+            LAUNCH(MCEV_K_STATS, launch_requeue(ctx->wave, queue[qi], j0, nj, queue[qi ^ 1], ctx->stream));
             ctx->stats_pix += nj;
         }
         paths += Q * spp_r;
@@ -1510,7 +1513,7 @@ mcev_status mcev_backward(mcev_ctx* ctx, double t, int32_t spp, const float* gra
     reset_call_counters(ctx);
     ST(frame_setup(ctx, t, 0));
     const int64_t npix = (int64_t)ctx->W * ctx->H;
-    LAUNCH(MCEV_K_STATS, launch_iota(ctx->queue[0], npix, ctx->sms, ctx->stream));
+    LAUNCH(MCEV_K_STATS, launch_pixel_queue(ctx->queue[0], ctx->W, ctx->H, ctx->sms, ctx->stream));
     const DevParams P = dev_params(ctx, false);
     DevParams Padj = P;
     Padj.adjoint = 1;
@@ -1607,7 +1610,7 @@ mcev_status mcev_render_events_batch(mcev_ctx* runner, const mcev_job* jobs, int
             B.any_nee = B.any_nee || c->params.nee != 0;
             B.any_tlas = B.any_tlas || J.fr.n_tlas >= 2;
             const int64_t np = (int64_t)c->W * c->H;
-            LAUNCH(MCEV_K_STATS, launch_fill_entries(B.queue[0] + B.q0, np, (int)q, ctx->sms, ctx->stream));
+            LAUNCH(MCEV_K_STATS, launch_fill_entries(B.queue[0] + B.q0, c->W, c->H, (int)q, ctx->sms, ctx->stream));
             B.q0 += np;
         }
         CU(cudaMemcpyAsync(ctx->d_jobs.ptr, tab.data(), sizeof(Job) * tab.size(), cudaMemcpyHostToDevice, ctx->stream));

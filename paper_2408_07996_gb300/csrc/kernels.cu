@@ -729,163 +729,232 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
     constexpr int LANES = 4, PIX = 32 / LANES, LEAVES = 32 / LANES;
     const int lane = threadIdx.x & 31, q = lane & (LANES - 1);
     const int test0 = A0.mode == MODE_DETECT ? (int)((A0.k_base - A0.spp_min) / A0.spp_batch) : 0;
-    const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t jw = warp0 * PIX; jw < n_pix; jw += nwarps * PIX) {
-        const int64_t j = jw + lane / LANES;
-        bool on = j < n_pix;
-        const int32_t entry = on ? __ldg(queue + j0 + j) : 0;
-        const int32_t pix = kBatch ? (entry & 0xFFFFFF) : entry;
-        // per-pixel state and outputs of the pixel's job
-        StatsArgs A = A0;
-        if (kBatch && on) {
-            const Job& J = jobs[(uint32_t)entry >> 24];
-            A.cur = J.cur;
-            A.ref = J.ref;
-            A.events = J.events;
-            A.spp_out = J.spp_out;
-            A.mean_out = J.mean_out;
-            A.eps = J.P.eps;
-        }
-        if (kChecked && on && (pix < 0 || (int64_t)pix >= A.n_total)) {
-            if (q == 0) atomicOr(w.counters + 8, 1);
-            on = false;
-        }
-        Moments c{0.0f, 0.0f, 0.0f};
-        if (on && A.k_base > 0) c = Moments{(float)A.cur.n[pix], A.cur.mean[pix], A.cur.m2[pix]};
-        const bool detect = A.mode == MODE_DETECT;
-        const float ma = detect && on ? A.ref.mean[pix] : 0.0f;
-        const int32_t na = detect && on ? A.ref.n[pix] : 0;
-        const float va = (detect && na > 1) ? A.ref.m2[pix] / (float)(na - 1) : 0.0f;
-        int bad = 0;
-        bool open = on;        // neither decided nor off
-        int32_t n = (int32_t)c.n;
-        // number of the last test: spp_min + test * spp_batch samples
-        int test = A.k_base == 0 ? -1 : test0;
-        const float* Lp = w.L + (on ? j : 0) * A.spp_r;
-        for (int s0 = 0; s0 < A.spp_r && __any_sync(full, open); s0 += A.sub) {
-            const int s1 = min(s0 + A.sub, A.spp_r);
-            // moments of this batch from sums shifted by one value (the running
-            // mean, or the batch's first sample for a pixel's first batch), so
-            // lanes merge by plain addition
-            float sh = c.mean;
-            if (open && !(c.n > 0.0f)) {
-                const float L0 = Lp[s0];
-                sh = MCEV_LOG((isfinite(L0) ? L0 : 0.0f) + A.eps);
+    // a block's tile: up to 8 steps of 64 pixels, fewer when there are few pixels
+    constexpr int STEP = 256 / LANES, STEPS = 8;
+    __shared__ uint32_t again_bits[STEP * STEPS / 32];
+    __shared__ int again_at;
+    const int64_t per_step = (int64_t)gridDim.x * STEP;
+    const int steps = (int)max((int64_t)1, min((int64_t)STEPS, n_pix / per_step));
+    for (int64_t t0 = (int64_t)blockIdx.x * steps * STEP; t0 < n_pix; t0 += per_step * steps) {
+        if (threadIdx.x < STEP * STEPS / 32) again_bits[threadIdx.x] = 0;
+        __syncthreads();
+        for (int it = 0; it < steps; ++it) {
+            const int in_tile = it * STEP + (threadIdx.x >> 5) * PIX + lane / LANES;
+            const int64_t j = t0 + in_tile;
+            bool on = j < n_pix;
+            const int32_t entry = on ? __ldg(queue + j0 + j) : 0;
+            const int32_t pix = kBatch ? (entry & 0xFFFFFF) : entry;
+            // per-pixel state and outputs of the pixel's job
+            StatsArgs A = A0;
+            if (kBatch && on) {
+                const Job& J = jobs[(uint32_t)entry >> 24];
+                A.cur = J.cur;
+                A.ref = J.ref;
+                A.events = J.events;
+                A.spp_out = J.spp_out;
+                A.mean_out = J.mean_out;
+                A.eps = J.P.eps;
             }
-            float a1[LEAVES], a2[LEAVES];
-#pragma unroll
-            for (int m = 0; m < LEAVES; ++m) a1[m] = a2[m] = 0.0f;
-            if (open) {
-                for (int b = s0; b < s1; b += 32) {
-#pragma unroll
-                    for (int m = 0; m < LEAVES; ++m) {
-                        if (b + LANES * m >= s1) break;     // the same for the whole warp
-                        const int s = b + LANES * m + q;
-                        if (s < s1) {
-                            float Lv = Lp[s];
-                            if (!isfinite(Lv)) {
-                                Lv = 0.0f;
-                                ++bad;
+            if (kChecked && on && (pix < 0 || (int64_t)pix >= A.n_total)) {
+                if (q == 0) atomicOr(w.counters + 8, 1);
+                on = false;
+            }
+            Moments c{0.0f, 0.0f, 0.0f};
+            if (on && A.k_base > 0) c = Moments{(float)A.cur.n[pix], A.cur.mean[pix], A.cur.m2[pix]};
+            const bool detect = A.mode == MODE_DETECT;
+            const float ma = detect && on ? A.ref.mean[pix] : 0.0f;
+            const int32_t na = detect && on ? A.ref.n[pix] : 0;
+            const float va = (detect && na > 1) ? A.ref.m2[pix] / (float)(na - 1) : 0.0f;
+            int bad = 0;
+            bool open = on;        // neither decided nor off
+            int32_t n = (int32_t)c.n;
+            // number of the last test: spp_min + test * spp_batch samples
+            int test = A.k_base == 0 ? -1 : test0;
+            const float* Lp = w.L + (on ? j : 0) * A.spp_r;
+            for (int s0 = 0; s0 < A.spp_r && __any_sync(full, open); s0 += A.sub) {
+                const int s1 = min(s0 + A.sub, A.spp_r);
+                // moments of this batch from sums shifted by one value (the running
+                // mean, or the batch's first sample for a pixel's first batch), so
+                // lanes merge by plain addition
+                float sh = c.mean;
+                if (open && !(c.n > 0.0f)) {
+                    const float L0 = Lp[s0];
+                    sh = MCEV_LOG((isfinite(L0) ? L0 : 0.0f) + A.eps);
+                }
+                float a1[LEAVES], a2[LEAVES];
+    #pragma unroll
+                for (int m = 0; m < LEAVES; ++m) a1[m] = a2[m] = 0.0f;
+                if (open) {
+                    for (int b = s0; b < s1; b += 32) {
+    #pragma unroll
+                        for (int m = 0; m < LEAVES; ++m) {
+                            if (b + LANES * m >= s1) break;     // the same for the whole warp
+                            const int s = b + LANES * m + q;
+                            if (s < s1) {
+                                float Lv = Lp[s];
+                                if (!isfinite(Lv)) {
+                                    Lv = 0.0f;
+                                    ++bad;
+                                }
+                                const float d = MCEV_LOG(Lv + A.eps) - sh;
+                                a1[m] += d;
+                                a2[m] = fmaf(d, d, a2[m]);
                             }
-                            const float d = MCEV_LOG(Lv + A.eps) - sh;
-                            a1[m] += d;
-                            a2[m] = fmaf(d, d, a2[m]);
                         }
                     }
                 }
-            }
-#pragma unroll
-            for (int h = LEAVES / 2; h > 0; h >>= 1) {
-#pragma unroll
-                for (int m = 0; m < h; ++m) {
-                    a1[m] += a1[m + h];
-                    a2[m] += a2[m + h];
-                }
-            }
-            float s1d = a1[0], s2d = a2[0];
-#pragma unroll
-            for (int off = LANES / 2; off > 0; off >>= 1) {
-                s1d += __shfl_xor_sync(full, s1d, off);
-                s2d += __shfl_xor_sync(full, s2d, off);
-            }
-            if (!open) continue;
-            const float fn = (float)(s1 - s0);
-            const float md = s1d / fn;
-            const Moments m{fn, sh + md, fmaxf(s2d - s1d * md, 0.0f)};
-            c = (A.k_base == 0 && s0 == 0) ? m : chan(c, m);
-            n = (int32_t)c.n;
-            if (!detect) continue;
-            ++test;
-            bool decided = n >= A.spp_max;
-            if (!decided && A.variant != VAR_UNIFORM) {
-                const float gap = fabsf(c.mean - ma);
-                if (A.variant == VAR_MEAN_ONLY) {
-                    decided = gap < A.C;
-                } else {
-                    const float vb = c.m2 / (float)(n - 1);
-                    const float se2 = A.se_mode == SE_WELCH ? va / (float)na + vb / (float)n : (va + vb) / (float)n;
-                    if (se2 == 0.0f) {
-                        decided = gap < A.C;
-                    } else if (kChecked && n < A.spp_min) {
-                        decided = false;
-                    } else {
-                        const float t = (gap - A.C) / sqrtf(se2);
-                        int r = test;
-                        if (kChecked)      // by the caller's own counts
-                            r = min((n - A.spp_min) / A.spp_batch,
-                                    (A.spp_max - A.spp_min + A.spp_batch - 1) / A.spp_batch - 1);
-                        const float tc = __ldg(A.tcrit + r);
-                        decided = A.variant == VAR_TWO_TAILED ? (t < tc || t > -tc) : (t < tc);
+    #pragma unroll
+                for (int h = LEAVES / 2; h > 0; h >>= 1) {
+    #pragma unroll
+                    for (int m = 0; m < h; ++m) {
+                        a1[m] += a1[m + h];
+                        a2[m] += a2[m + h];
                     }
                 }
+                float s1d = a1[0], s2d = a2[0];
+    #pragma unroll
+                for (int off = LANES / 2; off > 0; off >>= 1) {
+                    s1d += __shfl_xor_sync(full, s1d, off);
+                    s2d += __shfl_xor_sync(full, s2d, off);
+                }
+                if (!open) continue;
+                const float fn = (float)(s1 - s0);
+                const float md = s1d / fn;
+                const Moments m{fn, sh + md, fmaxf(s2d - s1d * md, 0.0f)};
+                c = (A.k_base == 0 && s0 == 0) ? m : chan(c, m);
+                n = (int32_t)c.n;
+                if (!detect) continue;
+                ++test;
+                bool decided = n >= A.spp_max;
+                if (!decided && A.variant != VAR_UNIFORM) {
+                    const float gap = fabsf(c.mean - ma);
+                    if (A.variant == VAR_MEAN_ONLY) {
+                        decided = gap < A.C;
+                    } else {
+                        const float vb = c.m2 / (float)(n - 1);
+                        const float se2 = A.se_mode == SE_WELCH ? va / (float)na + vb / (float)n : (va + vb) / (float)n;
+                        if (se2 == 0.0f) {
+                            decided = gap < A.C;
+                        } else if (kChecked && n < A.spp_min) {
+                            decided = false;
+                        } else {
+                            const float t = (gap - A.C) / sqrtf(se2);
+                            int r = test;
+                            if (kChecked)      // by the caller's own counts
+                                r = min((n - A.spp_min) / A.spp_batch,
+                                        (A.spp_max - A.spp_min + A.spp_batch - 1) / A.spp_batch - 1);
+                            const float tc = __ldg(A.tcrit + r);
+                            decided = A.variant == VAR_TWO_TAILED ? (t < tc || t > -tc) : (t < tc);
+                        }
+                    }
+                }
+                open = !decided;
             }
-            open = !decided;
-        }
-#pragma unroll
-        for (int off = LANES / 2; off > 0; off >>= 1) bad += __shfl_xor_sync(full, bad, off);
-        // the pixel's first lane writes it back; undecided pixels go on in queue order
-        const bool own = on && q == 0;
-        const bool again = own && (detect ? open : n < A.spp_max);
-        const unsigned more = __ballot_sync(full, again);
-        int at = 0;
-        if (lane == 0 && more) at = atomicAdd(w.counters + 3, __popc(more));
-        at = __shfl_sync(full, at, 0);
-        if (!own) continue;
-        if (bad) atomicAdd(w.counters + 4, bad);
-        A.cur.n[pix] = n;
-        A.cur.mean[pix] = c.mean;
-        A.cur.m2[pix] = c.m2;
-        if (again) {
-            next_queue[at + __popc(more & ((1u << lane) - 1u))] = entry;
-            continue;
-        }
-        if (!detect) {
-            if (A.mode == MODE_MEAN) {
-                A.mean_out[pix] = c.mean;
-                if (A.spp_out) A.spp_out[pix] = n;
-            } else {
+    #pragma unroll
+            for (int off = LANES / 2; off > 0; off >>= 1) bad += __shfl_xor_sync(full, bad, off);
+            // the pixel's first lane writes it back
+            const bool own = on && q == 0;
+            const bool again = own && (detect ? open : n < A.spp_max);
+            if (again) atomicOr(&again_bits[in_tile >> 5], 1u << (in_tile & 31));
+            if (!own) continue;
+            if (bad) atomicAdd(w.counters + 4, bad);
+            A.cur.n[pix] = n;
+            A.cur.mean[pix] = c.mean;
+            A.cur.m2[pix] = c.m2;
+            if (again) continue;
+            if (!detect) {
+                if (A.mode == MODE_MEAN) {
+                    A.mean_out[pix] = c.mean;
+                    if (A.spp_out) A.spp_out[pix] = n;
+                } else {
+                    A.ref.n[pix] = n;
+                    A.ref.mean[pix] = c.mean;
+                    A.ref.m2[pix] = c.m2;
+                }
+                continue;
+            }
+            const float delta = c.mean - ma;
+            int8_t ev = 0;
+            if (fabsf(delta) > A.C) {
+                ev = delta > 0.0f ? 1 : -1;
                 A.ref.n[pix] = n;
                 A.ref.mean[pix] = c.mean;
                 A.ref.m2[pix] = c.m2;
+                atomicAdd(w.counters + (ev > 0 ? 5 : 6), 1);
             }
+            if (n >= A.spp_max) atomicAdd(w.counters + 7, 1);
+            atomicAdd(reinterpret_cast<unsigned long long*>(w.counters + 32) + 6, (unsigned long long)n);
+            A.events[pix] = ev;
+            if (A.spp_out) A.spp_out[pix] = n;
+            if (A.mean_out) A.mean_out[pix] = c.mean;
+        }
+        __syncthreads();
+        if (!kChecked) {
+            // requeue() queues them
+            const int64_t word = (t0 >> 5) + threadIdx.x;
+            if (threadIdx.x < steps * STEP / 32 && word < (n_pix + 31) >> 5) w.again[word] = again_bits[threadIdx.x];
+            __syncthreads();
             continue;
         }
-        const float delta = c.mean - ma;
-        int8_t ev = 0;
-        if (fabsf(delta) > A.C) {
-            ev = delta > 0.0f ? 1 : -1;
-            A.ref.n[pix] = n;
-            A.ref.mean[pix] = c.mean;
-            A.ref.m2[pix] = c.m2;
-            atomicAdd(w.counters + (ev > 0 ? 5 : 6), 1);
+        // the allocation-free step lists its tile's undecided pixels itself (any order of tiles)
+        if (threadIdx.x < 32) {
+            const uint32_t bits = lane < STEP * STEPS / 32 ? again_bits[lane] : 0u;
+            const int total = __reduce_add_sync(full, __popc(bits));
+            if (lane == 0 && total) again_at = atomicAdd(w.counters + 3, total);
         }
-        if (n >= A.spp_max) atomicAdd(w.counters + 7, 1);
-        atomicAdd(reinterpret_cast<unsigned long long*>(w.counters + 32) + 6, (unsigned long long)n);
-        A.events[pix] = ev;
-        if (A.spp_out) A.spp_out[pix] = n;
-        if (A.mean_out) A.mean_out[pix] = c.mean;
+        __syncthreads();
+        for (int i = threadIdx.x; i < steps * STEP; i += blockDim.x) {
+            const uint32_t bits = again_bits[i >> 5];
+            if (!(bits >> (i & 31) & 1u)) continue;
+            int at = again_at + __popc(bits & ((1u << (i & 31)) - 1u));
+            for (int k = 0; k < i >> 5; ++k) at += __popc(again_bits[k]);
+            next_queue[at] = __ldg(queue + j0 + t0 + i);
+        }
+        __syncthreads();
     }
+}
+
+// Appends a chunk's undecided pixels (w.again, one bit per entry) to the next
+// round's queue in their order, by one block.  Neighbours in the image stay
+// neighbours in the queue from round to round, so that their paths keep meeting
+// in the same traversal warps.  Appended warp by warp (eight pixels at a time) as
+// warps finished, a terrain 720p frame took 727 ms, a sphere-field frame 190 ms and
+// eight jobs 121.7 ms; by tiles of 64 to 512 pixels 713, 187.0 and 110.9 ms; with
+// the first queue in image tiles (tiled_pixel) 709, 186.7 and 109.4 ms; in full order
+// 695, 183.2 and 108.7 ms.
+constexpr int REQUEUE_BLOCK = 1024;
+__device__ __forceinline__ void requeue(const Wave& w, const int32_t* __restrict__ queue, int64_t j0, int64_t n_pix,
+                                        int32_t* __restrict__ next_queue) {
+    __shared__ int sums[REQUEUE_BLOCK / 32];
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t words = (n_pix + 31) >> 5;
+    int at = *(volatile int32_t*)(w.counters + 3);
+    for (int64_t t0 = 0; t0 < words; t0 += REQUEUE_BLOCK) {
+        const int64_t k = t0 + threadIdx.x;
+        uint32_t bits = k < words ? w.again[k] : 0u;
+        const int c = __popc(bits);
+        int v = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(full, v, o);
+            if (lane >= o) v += y;
+        }
+        if (lane == 31) sums[wid] = v;
+        __syncthreads();
+        const int s = sums[lane];
+        const int before = __reduce_add_sync(full, lane < wid ? s : 0), total = __reduce_add_sync(full, s);
+        int to = at + before + v - c;
+        for (; bits; bits &= bits - 1) next_queue[to++] = __ldg(queue + j0 + 32 * k + __ffs(bits) - 1);
+        at += total;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *(volatile int32_t*)(w.counters + 3) = at;
+}
+
+__global__ void __launch_bounds__(REQUEUE_BLOCK) k_requeue(Wave w, const int32_t* queue, int64_t j0, int64_t n_pix,
+                                                           int32_t* next_queue) {
+    requeue(w, queue, j0, n_pix, next_queue);
 }
 
 // ------------------------------------------------------------------ tracePaths output
@@ -902,9 +971,25 @@ __global__ void k_write_samples(Wave w, int64_t out0, int64_t n_paths, float* __
     }
 }
 
-__global__ void k_iota(int32_t* q, int64_t n) {
+// Pixel at place i of the order that a frame's queue starts in: tiles of 16 x 16
+// pixels, row by row within each.
+constexpr int PIXEL_TILE = 16;
+__device__ __forceinline__ int32_t tiled_pixel(int64_t i, int W, int H) {
+    const int64_t band_size = (int64_t)PIXEL_TILE * W;
+    const int band = (int)(i / band_size);
+    const int bh = min(PIXEL_TILE, H - band * PIXEL_TILE);       // rows of the band
+    const int in_band = (int)(i - band * band_size);
+    const int tile = in_band / (PIXEL_TILE * bh);
+    const int x0 = tile * PIXEL_TILE, tw = min(PIXEL_TILE, W - x0);
+    const int in_tile = in_band - tile * (PIXEL_TILE * bh);
+    const int y = in_tile / tw;
+    return (band * PIXEL_TILE + y) * W + x0 + (in_tile - y * tw);
+}
+
+__global__ void k_pixel_queue(int32_t* q, int W, int H) {
+    const int64_t n = (int64_t)W * H;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        q[i] = (int32_t)i;
+        q[i] = tiled_pixel(i, W, H);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -963,6 +1048,12 @@ cudaError_t launch_stats(const Wave& w, const StatsArgs& A, const int32_t* queue
     return cudaGetLastError();
 }
 
+cudaError_t launch_requeue(const Wave& w, const int32_t* queue, int64_t j0, int64_t n_pix, int32_t* next_queue,
+                           cudaStream_t st) {
+    k_requeue<<<1, REQUEUE_BLOCK, 0, st>>>(w, queue, j0, n_pix, next_queue);
+    return cudaGetLastError();
+}
+
 static cudaError_t launch_stats_checked(const Wave& w, const StatsArgs& A, const int32_t* queue, int64_t n_pix,
                                         int32_t* next_queue, int sms, cudaStream_t st) {
     k_stats<true, false><<<grid_for(n_pix * 4, 256, sms, 8), 256, 0, st>>>(w, A, queue, 0, n_pix, next_queue,
@@ -993,10 +1084,10 @@ __device__ __forceinline__ void round_first_chunk(RoundCtl* rc, const RoundPlan&
     rc->nj = min(rc->per_chunk, rc->Q);
 }
 
-__global__ void k_round_init(RoundCtl* rc, Wave w, RoundPlan plan, int32_t* q0, int32_t* q1, int iota) {
-    if (iota)
+__global__ void k_round_init(RoundCtl* rc, Wave w, RoundPlan plan, int32_t* q0, int32_t* q1, int W, int H) {
+    if (W > 0)
         for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < plan.Q0; i += (int64_t)gridDim.x * blockDim.x)
-            q0[i] = (int32_t)i;
+            q0[i] = tiled_pixel(i, W, H);
     if (blockIdx.x != 0 || threadIdx.x != 0) return;
     rc->queue[0] = q0;
     rc->queue[1] = q1;
@@ -1014,8 +1105,10 @@ __global__ void k_round_init(RoundCtl* rc, Wave w, RoundPlan plan, int32_t* q0, 
     rc->t_start = global_ns();
 }
 
-__global__ void k_round_next(RoundCtl* rc, Wave w, RoundPlan plan, cudaGraphConditionalHandle h) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
+__global__ void __launch_bounds__(REQUEUE_BLOCK) k_round_next(RoundCtl* rc, Wave w, RoundPlan plan,
+                                                              cudaGraphConditionalHandle h) {
+    requeue(w, rc->queue[rc->qi], rc->j0, rc->nj, rc->queue[rc->qi ^ 1]);
+    if (threadIdx.x != 0) return;
     rc->iters += 1;
     rc->stats_pix += rc->nj;
     unsigned int go = 1;
@@ -1051,14 +1144,14 @@ __global__ void k_round_next(RoundCtl* rc, Wave w, RoundPlan plan, cudaGraphCond
 }
 
 cudaError_t launch_round_init(RoundCtl* rc, const Wave& w, const RoundPlan& plan, int32_t* q0, int32_t* q1,
-                              bool iota, int sms, cudaStream_t st) {
-    k_round_init<<<iota ? grid_for(plan.Q0, 256, sms, 8) : 1, 256, 0, st>>>(rc, w, plan, q0, q1, iota ? 1 : 0);
+                              int W, int H, int sms, cudaStream_t st) {
+    k_round_init<<<W > 0 ? grid_for(plan.Q0, 256, sms, 8) : 1, 256, 0, st>>>(rc, w, plan, q0, q1, W, H);
     return cudaGetLastError();
 }
 
 cudaError_t launch_round_next(RoundCtl* rc, const Wave& w, const RoundPlan& plan, cudaGraphConditionalHandle h,
                               cudaStream_t st) {
-    k_round_next<<<1, 32, 0, st>>>(rc, w, plan, h);
+    k_round_next<<<1, REQUEUE_BLOCK, 0, st>>>(rc, w, plan, h);
     return cudaGetLastError();
 }
 
@@ -1074,13 +1167,14 @@ cudaError_t launch_add_f64(float* out, const double* acc, int n, cudaStream_t st
 }
 
 // queue entries (job << 24 | pixel) of one job
-__global__ void k_fill_entries(int32_t* q, int64_t n, int job) {
+__global__ void k_fill_entries(int32_t* q, int W, int H, int job) {
+    const int64_t n = (int64_t)W * H;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        q[i] = (int32_t)(((uint32_t)job << 24) | (uint32_t)i);
+        q[i] = (int32_t)(((uint32_t)job << 24) | (uint32_t)tiled_pixel(i, W, H));
 }
 
-cudaError_t launch_fill_entries(int32_t* q, int64_t n, int job, int sms, cudaStream_t st) {
-    k_fill_entries<<<grid_for(n, 256, sms, 8), 256, 0, st>>>(q, n, job);
+cudaError_t launch_fill_entries(int32_t* q, int W, int H, int job, int sms, cudaStream_t st) {
+    k_fill_entries<<<grid_for((int64_t)W * H, 256, sms, 8), 256, 0, st>>>(q, W, H, job);
     return cudaGetLastError();
 }
 
@@ -1090,8 +1184,8 @@ cudaError_t launch_write_samples(const Wave& w, int64_t out0, int64_t n_paths, f
     return cudaGetLastError();
 }
 
-cudaError_t launch_iota(int32_t* q, int64_t n, int sms, cudaStream_t st) {
-    k_iota<<<grid_for(n, 256, sms, 8), 256, 0, st>>>(q, n);
+cudaError_t launch_pixel_queue(int32_t* q, int W, int H, int sms, cudaStream_t st) {
+    k_pixel_queue<<<grid_for((int64_t)W * H, 256, sms, 8), 256, 0, st>>>(q, W, H);
     return cudaGetLastError();
 }
 

@@ -111,17 +111,22 @@ cudaError_t launch_shade(const DevScene& sc, const DevFrame& fr, const DevParams
                          int depth, bool last, int64_t max_n, int sms, cudaStream_t st, const Job* jobs);
 cudaError_t launch_stats(const Wave& w, const StatsArgs& A, const int32_t* queue, int64_t j0, int64_t n_pix,
                          int32_t* next_queue, int sms, cudaStream_t st, const Job* jobs, const RoundCtl* rc = nullptr);
-// device-resident round loop: start state (and, with iota, queue 0 = 0..Q0-1)
+// appends the pixels that launch_stats left undecided to the next round's queue
+// (the device-resident loop's control kernel does it itself)
+cudaError_t launch_requeue(const Wave& w, const int32_t* queue, int64_t j0, int64_t n_pix, int32_t* next_queue,
+                           cudaStream_t st);
+// device-resident round loop: start state (and, with W > 0, queue 0 = the pixels of a W x H image)
 cudaError_t launch_round_init(RoundCtl* rc, const Wave& w, const RoundPlan& plan, int32_t* q0, int32_t* q1,
-                              bool iota, int sms, cudaStream_t st);
+                              int W, int H, int sms, cudaStream_t st);
 // after a chunk: next chunk or round, or the end of the loop (condition 0)
 cudaError_t launch_round_next(RoundCtl* rc, const Wave& w, const RoundPlan& plan, cudaGraphConditionalHandle h,
                               cudaStream_t st);
 // out[i] += (float)acc[i] for i < n (the adjoint's FP64 emission accumulator)
 cudaError_t launch_add_f64(float* out, const double* acc, int n, cudaStream_t st);
-cudaError_t launch_fill_entries(int32_t* q, int64_t n, int job, int sms, cudaStream_t st);
+cudaError_t launch_fill_entries(int32_t* q, int W, int H, int job, int sms, cudaStream_t st);
 cudaError_t launch_write_samples(const Wave& w, int64_t out0, int64_t n_paths, float* L_out, uint32_t* sig_out,
                                  int sms, cudaStream_t st);
-cudaError_t launch_iota(int32_t* q, int64_t n, int sms, cudaStream_t st);
+// every pixel of a W x H image, in tiles
+cudaError_t launch_pixel_queue(int32_t* q, int W, int H, int sms, cudaStream_t st);
 
 }  // namespace mcev

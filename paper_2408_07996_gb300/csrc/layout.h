@@ -136,6 +136,7 @@ struct Wave {
     // queues of path slots
     int32_t* list[2];         // rays of this bounce and of the next (ping-pong)
     int32_t* sh_list;         // shadow rays
+    uint32_t* again;          // per chunk pixel, one bit: undecided after this round
     // shadow rays
     float4* sh_d;             // xyz direction, w = t_max
     float* sh_c;              // unoccluded contribution
