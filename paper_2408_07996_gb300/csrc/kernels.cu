@@ -494,7 +494,8 @@ __global__ void __launch_bounds__(Q_BLOCK, Q_RESIDENT)
             VertexGrad vg{-1, -1, 0.0f, 0.0f};
             if (e < size) {
                 if (split) e = order[e];
-                key = shade_path<kBatch, kAdjoint>(sc, fr, P, w, list ? __ldg(list + t0 + e) : (int)(t0 + e), depth, jobs, vg);
+                const int p = list ? __ldg(list + t0 + e) : (int)(t0 + e);
+                key = shade_path<kBatch, kAdjoint>(sc, fr, P, w, p, depth, jobs, vg);
             }
             if (kAdjoint) {
                 __syncwarp();
