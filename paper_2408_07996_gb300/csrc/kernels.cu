@@ -1108,7 +1108,9 @@ __global__ void k_round_init(RoundCtl* rc, Wave w, RoundPlan plan, int32_t* q0, 
 
 __global__ void __launch_bounds__(REQUEUE_BLOCK) k_round_next(RoundCtl* rc, Wave w, RoundPlan plan,
                                                               cudaGraphConditionalHandle h) {
-    requeue(w, rc->queue[rc->qi], rc->j0, rc->nj, rc->queue[rc->qi ^ 1]);
+    // (every pixel is decided at spp_max)
+    if (rc->n_done + rc->spp_r < plan.spp_max)
+        requeue(w, rc->queue[rc->qi], rc->j0, rc->nj, rc->queue[rc->qi ^ 1]);
     if (threadIdx.x != 0) return;
     rc->iters += 1;
     rc->stats_pix += rc->nj;

@@ -56,3 +56,26 @@ def test_round_window_only_changes_what_is_traced(spp_max):
             assert torch.equal(a, b)
         assert out[window][3]["samples_used"] == out[1][3]["samples_used"]
         assert out[window][3]["paths"] >= out[1][3]["paths"]
+
+
+@pytest.mark.parametrize("W,H", [(1, 1), (15, 17), (16, 16), (33, 5), (5, 33), (257, 64), (640, 131)])
+def test_every_pixel_is_queued_once(W, H):
+    """The tiled first queue and the ordered re-queueing on ragged images and
+    across the statistics kernel's and the re-queue's tile sizes: every pixel
+    gets its samples, and the frame is the one of a queue of single chunks."""
+    w = sg.workload("cornell64")
+    outs = []
+    for wavefront, host in ((0, 0), (4096, 0), (4096, 1)):
+        r = Renderer(W, H)
+        r.upload(w.scene)
+        r.configure(w)
+        r.set_params(wavefront=wavefront, host_rounds=host)
+        r.render_reference(0.0, 24)
+        assert bool((r.reference_arrays()[0] == 24).all())
+        o = r.render_events(0.0, 1.0, w.C, w.alpha, w.spp_batch, 80)
+        assert int(o["spp"].min()) >= w.spp_min and int(o["spp"].max()) <= 80
+        assert o["stats"]["samples_used"] == int(o["spp"].sum())
+        outs.append([o[k].clone() for k in ("events", "spp", "mean")])
+        r.close()
+    for o in outs[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(outs[0], o))
