@@ -65,7 +65,7 @@ def parse():
 
 def profile_band(args):
     """tracePaths over one band of image rows: the first launches of the
-    process are full-size raygen / extend / shade / shadow launches."""
+    process are full-size traversal and shading launches."""
     import torch
 
     import scenegen as sg
@@ -313,19 +313,15 @@ def run_batch(args):
     print(json.dumps(line), flush=True)
 
 
-# algorithmic bytes of one mcev_event_quality call: per voxel the frame error
-# reads 2, and each of the 4 transforms (2 directions x 2 polarities) reads
-# its video (1) and writes 4 in the row pass, reads 4 and writes 4 in each
-# column pass, and reads the query video (1) in the match pass; per event,
-# the match pass reads its 4-byte distance
-QUALITY_BYTES_PER_VOXEL = 2 + 4 * (1 + 4 + 8 + 8 + 1)
+# bytes one mcev_event_quality call cannot do without: each video read once
+# (the event bits it packs, 1/2 byte per voxel, stay in L2)
+QUALITY_BYTES_PER_VOXEL = 2
 # statistics kernel (a7-a10 fused): per pixel visit it reads the queue entry
 # (4), the running and reference (n, mean, M2) (24) and writes the running
-# state (12) and a re-queue entry or event/spp (4); per path it reads one
+# state (12) and a re-queue bit or event/spp (4); per path it reads one
 # 4-byte radiance
 STATS_BYTES_PER_PIXEL_VISIT = 44
 STATS_BYTES_PER_PATH = 4
-QUALITY_BYTES_PER_EVENT = 4
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per traced ray of
 # the traversal launches (k_extend + k_shadow_extend, two-wide BVH), from a
@@ -387,19 +383,19 @@ def run_quality(args):
     n = T * H * W
     peak, basis = _hbm_peak()
     q = res[-1]
-    algo_bytes = QUALITY_BYTES_PER_VOXEL * n + QUALITY_BYTES_PER_EVENT * (q["n_a"] + q["n_b"])
+    algo_bytes = QUALITY_BYTES_PER_VOXEL * n
     achieved = algo_bytes / (gpu_ms / 1e3) / 1e9
     line = {"metric": "event-video quality metrics (RMSE, PSNR, F1, PSCD) throughput", "value": n * K / (ms / 1e3) / 1e9,
             "unit": "Gvoxels/s", "n_gpus": 1, "steps": K, "warmup": Wm, "ms_per_step": ms / K,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "int32", "data": "synthetic",
             "config": {"workload": f"quality_{W}x{H}x{T}", "width": W, "height": H, "frames": T, "tau2": 3,
                        "events_a": q["n_a"], "events_b": q["n_b"],
-                       "l2": "two int32 scratch volumes of 369 MB each are streamed every step (> L2)"},
+                       "l2": "the two 92 MB videos are read every step (> L2)"},
             "gpu_launches": sum(r["kernel_launches"] for r in res),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": None, "basis": basis,
                          "bytes_per_call": algo_bytes, "bytes_per_voxel": QUALITY_BYTES_PER_VOXEL,
-                         "bytes_per_event": QUALITY_BYTES_PER_EVENT, "avg_call_ms": gpu_ms},
+                         "avg_call_ms": gpu_ms},
             "metrics": {k: q[k] for k in ("rmse", "psnr", "precision", "recall", "f1", "pscd")},
             "clocks": clk}
     print(json.dumps(line), flush=True)
@@ -618,7 +614,7 @@ def main():
     peak_tflops = sm_count * FP32_LANES_PER_SM * FLOP_PER_LANE_CLOCK * sm_max_mhz * 1e6 / 1e12
     achieved = flop / n_trav / (ext_ms / n_trav / 1e3) / 1e12 if ext_ms > 0 else None
     total_kms = sum(kms)
-    roofline = {"kernel": "BVH traversal: k_extend, k_shadow_extend (closest-hit + shadow rays)", "bound": "alu",
+    roofline = {"kernel": "BVH traversal: k_trace (closest-hit + shadow rays)", "bound": "alu",
                 "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
                 "frac": (achieved / peak_tflops) if achieved else None,
                 "traffic": traversal_traffic(rays / n_trav, args.bvh_width),
