@@ -386,15 +386,20 @@ __device__ __forceinline__ int32_t cells_near(const uint32_t* __restrict__ row, 
 // ring around the event (ring r is at least 8 (r - 1) + 1 frames or rows away);
 // an occupied cell bounds the distance from above and below, and of those that
 // could hold a nearer event the nearest is searched first, its 64 rows two per
-// lane.  Bound by the dependent loads of one event after the
-// other and some 4000 instructions each (477 us on 1280x720x100;
-// cells of 4 frames and no bound from above 482 us); the exact transform of the four
-// sets took 8.3 ms there.
-__global__ void __launch_bounds__(QBLOCK) k_search_far(QGrid G, const uint32_t* __restrict__ masks,
-                                                       const uint32_t* __restrict__ cells, int tau2,
-                                                       int32_t* __restrict__ d2_a, int32_t* __restrict__ d2_b,
-                                                       const uint64_t* __restrict__ far_list, int64_t far_cap,
-                                                       unsigned long long* acc) {
+// lane.  Bound by the dependent loads of one event after the other and some 4000
+// instructions each.  Events differ widely in cost, so the blocks are small and up
+// to five times as many as are resident (20 of 64 threads, 48 registers, no
+// spills): whole quality calls of 1280x720x100, two videos, 0.79 and 0.71 ms with 8
+// blocks of 256 threads per SM, 0.72 and 0.66 ms with 40, 0.69 and 0.62 ms with 100
+// blocks of 64, the same with 300 or with a cursor on the device; 0.72 and
+// 0.65 ms with 40 registers.  Lane s adds up what its warp found for set s: one
+// addition per warp to the set's words instead of one per event.
+constexpr int FWARPS = 2;
+__global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const uint32_t* __restrict__ masks,
+                                                                const uint32_t* __restrict__ cells, int tau2,
+                                                                int32_t* __restrict__ d2_a, int32_t* __restrict__ d2_b,
+                                                                const uint64_t* __restrict__ far_list, int64_t far_cap,
+                                                                unsigned long long* acc) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int64_t n = (int64_t)acc[QACC_FAR];
@@ -402,6 +407,8 @@ __global__ void __launch_bounds__(QBLOCK) k_search_far(QGrid G, const uint32_t* 
     if (n > far_cap) return;
     const int sw = (G.ww + 31) / 32, cy_n = (G.H + QCELL - 1) / QCELL, ct_n = (G.T + QCELL - 1) / QCELL;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    unsigned long long closed = 0, matched = 0;      // of the set whose number the lane has
+    double sum = 0.0;
     for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += nw) {
         const uint64_t id = far_list[k];
         const int s = (int)(id >> 60);
@@ -469,16 +476,20 @@ __global__ void __launch_bounds__(QBLOCK) k_search_far(QGrid G, const uint32_t* 
                 }
             }
         }
-        if (lane != 0) continue;
         // (the set's target has events, so one was found)
-        unsigned long long* as = acc + QACC_SET + s * QSET_WORDS;
-        atomicAdd(as + QSET_OPEN, ~0ull);      // one less
-        if (best <= tau2) atomicAdd(as + QSET_MATCH, 1ull);
-        if (best < QHIST) atomicAdd(as + QSET_HIST + best, 1ull);
-        else atomicAdd(reinterpret_cast<double*>(as + QSET_SUM), sqrt((double)best));
+        if (lane != s) continue;
+        ++closed;
+        matched += best <= tau2;
+        if (best < QHIST) atomicAdd(acc + QACC_SET + s * QSET_WORDS + QSET_HIST + best, 1ull);
+        else sum += sqrt((double)best);
         int32_t* d2 = s < 2 ? d2_a : d2_b;
         if (d2) d2[voxel] = best;
     }
+    if (closed == 0) return;                         // (lanes from QSETS on, and warps without an event)
+    unsigned long long* as = acc + QACC_SET + lane * QSET_WORDS;
+    atomicAdd(as + QSET_OPEN, 0ull - closed);
+    if (matched) atomicAdd(as + QSET_MATCH, matched);
+    if (sum != 0.0) atomicAdd(reinterpret_cast<double*>(as + QSET_SUM), sum);
 }
 
 // ---------------------------------------------------------------- rows: 1-D distance to the nearest event
@@ -718,7 +729,8 @@ cudaError_t launch_quality(const QualityArgs& A, int sms, cudaStream_t st, int* 
     k_search<<<grid_of(G.n_words, 32 * QWARPS, sms, 32), 32 * QWARPS, 0, st>>>(G, A.masks, A.tau2, A.d2_a, A.d2_b,
                                                                             A.far_list, far_cap, A.acc);
     k_cells<<<sms * 8, QBLOCK, 0, st>>>(G, A.masks, A.cells, A.acc);
-    k_search_far<<<sms * 8, QBLOCK, 0, st>>>(G, A.masks, A.cells, A.tau2, A.d2_a, A.d2_b, A.far_list, far_cap, A.acc);
+    k_search_far<<<grid_of(far_cap, FWARPS, sms, 100), 32 * FWARPS, 0, st>>>(G, A.masks, A.cells, A.tau2, A.d2_a,
+                                                                             A.d2_b, A.far_list, far_cap, A.acc);
     *launches += 4;
     return cudaGetLastError();
 }
