@@ -1056,7 +1056,7 @@ mcev_status run_rounds(mcev_ctx* ctx, const Frame& fr, StatsArgs A, int64_t* pat
             ST(trace_chunk(ctx, fr, P, queue[qi], j0, spp_r, n_done, nj * spp_r, B));
             LAUNCH(MCEV_K_STATS,
                    launch_stats(ctx->wave, A, queue[qi], j0, nj, queue[qi ^ 1], ctx->sms, ctx->stream, jobs, nullptr));
-            if (n_done + spp_r < A.spp_max)   // every pixel is decided at spp_max
+            if (n_done + spp_r < A.spp_max)   // no pixel goes on from the round that reaches spp_max
                 LAUNCH(MCEV_K_STATS, launch_requeue(ctx->wave, queue[qi], j0, nj, queue[qi ^ 1], ctx->stream));
             ctx->stats_pix += nj;
         }

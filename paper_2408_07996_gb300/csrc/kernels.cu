@@ -857,6 +857,10 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
             const bool own = on && q == 0;
             const bool again = own && (detect ? open : n < A.spp_max);
             if (again) atomicOr(&again_bits[in_tile >> 5], 1u << (in_tile & 31));
+            // Nothing is queued in the round that reaches spp_max; a pixel it leaves open (its
+            // FP32 count cannot reach every spp_max above 2^24) is counted, which ends the call
+            // with an error.
+            if (!kChecked && again && A.k_base + A.spp_r >= A.spp_max) atomicAdd(w.counters + 3, 1);
             if (!own) continue;
             if (bad) atomicAdd(w.counters + 4, bad);
             A.cur.n[pix] = n;
@@ -1108,7 +1112,7 @@ __global__ void k_round_init(RoundCtl* rc, Wave w, RoundPlan plan, int32_t* q0, 
 
 __global__ void __launch_bounds__(REQUEUE_BLOCK) k_round_next(RoundCtl* rc, Wave w, RoundPlan plan,
                                                               cudaGraphConditionalHandle h) {
-    // (every pixel is decided at spp_max)
+    // (no pixel goes on from the round that reaches spp_max; k_stats counts those it leaves open)
     if (rc->n_done + rc->spp_r < plan.spp_max)
         requeue(w, rc->queue[rc->qi], rc->j0, rc->nj, rc->queue[rc->qi ^ 1]);
     if (threadIdx.x != 0) return;

@@ -147,7 +147,7 @@ struct Wave {
     // Device counters, 64 int32 words; every slot the kernels use:
     //   [0], [1]  ray queue sizes (ping-pong queues 0 and 1)
     //   [2], [19] shadow-ray counts of the bounces traced from ray queue 0 / 1
-    //   [3]       undecided pixels re-queued by the statistics kernel
+    //   [3]       undecided pixels: queued for the next round, or still open at spp_max
     //   [4]       non-finite path values (counted as 0)
     //   [5], [6]  positive / negative events
     //   [7]       pixels decided at spp_max
