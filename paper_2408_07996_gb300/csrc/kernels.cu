@@ -197,6 +197,7 @@ __device__ __forceinline__ void add_work(const Wave& w, int3 closest, int3 shado
     WorkAcc& a = work_acc();
     warp_work(a, 0, closest);
     warp_work(a, 3, shadow);
+    __syncwarp();      // orders the other lanes' additions to a.emit before lane 0's fence
     if ((threadIdx.x & 31) == 0) {
         __threadfence_block();
         if (atomicAdd(&a.done, 1u) == (blockDim.x >> 5) - 1u) {
