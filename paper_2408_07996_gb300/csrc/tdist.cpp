@@ -8,12 +8,15 @@
 //                 + (1*3*..*(nu-3)) / (2*4*..*(nu-2)) cos^(nu-2))
 // All terms are positive, so the sum is stable in FP64 for the nu <= 2^16
 // the renderer needs.  The critical value of the one-tailed test (Sec. 3.2)
-// is the alpha-quantile of that CDF: Newton steps from the expansion of the
-// quantile in 1/nu (A&S 26.7.5), kept inside a bracket and replaced by
-// bisection where a step leaves it.  The series costs nu/2 divisions in a
+// is the alpha-quantile of that CDF, rounded to FP32: Newton steps from the
+// expansion of the quantile in 1/nu (A&S 26.7.5), kept inside a bracket.  Where the
+// series' rounding leaves room for more than one FP32 value (small alpha, large
+// nu), the value is the one that bisection of the computed CDF ends at, so the tables
+// hold bisection's values for every alpha.  The series costs nu/2 divisions in a
 // chain, so the number of its evaluations is what the table costs: 2 to 4 per
-// value instead of about 60 by bisection alone (on an x86 host a 15-value
-// table up to nu = 255 0.137 -> 0.010 ms, 120 values up to 8191 22 -> 0.41 ms).
+// value instead of about 60 by bisection alone (on an x86 host, alpha 0.05 and 0.01:
+// a 15-value table up to nu = 255 0.13 -> 0.01 ms, 128 values up to 8191 21 -> 0.4
+// ms; alpha 1e-6 2.3 ms, 1e-12 11 ms).
 #include "tdist.h"
 
 #include <algorithm>
@@ -63,8 +66,31 @@ static double normal_quantile(double p) {
     return upper ? -z : z;
 }
 
+// The quantile by bisection of the computed CDF.  [a, b] holds every root that the
+// series' rounding allows: outside it the CDF lies on the side of p that the
+// position tells, so it is evaluated inside only.  Stops when both ends round to
+// the same FP32 value, which is what the tables hold.
+static double bisect(double p, int nu, double a, double b) {
+    auto cdf = [&](double t) { return t < a ? 0.0 : (t > b ? 1.0 : t_cdf_int(t, nu)); };
+    double lo = -1.0, hi = 1.0;
+    while (cdf(lo) > p) lo *= 2.0;
+    while (cdf(hi) < p) hi *= 2.0;
+    for (int it = 0; it < 200 && (float)lo != (float)hi; ++it) {
+        const double mid = 0.5 * (lo + hi);
+        if (mid == lo || mid == hi) break;
+        if (cdf(mid) < p) lo = mid;
+        else hi = mid;
+    }
+    return 0.5 * (lo + hi);
+}
+
 double t_quantile_int(double p, int nu) {
     if (!(p > 0.0 && p < 1.0)) return std::nan("");
+    // What rounding makes of the CDF: at most about 2 nu + 16 units of 2^-53 (every
+    // term of the series is a product of up to nu / 2 factors), taken twice.  A p of
+    // that size has no root worth the name, only the one that bisection ends at.
+    const double noise = (4.0 * nu + 32.0) * 0x1p-53;
+    if (std::min(p, 1.0 - p) < 64.0 * noise) return bisect(p, nu, -HUGE_VAL, HUGE_VAL);
     const double z = normal_quantile(p), z2 = z * z, v = 1.0 / nu;
     const double g1 = z * (z2 + 1.0) / 4.0;
     const double g2 = z * ((5.0 * z2 + 16.0) * z2 + 3.0) / 96.0;
@@ -74,12 +100,22 @@ double t_quantile_int(double p, int nu) {
     // log of the density's constant
     const double lc = std::lgamma(0.5 * (nu + 1.0)) - std::lgamma(0.5 * nu) - 0.5 * std::log(nu * M_PI);
     double lo = -HUGE_VAL, hi = HUGE_VAL;     // cdf(lo) < p <= cdf(hi)
-    for (int it = 0; it < 400; ++it) {
+    for (int it = 0; it < 100; ++it) {
         const double f = t_cdf_int(t, nu) - p;
+        const double pdf = std::exp(lc - 0.5 * (nu + 1.0) * std::log1p(t * t / nu));
+        const double step = f / pdf;
+        if (std::fabs(step) <= 1e-9 * std::fabs(t) || std::fabs(f) <= noise) {
+            // a Newton step of this size leaves an error below the CDF's own rounding
+            t -= step;
+            const double range = 2.0 * noise / pdf + 1e-15 * std::fabs(t);
+            if ((float)(t - range) == (float)(t + range)) return t;
+            // (the density must not fall off within the range)
+            if (range * (nu + 1.0) * std::fabs(t) < 0.1 * (nu + t * t)) return bisect(p, nu, t - range, t + range);
+            break;
+        }
         if (f < 0.0) lo = t;
         else hi = t;
-        const double pdf = std::exp(lc - 0.5 * (nu + 1.0) * std::log1p(t * t / nu));
-        double next = t - f / pdf;
+        double next = t - step;
         if (!(next > lo && next < hi)) {
             // outside the bracket (or no density left): halve it, or widen it
             if (std::isinf(lo)) next = hi > 0.0 ? -1.0 : 2.0 * hi - 1.0;
@@ -87,12 +123,9 @@ double t_quantile_int(double p, int nu) {
             else next = 0.5 * (lo + hi);
             if (next == lo || next == hi) break;
         }
-        const double step = std::fabs(next - t);
         t = next;
-        // a Newton step of this size leaves an error below the CDF's own rounding
-        if (step <= 1e-9 * std::fabs(t)) break;
     }
-    return t;
+    return bisect(p, nu, -HUGE_VAL, HUGE_VAL);
 }
 
 }  // namespace mcev
