@@ -699,42 +699,43 @@ __device__ __forceinline__ Moments chan(Moments a, Moments b) {
 #define MCEV_LOG(x) logf(x)
 #endif
 
-// Four lanes per pixel, eight pixels per warp.  A round traced spp_r samples of
-// a pixel: one batch, or a window of several spp_batch-sized batches.  Each
-// batch is merged and tested in order exactly as Alg. 1 would; once the pixel is
-// decided, the rest of the window is left unused.
+// Lanes per pixel of the statistics kernel: a warp, or four lanes (eight pixels per
+// warp).  A round traced spp_r samples of a pixel: one batch, or a window of
+// several batches of `sub`.  Each batch is merged and tested in order exactly as
+// Alg. 1 would; once the pixel is decided, the rest of the window is left unused.
 //
-// What bounds it: the instructions of the merge and the test (six divisions
-// and a square root), which every lane of a pixel repeats; with a warp per pixel
-// and 16-sample batches they were done 32 times over (90k pixels x 15 batches:
-// 431 us with a warp per pixel, 137 us with four lanes; eight jobs 131 -> 124 ms,
-// terrain 720p 751 -> 742 ms).  The order of the additions is fixed: sample s of a batch
-// belongs to leaf s % 32, leaves add up pairwise 16, 8, 4, 2 and 1 apart (a warp's
-// butterfly).  A lane holds every fourth leaf, so the last two steps are shuffles
-// (a + b on one lane, b + a on its partner: the same bits), and every lane of a
-// pixel ends with identical statistics and takes the same decisions.
-template <bool kChecked, bool kBatch>
-__global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32_t* __restrict__ queue, int64_t j0,
-                                               int64_t n_pix, int32_t* __restrict__ next_queue,
-                                               const Job* __restrict__ jobs, const RoundCtl* __restrict__ rc) {
-    if (rc) {
-        // sizes of the current chunk of the device-resident round loop
-        queue = rc->queue[rc->qi];
-        next_queue = rc->queue[rc->qi ^ 1];
-        j0 = rc->j0;
-        n_pix = rc->nj;
-        A0.spp_r = rc->spp_r;
-        A0.sub = rc->sub;
-        A0.k_base = rc->n_done;
-    }
+// What bounds it: with short batches the instructions of the merge and the test (six
+// divisions and a square root), which every lane of a pixel repeats: 90k pixels x
+// 15 batches of 16 431 us with a warp per pixel, 137 us with four lanes; eight jobs
+// 131 -> 124 ms, terrain 720p 751 -> 742 ms.  With long batches and few pixels the
+// latency of a pixel's own chain of loads and additions, which a warp shortens eightfold.
+// Whole detector steps, four lanes / a warp: 5000 pixels x 17 samples 19 / 27 us, 80000 x
+// 16 27 / 53, 20000 x 64 27 / 27, 20000 x 512 39 / 39, 9728 x 512 39 / 27, 1 x 64 27 / 19, 40000 x
+// 2048 138 / 103, 9728 x 2048 100 / 39, 1 x 8192 286 / 39: a warp pays up to about 32
+// pixels per sample of a batch, from batches of 64 on (a mean of 2^20 samples of one pixel:
+// 38 / 3.9 ms).
+//
+// The order of the additions is fixed: sample s of a batch belongs to leaf s % 32,
+// leaves add up pairwise 16, 8, 4, 2 and 1 apart (a warp's butterfly).  A lane holds
+// every LANES-th leaf, so the last steps are shuffles (a + b on one lane, b + a on its
+// partner: the same bits), and every lane of a pixel ends with identical
+// statistics and takes the same decisions.
+__host__ __device__ __forceinline__ bool stats_by_warp(int64_t n_pix, int64_t sub) {
+    return sub >= 64 && n_pix <= 32 * sub;
+}
+
+constexpr int STATS_STEPS = 8;
+template <bool kChecked, bool kBatch, int LANES>
+__device__ __forceinline__ void stats_tiles(const Wave& w, const StatsArgs& A0, const int32_t* __restrict__ queue,
+                                            int64_t j0, int64_t n_pix, int32_t* __restrict__ next_queue,
+                                            const Job* __restrict__ jobs, uint32_t* again_bits, int& again_at) {
     constexpr unsigned full = 0xffffffffu;
-    constexpr int LANES = 4, PIX = 32 / LANES, LEAVES = 32 / LANES;
+    constexpr int PIX = 32 / LANES, LEAVES = 32 / LANES;
+    constexpr int AHEAD = 8;       // samples that a lane of a warp's pixel loads at a time
     const int lane = threadIdx.x & 31, q = lane & (LANES - 1);
     const int test0 = A0.mode == MODE_DETECT ? (int)((A0.k_base - A0.spp_min) / A0.spp_batch) : 0;
-    // a block's tile: up to 8 steps of 64 pixels, fewer when there are few pixels
-    constexpr int STEP = 256 / LANES, STEPS = 8;
-    __shared__ uint32_t again_bits[STEP * STEPS / 32];
-    __shared__ int again_at;
+    // a block's tile: up to 8 steps of 64 (8) pixels, fewer when there are few pixels
+    constexpr int STEP = 256 / LANES, STEPS = STATS_STEPS;
     const int64_t per_step = (int64_t)gridDim.x * STEP;
     const int steps = (int)max((int64_t)1, min((int64_t)STEPS, n_pix / per_step));
     for (int64_t t0 = (int64_t)blockIdx.x * steps * STEP; t0 < n_pix; t0 += per_step * steps) {
@@ -784,37 +785,48 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
                     sh = MCEV_LOG((isfinite(L0) ? L0 : 0.0f) + A.eps);
                 }
                 float a1[LEAVES], a2[LEAVES];
-    #pragma unroll
+#pragma unroll
                 for (int m = 0; m < LEAVES; ++m) a1[m] = a2[m] = 0.0f;
                 if (open) {
-                    for (int b = s0; b < s1; b += 32) {
-    #pragma unroll
-                        for (int m = 0; m < LEAVES; ++m) {
-                            if (b + LANES * m >= s1) break;     // the same for the whole warp
-                            const int s = b + LANES * m + q;
-                            if (s < s1) {
-                                float Lv = Lp[s];
-                                if (!isfinite(Lv)) {
-                                    Lv = 0.0f;
-                                    ++bad;
-                                }
-                                const float d = MCEV_LOG(Lv + A.eps) - sh;
-                                a1[m] += d;
-                                a2[m] = fmaf(d, d, a2[m]);
+                    auto add = [&](int m, float x) {
+                        if (!isfinite(x)) {
+                            x = 0.0f;
+                            ++bad;
+                        }
+                        const float d = MCEV_LOG(x + A.eps) - sh;
+                        a1[m] += d;
+                        a2[m] = fmaf(d, d, a2[m]);
+                    };
+                    if constexpr (LANES == 32) {
+                        for (int b = s0 + q; b < s1; b += 32 * AHEAD) {
+                            float x[AHEAD];
+#pragma unroll
+                            for (int u = 0; u < AHEAD; ++u) x[u] = b + 32 * u < s1 ? Lp[b + 32 * u] : 0.0f;
+#pragma unroll
+                            for (int u = 0; u < AHEAD; ++u)
+                                if (b + 32 * u < s1) add(0, x[u]);
+                        }
+                    } else {
+                        for (int b = s0; b < s1; b += 32) {
+#pragma unroll
+                            for (int m = 0; m < LEAVES; ++m) {
+                                if (b + LANES * m >= s1) break;     // the same for the whole warp
+                                const int s = b + LANES * m + q;
+                                if (s < s1) add(m, Lp[s]);
                             }
                         }
                     }
                 }
-    #pragma unroll
+#pragma unroll
                 for (int h = LEAVES / 2; h > 0; h >>= 1) {
-    #pragma unroll
+#pragma unroll
                     for (int m = 0; m < h; ++m) {
                         a1[m] += a1[m + h];
                         a2[m] += a2[m + h];
                     }
                 }
                 float s1d = a1[0], s2d = a2[0];
-    #pragma unroll
+#pragma unroll
                 for (int off = LANES / 2; off > 0; off >>= 1) {
                     s1d += __shfl_xor_sync(full, s1d, off);
                     s2d += __shfl_xor_sync(full, s2d, off);
@@ -852,7 +864,7 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
                 }
                 open = !decided;
             }
-    #pragma unroll
+#pragma unroll
             for (int off = LANES / 2; off > 0; off >>= 1) bad += __shfl_xor_sync(full, bad, off);
             // the pixel's first lane writes it back
             const bool own = on && q == 0;
@@ -897,8 +909,9 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
         __syncthreads();
         if (!kChecked) {
             // requeue() queues them
-            const int64_t word = (t0 >> 5) + threadIdx.x;
-            if (threadIdx.x < steps * STEP / 32 && word < (n_pix + 31) >> 5) w.again[word] = again_bits[threadIdx.x];
+            const int64_t at = (t0 >> 3) + threadIdx.x;
+            if (threadIdx.x < steps * STEP / 8 && at < (n_pix + 7) >> 3)
+                reinterpret_cast<uint8_t*>(w.again)[at] = reinterpret_cast<const uint8_t*>(again_bits)[threadIdx.x];
             __syncthreads();
             continue;
         }
@@ -920,6 +933,28 @@ __global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A0, const int32
     }
 }
 
+template <bool kChecked, bool kBatch>
+__global__ void __launch_bounds__(256) k_stats(Wave w, StatsArgs A, const int32_t* __restrict__ queue, int64_t j0,
+                                               int64_t n_pix, int32_t* __restrict__ next_queue,
+                                               const Job* __restrict__ jobs, const RoundCtl* __restrict__ rc) {
+    __shared__ uint32_t again_bits[64 * STATS_STEPS / 32];
+    __shared__ int again_at;
+    if (rc) {
+        // sizes of the current chunk of the device-resident round loop
+        queue = rc->queue[rc->qi];
+        next_queue = rc->queue[rc->qi ^ 1];
+        j0 = rc->j0;
+        n_pix = rc->nj;
+        A.spp_r = rc->spp_r;
+        A.sub = rc->sub;
+        A.k_base = rc->n_done;
+    }
+    if (stats_by_warp(n_pix, A.sub))
+        stats_tiles<kChecked, kBatch, 32>(w, A, queue, j0, n_pix, next_queue, jobs, again_bits, again_at);
+    else
+        stats_tiles<kChecked, kBatch, 4>(w, A, queue, j0, n_pix, next_queue, jobs, again_bits, again_at);
+}
+
 // Appends a chunk's undecided pixels (w.again, one bit per entry) to the next
 // round's queue in their order, by one block.  Neighbours in the image stay
 // neighbours in the queue from round to round, so that their paths keep meeting
@@ -939,6 +974,7 @@ __device__ __forceinline__ void requeue(const Wave& w, const int32_t* __restrict
     for (int64_t t0 = 0; t0 < words; t0 += REQUEUE_BLOCK) {
         const int64_t k = t0 + threadIdx.x;
         uint32_t bits = k < words ? w.again[k] : 0u;
+        if (32 * k + 32 > n_pix && k < words) bits &= (1u << (n_pix & 31)) - 1u;    // (written up to a whole byte)
         const int c = __popc(bits);
         int v = c;
 #pragma unroll
@@ -1045,11 +1081,12 @@ cudaError_t launch_shade(const DevScene& sc, const DevFrame& fr, const DevParams
 cudaError_t launch_stats(const Wave& w, const StatsArgs& A, const int32_t* queue, int64_t j0, int64_t n_pix,
                          int32_t* next_queue, int sms, cudaStream_t st, const Job* jobs, const RoundCtl* rc) {
     // with rc, n_pix is an upper bound of the chunk's pixels (the size is on the device)
+    const int64_t lanes = n_pix * (rc || stats_by_warp(n_pix, A.sub) ? 32 : 4);
     if (jobs)
-        k_stats<false, true><<<grid_for(n_pix * 4, 256, sms, 8), 256, 0, st>>>(w, A, queue, j0, n_pix, next_queue,
+        k_stats<false, true><<<grid_for(lanes, 256, sms, 8), 256, 0, st>>>(w, A, queue, j0, n_pix, next_queue,
                                                                                  jobs, rc);
     else
-        k_stats<false, false><<<grid_for(n_pix * 4, 256, sms, 8), 256, 0, st>>>(w, A, queue, j0, n_pix, next_queue,
+        k_stats<false, false><<<grid_for(lanes, 256, sms, 8), 256, 0, st>>>(w, A, queue, j0, n_pix, next_queue,
                                                                                   nullptr, rc);
     return cudaGetLastError();
 }
@@ -1062,8 +1099,9 @@ cudaError_t launch_requeue(const Wave& w, const int32_t* queue, int64_t j0, int6
 
 static cudaError_t launch_stats_checked(const Wave& w, const StatsArgs& A, const int32_t* queue, int64_t n_pix,
                                         int32_t* next_queue, int sms, cudaStream_t st) {
-    k_stats<true, false><<<grid_for(n_pix * 4, 256, sms, 8), 256, 0, st>>>(w, A, queue, 0, n_pix, next_queue,
-                                                                             nullptr, nullptr);
+    const int64_t lanes = n_pix * (stats_by_warp(n_pix, A.sub) ? 32 : 4);
+    k_stats<true, false><<<grid_for(lanes, 256, sms, 8), 256, 0, st>>>(w, A, queue, 0, n_pix, next_queue, nullptr,
+                                                                         nullptr);
     return cudaGetLastError();
 }
 
