@@ -1765,10 +1765,10 @@ mcev_status mcev_event_quality(mcev_ctx* ctx, const int8_t* a, const int8_t* b, 
     CU(cudaEventRecord(ctx->ev1, ctx->stream));
     ST(read_acc());
     if (acc[QACC_BAD]) return fail(ctx, MCEV_ERR_ARG, "event values must be -1, 0 or +1");
-    // sets with more far events than their list holds: exact distance transform
+    // sets with more far events than the list holds, or too far ones: exact distance transform
     bool again = false;
     for (int set = 0; set < QSETS; ++set) {
-        if (!acc[QACC_SET + set * QSET_WORDS + QSET_OPEN]) continue;
+        if (!(acc[QACC_EDT] >> set & 1ull)) continue;
         const size_t vol = al(4 * n);
         ST(dev_alloc(ctx, ctx->d_qedt, 2 * vol + al(quality_stack_bytes(width, height, frames, ctx->sms))));
         A.vol0 = (int32_t*)ctx->d_qedt.ptr;

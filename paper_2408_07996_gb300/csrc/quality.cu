@@ -9,9 +9,10 @@
 // per voxel, which stays in L2), events whose own bit is set in the target are
 // counted by AND and population count, and only the rest search the target's
 // rows around them ring by ring until no nearer event can exist.  Events
-// without a neighbour in the rows and columns around them are searched for by a warp each
-// through a coarse grid of cells.  Sets (polarity and direction) with more of
-// them than their list holds are matched by an exact squared Euclidean
+// without a neighbour in two rings and 15 columns are listed and searched for by a warp
+// each through a coarse grid of cells, in a bounded number of steps.  Sets (polarity and
+// direction) with more of them than the list holds, or with one that is not found
+// in time, are matched by an exact squared Euclidean
 // distance transform on the integer lattice (x, y, t), separable by axis:
 //   rows (x): the input is binary, so a warp sweeps each row left to right
 //     with a max-scan of event columns and right to left with a min-scan;
@@ -172,6 +173,10 @@ constexpr int QRINGS = 2;      // its rings (a 1280x720x100 call at 1 / 2 / 3 / 
 // reads a cell row's 64 rows two per lane
 constexpr int QCELL = 8;
 __device__ __forceinline__ int set_target(int set) { return set ^ 2; }   // the other video, same polarity
+// The searches drop set s from here on; the transform matches all of it anew.
+__device__ __forceinline__ void leave_to_edt(unsigned long long* acc, int s) {
+    if (!(*(volatile unsigned long long*)(acc + QACC_EDT) >> s & 1ull)) atomicOr(acc + QACC_EDT, 1ull << s);
+}
 
 // squared column distance from x to the nearest set bit of the row within
 // QNEAR columns, or QINF
@@ -232,14 +237,15 @@ __global__ void __launch_bounds__(32 * QWARPS) k_search(QGrid G, const uint32_t*
                                                        unsigned long long* acc) {
     __shared__ uint16_t todo[QWARPS][2048];     // word << 5 | bit, + set << 10; a voxel is in at most 2 sets
     __shared__ uint32_t hist[QSETS][256];       // squared distances settled here are below 256
-    __shared__ uint32_t open_n[QSETS];          // events not settled here
     for (int i = threadIdx.x; i < QSETS * 256; i += blockDim.x) (&hist[0][0])[i] = 0;
-    if (threadIdx.x < QSETS) open_n[threadIdx.x] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    // no event to search for, or none that is worth it: earlier blocks have left the set to
+    // the transform (which counts it anew)
+    const unsigned edt = (unsigned)*(volatile unsigned long long*)(acc + QACC_EDT);
     bool lacks[QSETS];
 #pragma unroll
-    for (int s = 0; s < QSETS; ++s) lacks[s] = acc[QACC_COUNT + set_target(s)] == 0;
+    for (int s = 0; s < QSETS; ++s) lacks[s] = acc[QACC_COUNT + set_target(s)] == 0 || (edt >> s & 1u) != 0;
     unsigned long long matched[QSETS] = {0, 0, 0, 0}, none[QSETS] = {0, 0, 0, 0};
     const int64_t chunks = (G.n_words + 31) / 32;
     for (int64_t c = (int64_t)blockIdx.x * QWARPS + wib; c < chunks; c += (int64_t)gridDim.x * QWARPS) {
@@ -312,12 +318,13 @@ __global__ void __launch_bounds__(32 * QWARPS) k_search(QGrid G, const uint32_t*
                 int32_t* d2 = s < 2 ? d2_a : d2_b;
                 if (d2) d2[voxel] = best;
             } else {
-                // (a counter past the list's end says that the list is not complete)
-                atomicAdd(&open_n[s], 1u);
+                bool listed = false;
                 if ((int64_t)*(volatile unsigned long long*)(acc + QACC_FAR) <= far_cap) {
                     const unsigned long long k = atomicAdd(acc + QACC_FAR, 1ull);
-                    if ((int64_t)k < far_cap) far_list[k] = (uint64_t)s << 60 | (uint64_t)voxel;
+                    listed = (int64_t)k < far_cap;
+                    if (listed) far_list[k] = (uint64_t)s << 60 | (uint64_t)voxel;
                 }
+                if (!listed) leave_to_edt(acc, s);
             }
         }
         __syncwarp();
@@ -329,7 +336,6 @@ __global__ void __launch_bounds__(32 * QWARPS) k_search(QGrid G, const uint32_t*
         __syncthreads();
         for (int b = threadIdx.x; b < 256; b += blockDim.x)
             if (b > 0 && hist[s][b]) atomicAdd(as + QSET_HIST + b, (unsigned long long)hist[s][b]);
-        if (threadIdx.x == 0 && open_n[s]) atomicAdd(as + QSET_OPEN, (unsigned long long)open_n[s]);
     }
 }
 
@@ -338,12 +344,14 @@ __global__ void __launch_bounds__(32 * QWARPS) k_search(QGrid G, const uint32_t*
 __global__ void __launch_bounds__(QBLOCK) k_cells(QGrid G, const uint32_t* __restrict__ masks,
                                                   uint32_t* __restrict__ cells, const unsigned long long* acc) {
     if (acc[QACC_FAR] == 0) return;
+    const unsigned edt = (unsigned)acc[QACC_EDT];
     const int lane = threadIdx.x & 31;
     const int sw = (G.ww + 31) / 32, cy_n = (G.H + QCELL - 1) / QCELL, ct_n = (G.T + QCELL - 1) / QCELL;
     const int64_t per_set = (int64_t)cy_n * ct_n * sw, n = QSETS * per_set;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += nw) {
         const int64_t set = k / per_set, rest = k - set * per_set, cr = rest / sw;
+        if (edt >> set_target((int)set) & 1u) continue;     // (no event looks for this set's any more)
         const int word = (int)(rest - cr * sw) * 32 + lane;
         const int ct = (int)(cr / cy_n), cy = (int)(cr - (int64_t)ct * cy_n);
         uint32_t any = 0;
@@ -394,7 +402,17 @@ __device__ __forceinline__ int32_t cells_near(const uint32_t* __restrict__ row, 
 // blocks of 64, the same with 300 or with a cursor on the device; 0.72 and
 // 0.65 ms with 40 registers.  Lane s adds up what its warp found for set s: one
 // addition per warp to the set's words instead of one per event.
+//
+// The transform costs the same wherever the events are, this search the more the
+// farther they are, so an event may take FSTEPS steps (a step: 32 cell rows of a
+// ring, or the search of one cell row; wide rows count by their length).  An event that
+// is not settled then leaves its set to the transform, and the set's other events are
+// skipped.  Whole calls at 64 / 128 / 256 steps: 80000 events of 1280x720x100 100 rows from
+// the other video's 0.57 / 0.57 / 0.57 ms, 500 rows 2.72 / 1.61 / 1.62 (four transforms 3.96),
+// opposite ends of 64x64x8192 3.64 / 3.78 / 4.09 (5.46), 250000 events of 16384x16384x1
+// against one in a corner 31.0 / 13.6 / 13.6 (55.1).
 constexpr int FWARPS = 2;
+constexpr int FSTEPS = 128;
 __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const uint32_t* __restrict__ masks,
                                                                 const uint32_t* __restrict__ cells, int tau2,
                                                                 int32_t* __restrict__ d2_a, int32_t* __restrict__ d2_b,
@@ -402,9 +420,7 @@ __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const u
                                                                 unsigned long long* acc) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const int64_t n = (int64_t)acc[QACC_FAR];
-    // too many for the list: the sets with open events are matched by the transform
-    if (n > far_cap) return;
+    const int64_t n = min((int64_t)acc[QACC_FAR], far_cap);
     const int sw = (G.ww + 31) / 32, cy_n = (G.H + QCELL - 1) / QCELL, ct_n = (G.T + QCELL - 1) / QCELL;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     unsigned long long closed = 0, matched = 0;      // of the set whose number the lane has
@@ -412,6 +428,10 @@ __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const u
     for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += nw) {
         const uint64_t id = far_list[k];
         const int s = (int)(id >> 60);
+        // (read by one lane: the others could see it change)
+        unsigned edt = 0;
+        if (lane == 0) edt = (unsigned)*(volatile unsigned long long*)(acc + QACC_EDT);
+        if (__shfl_sync(full, edt, 0) >> s & 1u) continue;
         const int64_t voxel = (int64_t)(id & ((1ull << 60) - 1ull));
         const int64_t row = voxel / G.W;
         const int x = (int)(voxel - row * G.W);
@@ -421,49 +441,56 @@ __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const u
         const int cy0 = y / QCELL, ct0 = t / QCELL;
         const int r_end = max(max(cy0, cy_n - 1 - cy0), max(ct0, ct_n - 1 - ct0));
         int32_t best = QINF;
-        for (int r = 0; r <= r_end; ++r) {
+        int steps = 0;
+        for (int r = 0; r <= r_end && steps <= FSTEPS; ++r) {
             const int ring = QCELL * (r - 1) + 1;
             if (r > 0 && ring * ring >= best) break;
-            const int rows = r == 0 ? 1 : 8 * r;
-            for (int j0 = 0; j0 < rows; j0 += 32) {
+            // the ring's cell rows within the video: its first and last frame of cells,
+            // then the ends of the frames between
+            const int y0 = max(cy0 - r, 0), ny = min(cy0 + r, cy_n - 1) - y0 + 1;
+            const int t0 = max(ct0 - r + 1, 0), nt = max(min(ct0 + r - 1, ct_n - 1) - t0 + 1, 0);
+            const bool low = cy0 >= r, high = cy0 + r < cy_n;
+            const int first_rows = ct0 >= r ? ny : 0;
+            const int sides = first_rows + (r > 0 && ct0 + r < ct_n ? ny : 0);
+            const int rows = sides + nt * ((int)low + (int)high);
+            for (int j0 = 0; j0 < rows && steps <= FSTEPS; j0 += 32) {
                 const int j = j0 + lane;
                 int32_t bound = QINF;      // no event of this lane's cell row is nearer,
                 int32_t within = QINF;     // and one of them is nearer than this
                 int cy = 0, ct = 0;
                 if (j < rows) {
-                    // two full sides of 2r + 1 cell rows, then pairs
-                    const int side = 2 * r + 1;
-                    if (j < 2 * side) {
-                        ct = ct0 + (j < side ? -r : r);
-                        cy = cy0 + (j < side ? j : j - side) - r;
+                    if (j < sides) {
+                        ct = ct0 + (j < first_rows ? -r : r);
+                        cy = y0 + (j < first_rows ? j : j - first_rows);
                     } else {
-                        const int p = j - 2 * side;
-                        ct = ct0 + (p >> 1) - r + 1;
-                        cy = cy0 + ((p & 1) ? r : -r);
+                        const int p = j - sides;
+                        const bool both = low && high;
+                        ct = t0 + (both ? p >> 1 : p);
+                        cy = (both ? (p & 1) != 0 : high) ? cy0 + r : cy0 - r;
                     }
-                    if (cy >= 0 && cy < cy_n && ct >= 0 && ct < ct_n) {
-                        const int dy = max(0, max(cy * QCELL - y, y - (cy * QCELL + QCELL - 1)));
-                        const int dt = max(0, max(ct * QCELL - t, t - (ct * QCELL + QCELL - 1)));
-                        const int32_t d = dy * dy + dt * dt;
-                        if (d < best) {
-                            const int32_t dx = cells_near(C + ((int64_t)ct * cy_n + cy) * sw, sw, x);
-                            if (dx < QINF) {
-                                const int uy = max(abs(cy * QCELL - y), abs(cy * QCELL + QCELL - 1 - y));
-                                const int ut = max(abs(ct * QCELL - t), abs(ct * QCELL + QCELL - 1 - t));
-                                bound = d + dx * dx;
-                                within = uy * uy + ut * ut + (dx + 31) * (dx + 31) + 1;
-                            }
+                    const int dy = max(0, max(cy * QCELL - y, y - (cy * QCELL + QCELL - 1)));
+                    const int dt = max(0, max(ct * QCELL - t, t - (ct * QCELL + QCELL - 1)));
+                    const int32_t d = dy * dy + dt * dt;
+                    if (d < best) {
+                        const int32_t dx = cells_near(C + ((int64_t)ct * cy_n + cy) * sw, sw, x);
+                        if (dx < QINF) {
+                            const int uy = max(abs(cy * QCELL - y), abs(cy * QCELL + QCELL - 1 - y));
+                            const int ut = max(abs(ct * QCELL - t), abs(ct * QCELL + QCELL - 1 - t));
+                            bound = d + dx * dx;
+                            within = uy * uy + ut * ut + (dx + 31) * (dx + 31) + 1;
                         }
                     }
                 }
+                steps += 1 + (sw >> 2);
                 best = min(best, __reduce_min_sync(full, within));
-                while (true) {
+                while (steps <= FSTEPS) {
                     const int32_t first = __reduce_min_sync(full, bound);
                     if (first >= best) break;
                     const int src = __ffs(__ballot_sync(full, bound == first)) - 1;
                     const int yy = __shfl_sync(full, cy, src) * QCELL + (lane & (QCELL - 1));
                     const int tt0 = __shfl_sync(full, ct, src) * QCELL + lane / QCELL;
                     if (lane == src) bound = QINF;
+                    steps += 1 + (int)(sqrtf((float)best) * (1.0f / 256.0f));
                     int32_t got = best;
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
@@ -476,6 +503,10 @@ __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const u
                 }
             }
         }
+        if (steps > FSTEPS) {
+            if (lane == 0) leave_to_edt(acc, s);
+            continue;
+        }
         // (the set's target has events, so one was found)
         if (lane != s) continue;
         ++closed;
@@ -487,16 +518,19 @@ __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const u
     }
     if (closed == 0) return;                         // (lanes from QSETS on, and warps without an event)
     unsigned long long* as = acc + QACC_SET + lane * QSET_WORDS;
-    atomicAdd(as + QSET_OPEN, 0ull - closed);
     if (matched) atomicAdd(as + QSET_MATCH, matched);
     if (sum != 0.0) atomicAdd(reinterpret_cast<double*>(as + QSET_SUM), sum);
 }
 
 // ---------------------------------------------------------------- rows: 1-D distance to the nearest event
 // One warp per row; `left` (shared) keeps the column of the nearest event at
-// or left of each x between the two sweeps.
-__global__ void k_edt_rows(const int8_t* __restrict__ v, int W, int64_t rows, int pol, int32_t* __restrict__ out) {
+// or left of each x between the two sweeps.  The first block also clears what the
+// searches left in the set's accumulators.
+__global__ void k_edt_rows(const int8_t* __restrict__ v, int W, int64_t rows, int pol, int32_t* __restrict__ out,
+                           unsigned long long* acc) {
     extern __shared__ int32_t q_left[];
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < QSET_WORDS; i += blockDim.x) acc[i] = 0;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     int32_t* left = q_left + (size_t)wib * W;
     for (int64_t r = (int64_t)blockIdx.x * wpb + wib; r < rows; r += (int64_t)gridDim.x * wpb) {
@@ -712,9 +746,14 @@ int64_t quality_cell_bytes(int32_t W, int32_t H, int32_t T) {
     return 4 * QSETS * sw * ((H + QCELL - 1) / QCELL) * ((T + QCELL - 1) / QCELL);
 }
 
-// Far events the list holds; more of them are cheaper to settle by the exact
-// transform (2.5 ms for one set of a 1280x720x100 video).
-int64_t quality_far_cap(int32_t W, int32_t H, int32_t T) { return (int64_t)W * H * T / 1024 + 1024; }
+// Far events the list holds.  Their search takes 1.6 ms per 80000 events of some
+// 100 steps each at 1280x720x100 (all four sets by the transform: 4 to 10 ms) and a
+// tenth of that for events a few cells away, so the list may hold this many before the
+// transform is the better bet; small videos' events have few cells to look at.
+// Unrelated random videos, whole calls with a list of voxels / 1024 + 1024, this one and four
+// transforms: 10^-3 events per voxel 1280x720x100 6.11 / 0.72 / 5.81 ms, 203x199x31 0.43 /
+// 0.09 / 0.37; 10^-2 8.26 / 8.13 / 7.95 (more than either holds) and 0.64 / 0.12 / 0.57.
+int64_t quality_far_cap(int32_t W, int32_t H, int32_t T) { return (int64_t)W * H * T / 512 + 16384; }
 
 cudaError_t launch_quality(const QualityArgs& A, int sms, cudaStream_t st, int* launches) {
     const int64_t n = (int64_t)A.W * A.H * A.T;
@@ -729,7 +768,7 @@ cudaError_t launch_quality(const QualityArgs& A, int sms, cudaStream_t st, int* 
     k_search<<<grid_of(G.n_words, 32 * QWARPS, sms, 32), 32 * QWARPS, 0, st>>>(G, A.masks, A.tau2, A.d2_a, A.d2_b,
                                                                             A.far_list, far_cap, A.acc);
     k_cells<<<sms * 8, QBLOCK, 0, st>>>(G, A.masks, A.cells, A.acc);
-    k_search_far<<<grid_of(far_cap, FWARPS, sms, 100), 32 * FWARPS, 0, st>>>(G, A.masks, A.cells, A.tau2, A.d2_a,
+    k_search_far<<<grid_of(n / 1024 + 1024, FWARPS, sms, 100), 32 * FWARPS, 0, st>>>(G, A.masks, A.cells, A.tau2, A.d2_a,
                                                                              A.d2_b, A.far_list, far_cap, A.acc);
     *launches += 4;
     return cudaGetLastError();
@@ -752,12 +791,12 @@ cudaError_t launch_quality_edt(const QualityArgs& A, int set, int sms, cudaStrea
     const int8_t* query = dir ? A.b : A.a;
     int32_t* d2_out = dir ? A.d2_b : A.d2_a;
     unsigned long long* acc = A.acc + QACC_SET + set * QSET_WORDS;
-    if ((e = cudaMemsetAsync(acc, 0, QSET_WORDS * sizeof(unsigned long long), st)) != cudaSuccess) return e;
     // rows: warps per block bounded by the shared budget (W ints per warp)
     const int wpb = (int)std::max<int64_t>(1, std::min<int64_t>(8, SMEM_BUDGET / (4 * W)));
     int32_t* cur = A.vol0;
     int32_t* other = A.vol1;
-    k_edt_rows<<<grid_of(H * T, wpb, sms, 16), 32 * wpb, (size_t)wpb * W * 4, st>>>(target, (int)W, H * T, pol, cur);
+    k_edt_rows<<<grid_of(H * T, wpb, sms, 16), 32 * wpb, (size_t)wpb * W * 4, st>>>(target, (int)W, H * T, pol, cur,
+                                                                                  acc);
     ++*launches;
     // column passes along y, then t
     const int64_t lines[2] = {T * W, H * W}, ostride[2] = {H * W, W}, stp[2] = {W, H * W};

@@ -21,13 +21,13 @@ enum {
     QACC_BAD = 1,       // nonzero if a value outside {-1, 0, 1} was seen
     QACC_COUNT = 2,     // events per set's query: a+, a-, b+, b-
     QACC_FAR = 6,       // events listed for the far search
+    QACC_EDT = 7,       // bit s: set s is left to the exact transform
     QACC_SET = 8,       // per set: QSET_WORDS
     QSET_MATCH = 0,     // events within sqrt(tau2)
     QSET_NONE = 1,      // events whose polarity the other video lacks
     QSET_SUM = 2,       // double: sum of the distances with d^2 >= QHIST
-    QSET_OPEN = 3,      // events the searches have not settled
-    QSET_HIST = 4,      // counts per squared distance 1..QHIST-1 (index = d^2)
-    QSET_WORDS = 4 + QHIST,
+    QSET_HIST = 3,      // counts per squared distance 1..QHIST-1 (index = d^2)
+    QSET_WORDS = 3 + QHIST,
     QACC_WORDS = QACC_SET + QSETS * QSET_WORDS
 };
 
@@ -42,7 +42,7 @@ struct QualityArgs {
     uint32_t* cells;             // quality_cell_bytes() of scratch: occupied cells of the masks
     uint64_t* far_list;          // quality_far_cap() entries: events whose nearest is not in the window
     unsigned long long* acc;     // QACC_WORDS words
-    // exact transform of the sets with open events (launch_quality_edt)
+    // exact transform of the sets in QACC_EDT (launch_quality_edt)
     int32_t* vol0;               // scratch volumes, W*H*T int32 each
     int32_t* vol1;
     void* stack;                 // quality_stack_bytes() of scratch for long-line envelopes
