@@ -109,7 +109,8 @@ struct mcev_ctx {
     float static_lo[3], static_hi[3];
 
     // device scene
-    DevBuf d_quality;                       // event-quality scratch: accumulators, event bits, far events
+    DevBuf d_qacc;                          // event-quality accumulators
+    DevBuf d_quality;                       // event-quality scratch of the searches: event bits, cells, far events
     DevBuf d_qedt;                          // its distance transform: two int32 volumes, envelope stacks
     DevBuf d_gemit;                         // FP64 emission-gradient accumulator of mcev_backward
     DevBuf d_nodes, d_wnodes, d_tris, d_tshade, d_uv, d_mats, d_env, d_marg, d_cond, d_tpdf;
@@ -1202,7 +1203,7 @@ void mcev_destroy(mcev_ctx* ctx) {
     cudaStreamSynchronize(ctx->stream);
     DevBuf* bufs[] = {&ctx->d_nodes, &ctx->d_wnodes, &ctx->d_tris, &ctx->d_tshade, &ctx->d_uv, &ctx->d_mats, &ctx->d_env, &ctx->d_marg, &ctx->d_cond,
                       &ctx->d_tpdf, &ctx->frames[0].buf, &ctx->frames[1].buf, &ctx->d_wave, &ctx->d_counters,
-                      &ctx->d_pix, &ctx->d_tcrit, &ctx->d_jobs, &ctx->d_bqueue, &ctx->d_quality, &ctx->d_qedt, &ctx->d_gemit,
+                      &ctx->d_pix, &ctx->d_tcrit, &ctx->d_jobs, &ctx->d_bqueue, &ctx->d_qacc, &ctx->d_quality, &ctx->d_qedt, &ctx->d_gemit,
                       &ctx->d_round};
     for (DevBuf* b : bufs) dev_free(ctx, *b);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
@@ -1732,12 +1733,27 @@ mcev_status mcev_event_quality(mcev_ctx* ctx, const int8_t* a, const int8_t* b, 
     if (tau2 < 0) return fail(ctx, MCEV_ERR_ARG, "tau2 must be >= 0");
     CU(cudaSetDevice(ctx->device));
     const int64_t n = (int64_t)width * height * frames;
+    for (int k = 0; k < 2 && width == 1; ++k) {
+        // the same voxels in rows of `height` (the masks' rows are whole words; all axes count alike)
+        width = height;
+        height = frames;
+        frames = 1;
+    }
+    // the searches' scratch and the transform's are not in use at the same time: where there
+    // is no memory for one beside the other, the other is given back
+    auto either = [&](DevBuf& want, size_t bytes, DevBuf& other) -> mcev_status {
+        const mcev_status st = dev_alloc(ctx, want, bytes);
+        if (st != MCEV_ERR_OOM || !other.ptr) return st;
+        dev_free(ctx, other);
+        return dev_alloc(ctx, want, bytes);
+    };
     auto al = [](int64_t x) { return ((size_t)x + 255) & ~size_t(255); };
     const size_t nb_acc = QACC_WORDS * sizeof(unsigned long long);
     const size_t nb_mask = al(quality_mask_bytes(width, height, frames));
     const size_t nb_cell = al(quality_cell_bytes(width, height, frames));
     const size_t nb_far = 8 * (size_t)quality_far_cap(width, height, frames);
-    ST(dev_alloc(ctx, ctx->d_quality, al(nb_acc) + nb_mask + nb_cell + nb_far));
+    ST(dev_alloc(ctx, ctx->d_qacc, nb_acc));
+    ST(either(ctx->d_quality, nb_mask + nb_cell + nb_far, ctx->d_qedt));
     char* base = (char*)ctx->d_quality.ptr;
     QualityArgs A{};
     A.a = a;
@@ -1748,10 +1764,10 @@ mcev_status mcev_event_quality(mcev_ctx* ctx, const int8_t* a, const int8_t* b, 
     A.tau2 = tau2;
     A.d2_a = d2_a;
     A.d2_b = d2_b;
-    A.acc = (unsigned long long*)base;
-    A.masks = (uint32_t*)(base + al(nb_acc));
-    A.cells = (uint32_t*)(base + al(nb_acc) + nb_mask);
-    A.far_list = (uint64_t*)(base + al(nb_acc) + nb_mask + nb_cell);
+    A.acc = (unsigned long long*)ctx->d_qacc.ptr;
+    A.masks = (uint32_t*)base;
+    A.cells = (uint32_t*)(base + nb_mask);
+    A.far_list = (uint64_t*)(base + nb_mask + nb_cell);
     int nl = 0;
     std::vector<unsigned long long> acc(QACC_WORDS);
     auto read_acc = [&]() -> mcev_status {
@@ -1770,7 +1786,7 @@ mcev_status mcev_event_quality(mcev_ctx* ctx, const int8_t* a, const int8_t* b, 
     for (int set = 0; set < QSETS; ++set) {
         if (!(acc[QACC_EDT] >> set & 1ull)) continue;
         const size_t vol = al(4 * n);
-        ST(dev_alloc(ctx, ctx->d_qedt, 2 * vol + al(quality_stack_bytes(width, height, frames, ctx->sms))));
+        ST(either(ctx->d_qedt, 2 * vol + al(quality_stack_bytes(width, height, frames, ctx->sms)), ctx->d_quality));
         A.vol0 = (int32_t*)ctx->d_qedt.ptr;
         A.vol1 = (int32_t*)((char*)ctx->d_qedt.ptr + vol);
         A.stack = (char*)ctx->d_qedt.ptr + 2 * vol;
