@@ -1776,29 +1776,30 @@ mcev_status mcev_event_quality(mcev_ctx* ctx, const int8_t* a, const int8_t* b, 
         ctx->d2h += (int64_t)nb_acc;
         return MCEV_OK;
     };
+    // device time of the kernels; reading the accumulators and allocating in between is not part of it
+    float ms = 0.0f;
     CU(cudaEventRecord(ctx->ev0, ctx->stream));
     CU(launch_quality(A, ctx->sms, ctx->stream, &nl));
     CU(cudaEventRecord(ctx->ev1, ctx->stream));
     ST(read_acc());
+    CU(cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
     if (acc[QACC_BAD]) return fail(ctx, MCEV_ERR_ARG, "event values must be -1, 0 or +1");
     // sets with more far events than the list holds, or too far ones: exact distance transform
-    bool again = false;
-    for (int set = 0; set < QSETS; ++set) {
-        if (!(acc[QACC_EDT] >> set & 1ull)) continue;
+    if (acc[QACC_EDT]) {
         const size_t vol = al(4 * n);
         ST(either(ctx->d_qedt, 2 * vol + al(quality_stack_bytes(width, height, frames, ctx->sms)), ctx->d_quality));
         A.vol0 = (int32_t*)ctx->d_qedt.ptr;
         A.vol1 = (int32_t*)((char*)ctx->d_qedt.ptr + vol);
         A.stack = (char*)ctx->d_qedt.ptr + 2 * vol;
-        CU(launch_quality_edt(A, set, ctx->sms, ctx->stream, &nl));
-        again = true;
-    }
-    if (again) {
+        CU(cudaEventRecord(ctx->ev0, ctx->stream));
+        for (int set = 0; set < QSETS; ++set)
+            if (acc[QACC_EDT] >> set & 1ull) CU(launch_quality_edt(A, set, ctx->sms, ctx->stream, &nl));
         CU(cudaEventRecord(ctx->ev1, ctx->stream));
         ST(read_acc());
+        float edt_ms = 0.0f;
+        CU(cudaEventElapsedTime(&edt_ms, ctx->ev0, ctx->ev1));
+        ms += edt_ms;
     }
-    float ms = 0.0f;
-    CU(cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
     mcev_quality q{};
     q.voxels = n;
     q.n_a = (int64_t)(acc[QACC_COUNT] + acc[QACC_COUNT + 1]);

@@ -105,3 +105,20 @@ def test_narrow_videos_need_no_more_than_the_transform_did(shape):
     # (the list of far events: 128 KiB + 1/64 byte per voxel)
     assert c.peak <= _transform_bytes(W, H, T) + (256 << 10)
     c.close()
+
+
+def test_device_time_does_not_cover_the_allocations():
+    import time
+    a, b = _far_apart((200, 100, 40))
+    c = Limited(1 << 40)
+    first = c.cb[0]
+
+    def slow(n, user):
+        time.sleep(0.1)
+        return first(n, user)
+
+    c.slow = L.ALLOC_FN(slow)
+    assert c.lib.mcev_set_allocator(c.ctx, c.slow, c.cb[1], None) == 0
+    g = c.quality(a, b)                             # one allocation is between the searches and the transform
+    assert g["kernel_launches"] > 4 and 0.0 < g["gpu_ms"] < 50.0
+    c.close()
