@@ -116,7 +116,9 @@ typedef struct {
                              spp_batch per undecided pixel at once, merging and testing them in
                              order; samples after a pixel's decision are unused (a round adds about
                              a quarter of a pixel's samples, more when that would leave the GPU
-                             idle, never more than fill the wavefront).  1 = one batch per round; 0 = library default (16). */
+                             idle, never more than fill the wavefront; uniform sampling, which
+                             decides at spp_max only, always fills it).  1 = one batch per round;
+                             0 = library default (16). */
     int32_t bvh_width;  /* node layout of the per-mesh BVHs: 2 (two children per node) or 8
                            (compressed 8-wide nodes with 8-bit child boxes); 0 = library default.
                            Changing it rebuilds the BVHs of an uploaded scene.  Results are the

@@ -890,6 +890,7 @@ mcev_status run_rounds_device(mcev_ctx* ctx, const Frame& fr, StatsArgs A, int64
     plan.spp_max = A.spp_max;
     plan.window_max = ctx->params.batch_window > 0 ? ctx->params.batch_window : 16;
     const int64_t tus = ctx->params.device_timeout_us > 0 ? ctx->params.device_timeout_us : kDefaultDeviceTimeoutUs;
+    plan.uniform = A.variant == VAR_UNIFORM ? 1 : 0;
     plan.timeout_ns = (unsigned long long)tus * 1000ull;
     // chunks the schedule can need: rounds x chunks of the largest round
     const int64_t first = std::min(A.spp_min, A.spp_max);
@@ -1043,7 +1044,8 @@ mcev_status run_rounds(mcev_ctx* ctx, const Frame& fr, StatsArgs A, int64_t* pat
             spp_r = sub = std::min(A.spp_min, A.spp_max);
         } else {
             sub = A.spp_batch;
-            const int64_t m = round_window(ctx->wave.cap, Q, sub, n_done, A.spp_max, window_max);
+            const int64_t m = round_window(ctx->wave.cap, Q, sub, n_done, A.spp_max, window_max,
+                                           A.variant == VAR_UNIFORM);
             spp_r = (int32_t)std::min<int64_t>(m * sub, A.spp_max - n_done);
         }
         NvtxRange round_range("mcev round");

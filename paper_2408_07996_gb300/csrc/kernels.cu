@@ -1180,7 +1180,8 @@ __global__ void __launch_bounds__(REQUEUE_BLOCK) k_round_next(RoundCtl* rc, Wave
             go = 0;
         } else {
             const int64_t sub = plan.spp_batch;
-            const int64_t m = round_window(plan.cap, q, sub, rc->n_done, plan.spp_max, plan.window_max);
+            const int64_t m = round_window(plan.cap, q, sub, rc->n_done, plan.spp_max, plan.window_max,
+                                           plan.uniform != 0);
             rc->sub = (int32_t)sub;
             rc->spp_r = (int32_t)min(m * sub, (int64_t)plan.spp_max - rc->n_done);
             round_first_chunk(rc, plan);

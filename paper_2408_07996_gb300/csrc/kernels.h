@@ -59,7 +59,7 @@ struct RoundPlan {
     int64_t Q0;               // pixels queued in the first round
     int32_t spp_min, spp_batch, spp_max, window_max;
     int32_t max_iters;        // chunks after which the loop gives up (RC_TIMEOUT)
-    int32_t pad;
+    int32_t uniform;          // 1: no pixel is decided before spp_max (VAR_UNIFORM)
     unsigned long long timeout_ns;  // wall-clock bound of the loop (RC_TIMEOUT)
 };
 
@@ -78,14 +78,17 @@ struct RoundPlan {
 // 132 / 137 ms; at a quarter with 2^17, 2^19, 2^20, 2^21 paths the 346x260 frame
 // takes 14.8, 12.9, 12.2, 12.5 ms.
 constexpr int64_t ROUND_FILL = (int64_t)1 << 20;
+// Uniform sampling (`uniform`) decides at the cap only, traces nothing in vain and
+// fills the wavefront: sphere field 346x260 to 1024 samples 57.3 (19 rounds) -> 48.5 ms (5),
+// 128x96 to 2048 20.0 -> 15.7, 640x480 to 4096 659 -> 650, terrain 640x360 328 -> 322.
 MCEV_HD inline int64_t round_window(int64_t cap, int64_t q, int64_t sub, int64_t n_done, int64_t spp_max,
-                                    int64_t window_max) {
+                                    int64_t window_max, bool uniform) {
     const int64_t left = (spp_max - n_done + sub - 1) / sub;
     const int64_t per_batch = q * sub;
     const int64_t fill = (ROUND_FILL + per_batch - 1) / per_batch;
     int64_t m = n_done / (4 * sub);
     if (m < fill) m = fill;
-    if (m > cap / per_batch) m = cap / per_batch;
+    if (uniform || m > cap / per_batch) m = cap / per_batch;
     if (m > left) m = left;
     if (m > window_max) m = window_max;
     return m < 1 ? 1 : m;
