@@ -404,20 +404,22 @@ __device__ __forceinline__ int32_t cells_near(const uint32_t* __restrict__ row, 
 // addition per warp to the set's words instead of one per event.
 //
 // The transform costs the same wherever the events are, this search the more the
-// farther they are, so an event may take FSTEPS steps (a step: 32 cell rows of a
-// ring, or the search of one cell row; wide rows count by their length).  An event that
-// is not settled then leaves its set to the transform, and the set's other events are
-// skipped.  Whole calls at 64 / 128 / 256 steps: 80000 events of 1280x720x100 100 rows from
-// the other video's 0.57 / 0.57 / 0.57 ms, 500 rows 2.72 / 1.61 / 1.62 (four transforms 3.96),
-// opposite ends of 64x64x8192 3.64 / 3.78 / 4.09 (5.46), 250000 events of 16384x16384x1
-// against one in a corner 31.0 / 13.6 / 13.6 (55.1).
+// farther they are.  An event may take FSTEPS steps (a step: 32 cell rows of a ring, or the
+// search of one cell row; wide rows count by their length), and all events together
+// `budget` beyond their first 64 (most take 10 to 30, the farthest of a video a
+// hundred or two).  An event that is not settled then leaves its set to the
+// transform, and the set's other events are skipped.  Whole calls / four transforms:
+// 80000 events of 1280x720x100 500 rows from the other video's 1.74 / 3.96 ms, opposite ends
+// of 64x64x8192 4.35 / 5.46, 250000 events of 16384x16384x1 against one in a corner 13.8 /
+// 55.1.  128 steps and no common budget: 1.61, 3.78 and 13.6 ms, but one 1280x720x100
+// drifting grating in fifteen went to the transform for an event of 130 steps (0.67 -> 2.03).
 constexpr int FWARPS = 2;
-constexpr int FSTEPS = 128;
+constexpr int FSTEPS = 512;
 __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const uint32_t* __restrict__ masks,
                                                                 const uint32_t* __restrict__ cells, int tau2,
                                                                 int32_t* __restrict__ d2_a, int32_t* __restrict__ d2_b,
                                                                 const uint64_t* __restrict__ far_list, int64_t far_cap,
-                                                                unsigned long long* acc) {
+                                                                int64_t budget, unsigned long long* acc) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int64_t n = min((int64_t)acc[QACC_FAR], far_cap);
@@ -442,6 +444,16 @@ __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const u
         const int r_end = max(max(cy0, cy_n - 1 - cy0), max(ct0, ct_n - 1 - ct0));
         int32_t best = QINF;
         int steps = 0;
+        auto spend = [&](int k) {
+            const int before = steps;
+            steps += k;
+            if ((before ^ steps) >> 6 == 0) return;
+            int stop = 0;      // (the whole warp is here)
+            if (lane == 0)
+                stop = (int64_t)atomicAdd(acc + QACC_STEPS, 64ull) >= budget ||
+                       (*(volatile unsigned long long*)(acc + QACC_EDT) >> s & 1ull) != 0;
+            if (__shfl_sync(full, stop, 0)) steps = FSTEPS + 1;
+        };
         for (int r = 0; r <= r_end && steps <= FSTEPS; ++r) {
             const int ring = QCELL * (r - 1) + 1;
             if (r > 0 && ring * ring >= best) break;
@@ -481,7 +493,7 @@ __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const u
                         }
                     }
                 }
-                steps += 1 + (sw >> 2);
+                spend(1 + (sw >> 2));
                 best = min(best, __reduce_min_sync(full, within));
                 while (steps <= FSTEPS) {
                     const int32_t first = __reduce_min_sync(full, bound);
@@ -490,7 +502,7 @@ __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const u
                     const int yy = __shfl_sync(full, cy, src) * QCELL + (lane & (QCELL - 1));
                     const int tt0 = __shfl_sync(full, ct, src) * QCELL + lane / QCELL;
                     if (lane == src) bound = QINF;
-                    steps += 1 + (int)(sqrtf((float)best) * (1.0f / 256.0f));
+                    spend(1 + (int)(sqrtf((float)best) * (1.0f / 256.0f)));
                     int32_t got = best;
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
@@ -746,13 +758,13 @@ int64_t quality_cell_bytes(int32_t W, int32_t H, int32_t T) {
     return 4 * QSETS * sw * ((H + QCELL - 1) / QCELL) * ((T + QCELL - 1) / QCELL);
 }
 
-// Far events the list holds.  Their search takes 1.6 ms per 80000 events of some
+// Far events the list holds.  Their search takes 1.5 ms per 80000 events of some
 // 100 steps each at 1280x720x100 (all four sets by the transform: 4 to 10 ms) and a
 // tenth of that for events a few cells away, so the list may hold this many before the
 // transform is the better bet; small videos' events have few cells to look at.
 // Unrelated random videos, whole calls with a list of voxels / 1024 + 1024, this one and four
-// transforms: 10^-3 events per voxel 1280x720x100 6.11 / 0.72 / 5.81 ms, 203x199x31 0.43 /
-// 0.09 / 0.37; 10^-2 8.26 / 8.13 / 7.95 (more than either holds) and 0.64 / 0.12 / 0.57.
+// transforms: 10^-3 events per voxel 1280x720x100 6.11 / 0.75 / 5.81 ms, 203x199x31 0.43 /
+// 0.09 / 0.37; 10^-2 8.26 / 8.12 / 7.95 (more than either holds) and 0.64 / 0.12 / 0.57.
 int64_t quality_far_cap(int32_t W, int32_t H, int32_t T) { return (int64_t)W * H * T / 512 + 16384; }
 
 cudaError_t launch_quality(const QualityArgs& A, int sms, cudaStream_t st, int* launches) {
@@ -769,7 +781,8 @@ cudaError_t launch_quality(const QualityArgs& A, int sms, cudaStream_t st, int* 
                                                                             A.far_list, far_cap, A.acc);
     k_cells<<<sms * 8, QBLOCK, 0, st>>>(G, A.masks, A.cells, A.acc);
     k_search_far<<<grid_of(n / 1024 + 1024, FWARPS, sms, 100), 32 * FWARPS, 0, st>>>(G, A.masks, A.cells, A.tau2, A.d2_a,
-                                                                             A.d2_b, A.far_list, far_cap, A.acc);
+                                                                             A.d2_b, A.far_list, far_cap, n / 8 + 65536,
+                                                                                       A.acc);
     *launches += 4;
     return cudaGetLastError();
 }

@@ -22,7 +22,8 @@ enum {
     QACC_COUNT = 2,     // events per set's query: a+, a-, b+, b-
     QACC_FAR = 6,       // events listed for the far search
     QACC_EDT = 7,       // bit s: set s is left to the exact transform
-    QACC_SET = 8,       // per set: QSET_WORDS
+    QACC_STEPS = 8,     // steps of the far search beyond the first 64 of an event
+    QACC_SET = 9,       // per set: QSET_WORDS
     QSET_MATCH = 0,     // events within sqrt(tau2)
     QSET_NONE = 1,      // events whose polarity the other video lacks
     QSET_SUM = 2,       // double: sum of the distances with d^2 >= QHIST

@@ -1,6 +1,6 @@
 """Where the event-video searches change path: two rings and 15 columns around an
 event (settled up to d^2 = 9), cells of 32 columns x 8 rows x 8 frames for the
-listed events, at most voxels / 512 + 16384 of them and 128 steps each, and the
+listed events, at most voxels / 512 + 16384 of them and 512 steps each, and the
 exact transform for the sets beyond.  Counts and squared distances are integers
 and equal the FP64 oracle's (or the closed form's)."""
 import numpy as np
@@ -66,18 +66,48 @@ def test_as_many_far_events_as_the_list_holds(over):
 
 
 def test_opposite_ends_of_a_long_video_go_to_the_transform():
-    """A search ring by ring would visit 250 rings for every event."""
-    shape = (2048, 16, 64)
+    """A search ring by ring would visit 740 rings for every event."""
+    shape = (6000, 16, 24)
     rng = np.random.default_rng(2)
     a, b = np.zeros(shape, np.int8), np.zeros(shape, np.int8)
-    a[:40] = rng.random((40, 16, 64)) < 0.01
-    b[-40:] = rng.random((40, 16, 64)) < 0.01
+    a[:40] = rng.random((40, 16, 24)) < 0.01
+    b[-40:] = rng.random((40, 16, 24)) < 0.01
     # the other polarity has its counterparts near by: the searches settle it
-    a[1000:1010] -= (rng.random((10, 16, 64)) < 0.05).astype(np.int8)
-    b[1010:1022] -= (rng.random((12, 16, 64)) < 0.05).astype(np.int8)
+    a[1000:1010] -= (rng.random((10, 16, 24)) < 0.05).astype(np.int8)
+    b[1010:1022] -= (rng.random((12, 16, 24)) < 0.05).astype(np.int8)
     g, _ = _compare(a, b)
     assert g["kernel_launches"] == SEARCHES + 2 * 4
-    assert int(g["d2_a"].max()) > 1900 ** 2
+    assert int(g["d2_a"].max()) > 5900 ** 2
+
+
+def test_a_far_event_among_near_ones_does_not_need_the_transform():
+    """One event in thousands whose nearest is some 200 steps away is searched for all the
+    same: 25 rings of an empty volume, with occupied cell rows all around at one distance."""
+    shape = (60, 420, 64)
+    rng = np.random.default_rng(4)
+    T, H, W = shape
+    t, y, x = np.mgrid[:T, :H, :W]
+    a, b = np.zeros(shape, np.int8), np.zeros(shape, np.int8)
+    shell = ((t - 30) ** 2 + (y - 210) ** 2 > 200 ** 2) & (rng.random(shape) < 0.02)
+    a[shell] = 1
+    b[shell] = 1
+    move = shell & (rng.random(shape) < 0.2)
+    a[move] = 0
+    a[30, 210, 32] = 1
+    g, _ = _compare(a, b)
+    assert g["kernel_launches"] == SEARCHES
+    assert int(g["d2_a"].max()) > 199 ** 2
+
+
+def test_many_far_events_spend_the_budget():
+    """Thousands of events some 300 steps away: together more than voxels / 8 + 65536 steps."""
+    shape = (2600, 24, 16)
+    rng = np.random.default_rng(5)
+    a, b = np.zeros(shape, np.int8), np.zeros(shape, np.int8)
+    a[:20] = rng.random((20, 24, 16)) < 0.2
+    b[-20:] = rng.random((20, 24, 16)) < 0.2
+    g, _ = _compare(a, b)
+    assert g["kernel_launches"] > SEARCHES
 
 
 @pytest.mark.parametrize("shape", [(1, 3000, 2500), (1, 64, 16384), (3000, 2, 40), (64, 2000, 1)])
