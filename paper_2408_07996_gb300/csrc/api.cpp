@@ -814,7 +814,6 @@ DevParams dev_params(const mcev_ctx* ctx, bool want_sig) {
         ST(ev_mark(ctx, cls, false));                                                                 \
     } while (0)
 
-// one chunk of n_paths = nj * spp_r paths through every bounce
 // Batched render (several contexts' frame pairs in one set of rounds): the
 // device job table, the union queues of (job << 24 | pixel) entries, and the
 // largest depth / any NEE over the jobs (the per-path kernels use each job's

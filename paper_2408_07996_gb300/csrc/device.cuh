@@ -720,37 +720,34 @@ __device__ __forceinline__ void two_level(const DevScene& sc, const DevFrame& fr
                 base = sp;
             }
         }
-#ifndef MCEV_TL_STEPS
-#define MCEV_TL_STEPS 2
-#endif
 #pragma unroll
-        for (int step = 0; step < MCEV_TL_STEPS; ++step) {
-        if (pcount == 0 && node != MCEV_NO_NODE && (in_blas || pend0 < 0)) {
-            const Node n = load_node(in_blas ? sc.nodes : fr.tlas, node);
-            work.x += 1;
-            float tl, tr;
-            const int m = node_hits(r, n, tmin, h.t, tl, tr);
-            const bool lh = (m & 1) && n.d.x < 0, rh = (m & 2) && n.d.y < 0;
-            if (in_blas) {
-                pfirst = lh ? ~n.d.x : ~n.d.y;
-                pcount = (lh ? n.d.z : 0) + (rh ? n.d.w : 0);
-            } else {
-                pend0 = lh ? ~n.d.x : (rh ? ~n.d.y : -1);
-                pend1 = (lh && rh) ? ~n.d.y : -1;
+        for (int step = 0; step < MCEV_NODE_STEPS; ++step) {
+            if (pcount == 0 && node != MCEV_NO_NODE && (in_blas || pend0 < 0)) {
+                const Node n = load_node(in_blas ? sc.nodes : fr.tlas, node);
+                work.x += 1;
+                float tl, tr;
+                const int m = node_hits(r, n, tmin, h.t, tl, tr);
+                const bool lh = (m & 1) && n.d.x < 0, rh = (m & 2) && n.d.y < 0;
+                if (in_blas) {
+                    pfirst = lh ? ~n.d.x : ~n.d.y;
+                    pcount = (lh ? n.d.z : 0) + (rh ? n.d.w : 0);
+                } else {
+                    pend0 = lh ? ~n.d.x : (rh ? ~n.d.y : -1);
+                    pend1 = (lh && rh) ? ~n.d.y : -1;
+                }
+                const bool gl = (m & 1) && n.d.x >= 0 && (kAny || tl <= h.t);
+                const bool gr = (m & 2) && n.d.y >= 0 && (kAny || tr <= h.t);
+                node = gl ? n.d.x : n.d.y;
+                if (gl && gr) {
+                    if (sp < MCEV_STACK) stack[sp++] = tl <= tr ? n.d.y : n.d.x;
+                    else atomicOr(err, 1);
+                    node = tl <= tr ? n.d.x : n.d.y;
+                } else if (!(gl || gr)) {
+                    // within the level; a finished BLAS and pending instances are handled above
+                    node = MCEV_NO_NODE;
+                    if (in_blas ? sp > base : (sp > 0 && pend0 < 0)) node = stack[--sp];
+                }
             }
-            const bool gl = (m & 1) && n.d.x >= 0 && (kAny || tl <= h.t);
-            const bool gr = (m & 2) && n.d.y >= 0 && (kAny || tr <= h.t);
-            node = gl ? n.d.x : n.d.y;
-            if (gl && gr) {
-                if (sp < MCEV_STACK) stack[sp++] = tl <= tr ? n.d.y : n.d.x;
-                else atomicOr(err, 1);
-                node = tl <= tr ? n.d.x : n.d.y;
-            } else if (!(gl || gr)) {
-                // within the level; a finished BLAS and pending instances are handled above
-                node = MCEV_NO_NODE;
-                if (in_blas ? sp > base : (sp > 0 && pend0 < 0)) node = stack[--sp];
-            }
-        }
         }
         if (pcount > 0) {
             work.y += 1;

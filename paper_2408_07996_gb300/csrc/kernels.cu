@@ -7,9 +7,8 @@
 // counters, no host round trip) that shade fills tile by tile in direction
 // order.  `stats` fuses, per queued pixel, the log-luminance batch statistics
 // (Sec. 3.1, Eq. 3-4), the Chan merge into the running statistics, the t-test
-// of Eq. 7 (Sec. 3.2), the re-queue of undecided pixels (Sec. 3.3; one atomic
-// per warp) and the event rule with the reference
-// update (Alg. 1, Eq. 1).
+// of Eq. 7 (Sec. 3.2), a bit for the re-queue of undecided pixels in order
+// (Sec. 3.3) and the event rule with the reference update (Alg. 1, Eq. 1).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -1108,7 +1107,7 @@ static cudaError_t launch_stats_checked(const Wave& w, const StatsArgs& A, const
 // ------------------------------------------------------------------ device-resident round loop
 // The rounds of Alg. 1's sampling schedule (Sec. 3.3) without the host: a
 // CUDA graph runs k_round_init, then a conditional WHILE node whose body is
-// one wavefront chunk (raygen, bounces, statistics) followed by
+// one wavefront chunk (bounces, statistics) followed by
 // k_round_next, which moves to the next chunk of the round or, at the end
 // of a round, reads the number of re-queued pixels and sizes the next round
 // (first round spp_min samples, then windows of spp_batch batches:

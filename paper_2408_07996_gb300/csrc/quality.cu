@@ -6,7 +6,7 @@
 // Two event videos of one scene differ by little: most events have their
 // counterpart in the same voxel and nearly all within a few.  So both videos are
 // first packed into bit masks (one bit per voxel, polarity and video: 1/2 byte
-// per voxel, which stays in L2), events whose own bit is set in the target are
+// per voxel and rows padded to 32 columns, which stays in L2), events whose own bit is set in the target are
 // counted by AND and population count, and only the rest search the target's
 // rows around them ring by ring until no nearer event can exist.  Events
 // without a neighbour in two rings and 15 columns are listed and searched for by a warp
@@ -127,9 +127,11 @@ __device__ __forceinline__ void pack32(const uint32_t v[8], uint32_t& pos, uint3
     }
 }
 
-// One thread packs 32 voxels of a row of both videos and tallies them.  HBM
-// bound: 2 B read and 1/2 B written per voxel; 1280x720x100 in 69 us (3.1
-// TB/s) against 75 us for the tally alone one voxel at a time.
+// One thread packs 32 voxels of a row of both videos and tallies them: 2 B read and
+// 1/2 B written per voxel (rows are padded to whole words).  1280x720x100 in 68 us, 3.4
+// TB/s, half of the measured copy rate (6.67 TB/s): bound by the latency of its few loads
+// in flight (two or four 16-byte ones per thread and step) and the compares and multiplies
+// that pack them.  The tally alone, one voxel at a time, took 75 us.
 __global__ void __launch_bounds__(QBLOCK) k_pack(const int8_t* __restrict__ a, const int8_t* __restrict__ b, int W,
                                                  int ww, int64_t n_words, int64_t n, uint32_t* __restrict__ masks,
                                                  unsigned long long* acc) {
@@ -169,6 +171,7 @@ struct QGrid {
 };
 constexpr int QNEAR = 15;     // columns of the first search's window
 constexpr int QRINGS = 2;      // its rings (a 1280x720x100 call at 1 / 2 / 3 / 5 rings: 0.80 / 0.81 / 0.89 / 1.14 ms)
+constexpr int QSETTLED = (QRINGS + 1) * (QRINGS + 1);   // what it has not looked at is this far away at least
 // cells of the far search: 32 columns (a mask word) x 8 rows x 8 frames; a warp
 // reads a cell row's 64 rows two per lane
 constexpr int QCELL = 8;
@@ -236,8 +239,8 @@ __global__ void __launch_bounds__(32 * QWARPS) k_search(QGrid G, const uint32_t*
                                                        uint64_t* __restrict__ far_list, int64_t far_cap,
                                                        unsigned long long* acc) {
     __shared__ uint16_t todo[QWARPS][2048];     // word << 5 | bit, + set << 10; a voxel is in at most 2 sets
-    __shared__ uint32_t hist[QSETS][256];       // squared distances settled here are below 256
-    for (int i = threadIdx.x; i < QSETS * 256; i += blockDim.x) (&hist[0][0])[i] = 0;
+    __shared__ uint32_t hist[QSETS][QSETTLED + 1];
+    for (int i = threadIdx.x; i < QSETS * (QSETTLED + 1); i += blockDim.x) (&hist[0][0])[i] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     // no event to search for, or none that is worth it: earlier blocks have left the set to
@@ -310,9 +313,9 @@ __global__ void __launch_bounds__(32 * QWARPS) k_search(QGrid G, const uint32_t*
                     }
                 }
             }
-            // anything not looked at is at least QRINGS + 1 rings away (or more than QNEAR columns)
+            // (what was not looked at is at least QRINGS + 1 rings or QNEAR + 1 columns away)
             const int64_t voxel = row * G.W + x;
-            if (best <= (QRINGS + 1) * (QRINGS + 1)) {
+            if (best <= QSETTLED) {
                 if (best <= tau2) ++matched[0 + s];
                 atomicAdd(&hist[s][best], 1u);
                 int32_t* d2 = s < 2 ? d2_a : d2_b;
@@ -334,7 +337,7 @@ __global__ void __launch_bounds__(32 * QWARPS) k_search(QGrid G, const uint32_t*
         unsigned long long* as = acc + QACC_SET + s * QSET_WORDS;
         block_flush(matched[s], none[s], 0ull, 0.0, as, QSET_MATCH, QSET_NONE, -1, -1);
         __syncthreads();
-        for (int b = threadIdx.x; b < 256; b += blockDim.x)
+        for (int b = threadIdx.x; b <= QSETTLED; b += blockDim.x)
             if (b > 0 && hist[s][b]) atomicAdd(as + QSET_HIST + b, (unsigned long long)hist[s][b]);
     }
 }
@@ -396,8 +399,8 @@ __device__ __forceinline__ int32_t cells_near(const uint32_t* __restrict__ row, 
 // could hold a nearer event the nearest is searched first, its 64 rows two per
 // lane.  Bound by the dependent loads of one event after the other and some 4000
 // instructions each.  Events differ widely in cost, so the blocks are small and up
-// to five times as many as are resident (20 of 64 threads, 48 registers, no
-// spills): whole quality calls of 1280x720x100, two videos, 0.79 and 0.71 ms with 8
+// to five times as many as are resident (20 of 64 threads, 48 registers, one
+// spilled): whole quality calls of 1280x720x100, two videos, 0.79 and 0.71 ms with 8
 // blocks of 256 threads per SM, 0.72 and 0.66 ms with 40, 0.69 and 0.62 ms with 100
 // blocks of 64, the same with 300 or with a cursor on the device; 0.72 and
 // 0.65 ms with 40 registers.  Lane s adds up what its warp found for set s: one
