@@ -399,25 +399,27 @@ __device__ __forceinline__ int32_t cells_near(const uint32_t* __restrict__ row, 
 // could hold a nearer event the nearest is searched first, its 64 rows two per
 // lane.  Bound by the dependent loads of one event after the other and some 4000
 // instructions each.  Events differ widely in cost, so the blocks are small and up
-// to five times as many as are resident (20 of 64 threads, 48 registers, one
-// spilled): whole quality calls of 1280x720x100, two videos, 0.79 and 0.71 ms with 8
+// to five times as many as are resident (20 of 64 threads, 48 registers, no
+// spills): whole quality calls of 1280x720x100, two videos, 0.79 and 0.71 ms with 8
 // blocks of 256 threads per SM, 0.72 and 0.66 ms with 40, 0.69 and 0.62 ms with 100
 // blocks of 64, the same with 300 or with a cursor on the device; 0.72 and
 // 0.65 ms with 40 registers.  Lane s adds up what its warp found for set s: one
 // addition per warp to the set's words instead of one per event.
 //
 // The transform costs the same wherever the events are, this search the more the
-// farther they are.  An event may take FSTEPS steps (a step: 32 cell rows of a ring, or the
-// search of one cell row; wide rows count by their length), and all events together
+// farther they are.  An event may take 512 steps (a step: 32 cell rows of a ring, or the
+// search of one cell row; more where rows are wider than 2048), and all events together
 // `budget` beyond their first 64 (most take 10 to 30, the farthest of a video a
 // hundred or two).  An event that is not settled then leaves its set to the
 // transform, and the set's other events are skipped.  Whole calls / four transforms:
-// 80000 events of 1280x720x100 500 rows from the other video's 1.74 / 3.96 ms, opposite ends
+// 80000 events of 1280x720x100 500 rows from the other video's 1.53 / 3.96 ms, opposite ends
 // of 64x64x8192 4.35 / 5.46, 250000 events of 16384x16384x1 against one in a corner 13.8 /
-// 55.1.  128 steps and no common budget: 1.61, 3.78 and 13.6 ms, but one 1280x720x100
-// drifting grating in fifteen went to the transform for an event of 130 steps (0.67 -> 2.03).
+// 55.1.  (With 128 steps and no common budget one 1280x720x100 drifting grating in fifteen went
+// to the transform for an event of 130 steps, 0.67 -> 2.03 ms.)  A search without the bound or
+// the rings' clipping took 258 us of a benchmark call, this one 282; with every ring clipped
+// and the budget looked at in every step it took 303.
 constexpr int FWARPS = 2;
-constexpr int FSTEPS = 512;
+constexpr int FSTEPS = 448;      // beyond the first 64
 __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const uint32_t* __restrict__ masks,
                                                                 const uint32_t* __restrict__ cells, int tau2,
                                                                 int32_t* __restrict__ d2_a, int32_t* __restrict__ d2_b,
@@ -430,13 +432,13 @@ __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const u
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     unsigned long long closed = 0, matched = 0;      // of the set whose number the lane has
     double sum = 0.0;
+    unsigned edt = (unsigned)acc[QACC_EDT];          // sets left to the transform: lane 0's view counts
     for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += nw) {
         const uint64_t id = far_list[k];
         const int s = (int)(id >> 60);
-        // (read by one lane: the others could see it change)
-        unsigned edt = 0;
-        if (lane == 0) edt = (unsigned)*(volatile unsigned long long*)(acc + QACC_EDT);
-        if (__shfl_sync(full, edt, 0) >> s & 1u) continue;
+        const unsigned skip = __shfl_sync(full, edt, 0);
+        if (lane == 0) edt = (unsigned)*(volatile unsigned long long*)(acc + QACC_EDT);   // for the next event
+        if (skip >> s & 1u) continue;
         const int64_t voxel = (int64_t)(id & ((1ull << 60) - 1ull));
         const int64_t row = voxel / G.W;
         const int x = (int)(voxel - row * G.W);
@@ -446,79 +448,103 @@ __global__ void __launch_bounds__(32 * FWARPS, 20) k_search_far(QGrid G, const u
         const int cy0 = y / QCELL, ct0 = t / QCELL;
         const int r_end = max(max(cy0, cy_n - 1 - cy0), max(ct0, ct_n - 1 - ct0));
         int32_t best = QINF;
-        int steps = 0;
-        auto spend = [&](int k) {
-            const int before = steps;
-            steps += k;
-            if ((before ^ steps) >> 6 == 0) return;
-            int stop = 0;      // (the whole warp is here)
-            if (lane == 0)
-                stop = (int64_t)atomicAdd(acc + QACC_STEPS, 64ull) >= budget ||
-                       (*(volatile unsigned long long*)(acc + QACC_EDT) >> s & 1ull) != 0;
-            if (__shfl_sync(full, stop, 0)) steps = FSTEPS + 1;
+        int left = 64, paid = 0;       // steps in hand, and those taken beyond the first 64
+        const int cost = 1 + (G.ww >> 6);
+        // this lane's cell row, if it has one in the video: bounds first, then the searches
+        auto look = [&](bool in, int cy, int ct) {
+            int32_t bound = QINF;      // no event of the cell row is nearer,
+            int32_t within = QINF;     // and one of them is nearer than this
+            if (in) {
+                const int dy = max(0, max(cy * QCELL - y, y - (cy * QCELL + QCELL - 1)));
+                const int dt = max(0, max(ct * QCELL - t, t - (ct * QCELL + QCELL - 1)));
+                const int32_t d = dy * dy + dt * dt;
+                if (d < best) {
+                    const int32_t dx = cells_near(C + ((int64_t)ct * cy_n + cy) * sw, sw, x);
+                    if (dx < QINF) {
+                        const int uy = max(abs(cy * QCELL - y), abs(cy * QCELL + QCELL - 1 - y));
+                        const int ut = max(abs(ct * QCELL - t), abs(ct * QCELL + QCELL - 1 - t));
+                        bound = d + dx * dx;
+                        within = uy * uy + ut * ut + (dx + 31) * (dx + 31) + 1;
+                    }
+                }
+            }
+            left -= cost;
+            best = min(best, __reduce_min_sync(full, within));
+            while (true) {
+                const int32_t first = __reduce_min_sync(full, bound);
+                if (first >= best) break;
+                const int src = __ffs(__ballot_sync(full, bound == first)) - 1;
+                const int yy = __shfl_sync(full, cy, src) * QCELL + (lane & (QCELL - 1));
+                const int tt0 = __shfl_sync(full, ct, src) * QCELL + lane / QCELL;
+                if (lane == src) bound = QINF;
+                left -= cost;
+                int32_t got = best;
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    const int tt = tt0 + half * (QCELL / 2);
+                    const int32_t d = (yy - y) * (yy - y) + (tt - t) * (tt - t);
+                    if (yy < G.H && tt < G.T && d < got)
+                        got = row_wide(M + ((int64_t)tt * G.H + yy) * G.ww, G.ww, x, got - d) + d;
+                }
+                best = min(best, __reduce_min_sync(full, got));
+            }
         };
-        for (int r = 0; r <= r_end && steps <= FSTEPS; ++r) {
+        auto ring_is_nearer = [&](int r) {
             const int ring = QCELL * (r - 1) + 1;
-            if (r > 0 && ring * ring >= best) break;
-            // the ring's cell rows within the video: its first and last frame of cells,
-            // then the ends of the frames between
+            return r == 0 || ring * ring < best;
+        };
+        // the rings of up to 32 cell rows, one lane each wherever they lie: two full sides
+        // of 2r + 1 cell rows, then pairs
+        int r = 0;
+        for (; r <= min(r_end, 4) && ring_is_nearer(r); ++r) {
+            const int side = 2 * r + 1;
+            int cy, ct;
+            if (lane < 2 * side) {
+                ct = ct0 + (lane < side ? -r : r);
+                cy = cy0 + (lane < side ? lane : lane - side) - r;
+            } else {
+                const int p = lane - 2 * side;
+                ct = ct0 + (p >> 1) - r + 1;
+                cy = cy0 + ((p & 1) ? r : -r);
+            }
+            look(lane < (r == 0 ? 1 : 8 * r) && cy >= 0 && cy < cy_n && ct >= 0 && ct < ct_n, cy, ct);
+        }
+        // larger rings: only the cell rows within the video, in the same order
+        for (; r <= r_end && paid <= FSTEPS && ring_is_nearer(r); ++r) {
             const int y0 = max(cy0 - r, 0), ny = min(cy0 + r, cy_n - 1) - y0 + 1;
             const int t0 = max(ct0 - r + 1, 0), nt = max(min(ct0 + r - 1, ct_n - 1) - t0 + 1, 0);
             const bool low = cy0 >= r, high = cy0 + r < cy_n;
             const int first_rows = ct0 >= r ? ny : 0;
-            const int sides = first_rows + (r > 0 && ct0 + r < ct_n ? ny : 0);
+            const int sides = first_rows + (ct0 + r < ct_n ? ny : 0);
             const int rows = sides + nt * ((int)low + (int)high);
-            for (int j0 = 0; j0 < rows && steps <= FSTEPS; j0 += 32) {
+            for (int j0 = 0; j0 < rows; j0 += 32) {
+                // (a look takes at most 33 steps, so it is enough to pay here)
+                if (left < 0) {
+                    const int more = (63 - left) & ~63;
+                    left += more;
+                    paid += more;
+                    int stop = 0;
+                    if (lane == 0)
+                        stop = (int64_t)atomicAdd(acc + QACC_STEPS, (unsigned long long)more) >= budget ||
+                               (*(volatile unsigned long long*)(acc + QACC_EDT) >> s & 1ull) != 0;
+                    if (__shfl_sync(full, stop, 0)) paid = FSTEPS + 1;
+                    if (paid > FSTEPS) break;
+                }
                 const int j = j0 + lane;
-                int32_t bound = QINF;      // no event of this lane's cell row is nearer,
-                int32_t within = QINF;     // and one of them is nearer than this
-                int cy = 0, ct = 0;
-                if (j < rows) {
-                    if (j < sides) {
-                        ct = ct0 + (j < first_rows ? -r : r);
-                        cy = y0 + (j < first_rows ? j : j - first_rows);
-                    } else {
-                        const int p = j - sides;
-                        const bool both = low && high;
-                        ct = t0 + (both ? p >> 1 : p);
-                        cy = (both ? (p & 1) != 0 : high) ? cy0 + r : cy0 - r;
-                    }
-                    const int dy = max(0, max(cy * QCELL - y, y - (cy * QCELL + QCELL - 1)));
-                    const int dt = max(0, max(ct * QCELL - t, t - (ct * QCELL + QCELL - 1)));
-                    const int32_t d = dy * dy + dt * dt;
-                    if (d < best) {
-                        const int32_t dx = cells_near(C + ((int64_t)ct * cy_n + cy) * sw, sw, x);
-                        if (dx < QINF) {
-                            const int uy = max(abs(cy * QCELL - y), abs(cy * QCELL + QCELL - 1 - y));
-                            const int ut = max(abs(ct * QCELL - t), abs(ct * QCELL + QCELL - 1 - t));
-                            bound = d + dx * dx;
-                            within = uy * uy + ut * ut + (dx + 31) * (dx + 31) + 1;
-                        }
-                    }
+                int cy, ct;
+                if (j < sides) {
+                    ct = ct0 + (j < first_rows ? -r : r);
+                    cy = y0 + (j < first_rows ? j : j - first_rows);
+                } else {
+                    const int p = j - sides;
+                    const bool both = low && high;
+                    ct = t0 + (both ? p >> 1 : p);
+                    cy = (both ? (p & 1) != 0 : high) ? cy0 + r : cy0 - r;
                 }
-                spend(1 + (sw >> 2));
-                best = min(best, __reduce_min_sync(full, within));
-                while (steps <= FSTEPS) {
-                    const int32_t first = __reduce_min_sync(full, bound);
-                    if (first >= best) break;
-                    const int src = __ffs(__ballot_sync(full, bound == first)) - 1;
-                    const int yy = __shfl_sync(full, cy, src) * QCELL + (lane & (QCELL - 1));
-                    const int tt0 = __shfl_sync(full, ct, src) * QCELL + lane / QCELL;
-                    if (lane == src) bound = QINF;
-                    spend(1 + (int)(sqrtf((float)best) * (1.0f / 256.0f)));
-                    int32_t got = best;
-#pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        const int tt = tt0 + half * (QCELL / 2);
-                        const int32_t d = (yy - y) * (yy - y) + (tt - t) * (tt - t);
-                        if (yy < G.H && tt < G.T && d < got)
-                            got = row_wide(M + ((int64_t)tt * G.H + yy) * G.ww, G.ww, x, got - d) + d;
-                    }
-                    best = min(best, __reduce_min_sync(full, got));
-                }
+                look(j < rows, cy, ct);
             }
         }
-        if (steps > FSTEPS) {
+        if (paid > FSTEPS) {
             if (lane == 0) leave_to_edt(acc, s);
             continue;
         }
@@ -761,13 +787,13 @@ int64_t quality_cell_bytes(int32_t W, int32_t H, int32_t T) {
     return 4 * QSETS * sw * ((H + QCELL - 1) / QCELL) * ((T + QCELL - 1) / QCELL);
 }
 
-// Far events the list holds.  Their search takes 1.5 ms per 80000 events of some
+// Far events the list holds.  Their search takes 1.3 ms per 80000 events of some
 // 100 steps each at 1280x720x100 (all four sets by the transform: 4 to 10 ms) and a
 // tenth of that for events a few cells away, so the list may hold this many before the
 // transform is the better bet; small videos' events have few cells to look at.
 // Unrelated random videos, whole calls with a list of voxels / 1024 + 1024, this one and four
-// transforms: 10^-3 events per voxel 1280x720x100 6.11 / 0.75 / 5.81 ms, 203x199x31 0.43 /
-// 0.09 / 0.37; 10^-2 8.26 / 8.12 / 7.95 (more than either holds) and 0.64 / 0.12 / 0.57.
+// transforms: 10^-3 events per voxel 1280x720x100 6.11 / 0.70 / 5.81 ms, 203x199x31 0.43 /
+// 0.09 / 0.37; 10^-2 8.26 / 8.16 / 7.95 (more than either holds) and 0.64 / 0.12 / 0.57.
 int64_t quality_far_cap(int32_t W, int32_t H, int32_t T) { return (int64_t)W * H * T / 512 + 16384; }
 
 cudaError_t launch_quality(const QualityArgs& A, int sms, cudaStream_t st, int* launches) {
