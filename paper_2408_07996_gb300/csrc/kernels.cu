@@ -710,9 +710,11 @@ __device__ __forceinline__ Moments chan(Moments a, Moments b) {
 // latency of a pixel's own chain of loads and additions, which a warp shortens eightfold.
 // Whole detector steps, four lanes / a warp: 5000 pixels x 17 samples 19 / 27 us, 80000 x
 // 16 27 / 53, 20000 x 64 27 / 27, 20000 x 512 39 / 39, 9728 x 512 39 / 27, 1 x 64 27 / 19, 40000 x
-// 2048 138 / 103, 9728 x 2048 100 / 39, 1 x 8192 286 / 39: a warp pays up to about 32
-// pixels per sample of a batch, from batches of 64 on (a mean of 2^20 samples of one pixel:
-// 38 / 3.9 ms).
+// 2048 138 / 103, 9728 x 2048 100 / 39, 1 x 8192 286 / 39 (a mean of 2^20 samples of one pixel
+// 38 / 3.9 ms).  So long batches (64 and more) have a warp per pixel up to 32 pixels per
+// sample.  Batches of 32 and more have one also where a warp for every pixel is resident at
+// once (152 SMs x 40), and the shortest below 1024 pixels: mean-only steps on 3072 pixels
+// with batches of 32 and 64 104 / 91 us, of 16 97 / 103; on 64 pixels of 16 96 / 92.
 //
 // The order of the additions is fixed: sample s of a batch belongs to leaf s % 32,
 // leaves add up pairwise 16, 8, 4, 2 and 1 apart (a warp's butterfly).  A lane holds
@@ -720,7 +722,9 @@ __device__ __forceinline__ Moments chan(Moments a, Moments b) {
 // partner: the same bits), and every lane of a pixel ends with identical
 // statistics and takes the same decisions.
 __host__ __device__ __forceinline__ bool stats_by_warp(int64_t n_pix, int64_t sub) {
-    return sub >= 64 && n_pix <= 32 * sub;
+    const int64_t resident = 152 * 40;
+    const int64_t most = sub >= 64 && 32 * sub > resident ? 32 * sub : (sub >= 32 ? resident : 1024);
+    return n_pix <= most;
 }
 
 constexpr int STATS_STEPS = 8;
@@ -730,6 +734,7 @@ __device__ __forceinline__ void stats_tiles(const Wave& w, const StatsArgs& A0, 
                                             const Job* __restrict__ jobs, uint32_t* again_bits, int& again_at) {
     constexpr unsigned full = 0xffffffffu;
     constexpr int PIX = 32 / LANES, LEAVES = 32 / LANES;
+    constexpr bool kOwnList = kChecked && LANES == 32;     // few pixels: listed one by one, in any order
     constexpr int AHEAD = 8;       // samples that a lane of a warp's pixel loads at a time
     const int lane = threadIdx.x & 31, q = lane & (LANES - 1);
     const int test0 = A0.mode == MODE_DETECT ? (int)((A0.k_base - A0.spp_min) / A0.spp_batch) : 0;
@@ -738,8 +743,10 @@ __device__ __forceinline__ void stats_tiles(const Wave& w, const StatsArgs& A0, 
     const int64_t per_step = (int64_t)gridDim.x * STEP;
     const int steps = (int)max((int64_t)1, min((int64_t)STEPS, n_pix / per_step));
     for (int64_t t0 = (int64_t)blockIdx.x * steps * STEP; t0 < n_pix; t0 += per_step * steps) {
-        if (threadIdx.x < STEP * STEPS / 32) again_bits[threadIdx.x] = 0;
-        __syncthreads();
+        if (!kOwnList) {
+            if (threadIdx.x < STEP * STEPS / 32) again_bits[threadIdx.x] = 0;
+            __syncthreads();
+        }
         for (int it = 0; it < steps; ++it) {
             const int in_tile = it * STEP + (threadIdx.x >> 5) * PIX + lane / LANES;
             const int64_t j = t0 + in_tile;
@@ -868,7 +875,8 @@ __device__ __forceinline__ void stats_tiles(const Wave& w, const StatsArgs& A0, 
             // the pixel's first lane writes it back
             const bool own = on && q == 0;
             const bool again = own && (detect ? open : n < A.spp_max);
-            if (again) atomicOr(&again_bits[in_tile >> 5], 1u << (in_tile & 31));
+            if (kOwnList && again) next_queue[atomicAdd(w.counters + 3, 1)] = entry;
+            if (!kOwnList && again) atomicOr(&again_bits[in_tile >> 5], 1u << (in_tile & 31));
             // Nothing is queued in the round that reaches spp_max; a pixel it leaves open (its
             // FP32 count cannot reach every spp_max above 2^24) is counted, which ends the call
             // with an error.
@@ -905,6 +913,7 @@ __device__ __forceinline__ void stats_tiles(const Wave& w, const StatsArgs& A0, 
             if (A.spp_out) A.spp_out[pix] = n;
             if (A.mean_out) A.mean_out[pix] = c.mean;
         }
+        if (kOwnList) continue;
         __syncthreads();
         if (!kChecked) {
             // requeue() queues them

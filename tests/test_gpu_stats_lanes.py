@@ -1,6 +1,7 @@
 """The statistics kernel gives a pixel a warp or four lanes, by the call's
-pixels and batch length (a warp up to 32 pixels per sample of a batch).  Both add
-the samples up in the same tree, so a pixel's statistics, event and decision
+pixels and batch length (a warp up to 32 pixels per sample of a batch of 64 or more
+and up to 6080 pixels; up to 6080 from batches of 32 on; up to 1024 below).  Both
+add the samples up in the same tree, so a pixel's statistics, event and decision
 are the same bits in a call of many pixels and in calls of few."""
 import ctypes
 
@@ -53,11 +54,11 @@ def _inputs(n, spp_min, count, first, spp_max):
 
 # (batch length, batches): the first batch of a frame, or a later window
 @pytest.mark.parametrize("first", [True, False])
-@pytest.mark.parametrize("batch,count", [(2, 3), (16, 5), (31, 4), (33, 3), (64, 7), (100, 2), (255, 2), (257, 1)])
+@pytest.mark.parametrize("batch,count", [(2, 3), (16, 5), (31, 4), (32, 4), (33, 3), (63, 2), (64, 7), (100, 2), (255, 2), (257, 1)])
 def test_a_pixel_does_not_depend_on_the_calls_size(first, batch, count):
     spp_min = batch if first else 16
     spp_max = spp_min + batch * count + 5
-    n = 32 * batch + 1                     # four lanes; the parts below: a warp per pixel
+    n = (1024 if batch < 32 else max(6080, 32 * batch)) + 1     # four lanes; the parts below: a warp per pixel
     k = spp_min if first else batch * count
     state, samples, pix = _inputs(n, spp_min, k, first, spp_max)
     whole = _step(state, pix, samples, 0 if first else spp_min, spp_min, batch, spp_max)
@@ -76,8 +77,7 @@ def test_a_pixel_does_not_depend_on_the_calls_size(first, batch, count):
 
 @pytest.mark.parametrize("shape", [(1, 1), (5, 3), (13, 37), (61, 40)])
 def test_frames_of_few_pixels_with_long_batches(shape):
-    """Re-queueing where pixels have a warp each (32 pixels per sample of a batch and
-    fewer), with chunks of ragged sizes, against rounds of the whole image."""
+    """Re-queueing where pixels have a warp each, with chunks of ragged sizes, against rounds of the whole image."""
     W, H = shape
     w = sg.workload("cornell64")
     outs = []
