@@ -314,7 +314,7 @@ def run_batch(args):
 
 
 # bytes one mcev_event_quality call cannot do without: each video read once
-# (the event bits it packs, 1/2 byte per voxel, stay in L2)
+# (the event bits it packs, 1/2 byte per voxel of padded rows, stay in L2)
 QUALITY_BYTES_PER_VOXEL = 2
 # statistics kernel (a7-a10 fused): per pixel visit it reads the queue entry
 # (4), the running and reference (n, mean, M2) (24) and writes the running

@@ -466,9 +466,10 @@ typedef struct mcev_quality {
  * event voxel of a (of b), the squared distance d^2 to the other video's
  * nearest same-polarity event, -2 where it has none, and -1 at voxels
  * without an event; NULL to skip.  Results go to *out (host).  The context
- * needs no scene; scratch (half a byte per voxel; where very many events have
- * their nearest counterpart far away also 8 bytes per voxel and up to 2 GiB of
- * envelope stacks) is allocated through it.
+ * needs no scene; scratch is allocated through it: half a byte per voxel of rows
+ * padded to 32 columns, 1/64 byte per voxel and 160 KiB, and where very many events
+ * have their nearest counterpart far away also 8 bytes per voxel and up to 2 GiB of
+ * envelope stacks (in place of the former where both do not fit).
  * Errors: ARG (NULL inputs, an extent outside 1..16384, tau2 < 0, a value
  * outside {-1, 0, 1}), OOM, CUDA.
  * Paper: the quality metrics of Sec. 4.2 (RMSE, PSNR, F1, PSCD). */

@@ -129,9 +129,8 @@ __device__ __forceinline__ void pack32(const uint32_t v[8], uint32_t& pos, uint3
 
 // One thread packs 32 voxels of a row of both videos and tallies them: 2 B read and
 // 1/2 B written per voxel (rows are padded to whole words).  1280x720x100 in 68 us, 3.4
-// TB/s, half of the measured copy rate (6.67 TB/s): bound by the latency of its few loads
-// in flight (two or four 16-byte ones per thread and step) and the compares and multiplies
-// that pack them.  The tally alone, one voxel at a time, took 75 us.
+// TB/s, half of the measured copy rate (6.67 TB/s): the compares and logic that pack the
+// bytes keep the ALU pipe 81 % busy.  The tally alone, one voxel at a time, took 75 us.
 __global__ void __launch_bounds__(QBLOCK) k_pack(const int8_t* __restrict__ a, const int8_t* __restrict__ b, int W,
                                                  int ww, int64_t n_words, int64_t n, uint32_t* __restrict__ masks,
                                                  unsigned long long* acc) {
@@ -232,7 +231,8 @@ __device__ __forceinline__ int32_t row_wide(const uint32_t* __restrict__ row, in
 // bit set have distance 0; the others are listed in shared memory, so that the
 // lanes share them evenly, and each searches its target rows ring by ring
 // (ring r: rows with max(|dy|, |dt|) = r, at least r^2 away).  Bound by the
-// latency of the mask words' loads, from L2: 192 us on 1280x720x100.
+// latency of the mask words' loads (72 % from L2; 11 of 32 lanes active): 212 us on
+// 1280x720x100.
 constexpr int QWARPS = 4;
 __global__ void __launch_bounds__(32 * QWARPS) k_search(QGrid G, const uint32_t* __restrict__ masks, int tau2,
                                                        int32_t* __restrict__ d2_a, int32_t* __restrict__ d2_b,
